@@ -61,13 +61,13 @@ typedef enum {
  * recomputes the TRUE residual with the FP64 matvec, restarting (refining)
  * from the current iterate until it converges (at most 10 restarts). */
 /* OZAKI: the two descriptor contractions run on the BF16 tensor cores with
- * FP64-class accuracy.  Each 256-entry chunk of an operand row is scaled by a
- * power of two and cut into 7 exact BF16 integer slices of 7 bits (49 bits);
- * slice pairs whose products are kept (i + j <= 8 counting slices from 1: 28 of 49) are accumulated exactly in
- * FP32 per level, combined in double-float and summed across chunks (the
- * error-free splitting of Ozaki, Ogita, Oishi and Rump, 2012; ~1e-14 relative
- * matvec error).  Preconditioner and PCG as for DF64.  Operand magnitudes must
- * stay inside the FP32 range (|x| < 1e38). */
+ * FP64-class accuracy, by exact integer products in a residue number system (the modular form
+ * of Ozaki's error-free products, 2025).  Every operand row is scaled by a power of two and
+ * rounded to integers of 57 bits relative to its norm; their residues modulo 14 pairwise
+ * coprime numbers up to 361 are exact in BF16 and multiplied with exact FP32 accumulation; the
+ * products follow by the Chinese remainder theorem (~5e-15 relative matvec error).
+ * Preconditioner and PCG as for DF64.  Operand magnitudes must stay inside the FP32 range
+ * (|x| < 1e38). */
 typedef enum { GDML_FP64 = 0, GDML_TF32 = 1, GDML_BF16 = 2, GDML_DF64 = 3, GDML_OZAKI = 4 } gdml_precision;
 
 /* Inducing-column selection rule (Sec. 3, "Column selection strategies"). */
@@ -116,7 +116,7 @@ gdml_status gdml_kernel_setup_sym(gdml_ctx** ctx, const double* R_dev, int64_t M
 /* out = K v (+ lambda v if add_lambda), both length n = 3 N M, in the
  * context's precision (FP64 contexts: FP64; TF32/BF16: tensor-core matvec
  * with FP32 accumulation, result stored as double; DF64: double-float
- * contractions; OZAKI: sliced-BF16 tensor-core contractions).  v_dev and out_dev must
+ * contractions; OZAKI: residue products on the BF16 tensor cores).  v_dev and out_dev must
  * not overlap.  The matvec is matrix-free: w_b = J_b v_b, u_a = sum_b H_ab w_b,
  * (K v)_a = J_a^T u_a (Sec. 2.1: CG touches K only through such products,
  * so K is never formed).
@@ -266,13 +266,14 @@ gdml_status gdml_set_inner_rtol(gdml_ctx* ctx, double inner_rtol);
 
 /* Slice levels of the matvec inside the PCG loop of an OZAKI context: mixed precision with a
  * cheaper inner operator and FP64 true residuals.  levels = 7 (the default) is the full product;
- * levels < 7 keeps only the slice pairs i + j < levels (slices counted from 0) in both
- * contractions: fewer tensor-core products (28, 21, 15, 10 for 7, 6, 5, 4 levels) and a matvec
- * error of roughly 2^-(7 levels - 2) relative to |K||v| instead of ~1e-14.  The recurrence then
+ * levels < 7 cuts every 256-entry chunk of an operand row into BF16 slices of 7 bits and keeps only
+ * the slice pairs i + j < levels (slices counted from 0) in both contractions (21, 15, 10 products
+ * for 6, 5, 4 levels): a matvec error of roughly 2^-(7 levels - 2) relative to |K||v| instead of
+ * ~1e-14.  The first call with levels < 7 sets up that form's operands.  The recurrence then
  * solves a slightly perturbed system; gdml_pcg_solve recomputes the true residual with the FP64
  * matvec whenever the recurrence passes and restarts PCG from alpha (at most 10 times), so the
  * reported residual is the FP64 one.  gdml_matvec and the build are not affected.
- * Errors: GDML_ERR_ARG (not an OZAKI context, levels outside 1..7). */
+ * Errors: GDML_ERR_ARG (not an OZAKI context, levels outside 1..7), GDML_ERR_OOM, GDML_ERR_CUDA. */
 gdml_status gdml_set_inner_levels(gdml_ctx* ctx, int32_t levels);
 
 /* Outer refinement steps of the last gdml_pcg_solve: for FP64, DF64 and OZAKI contexts the
@@ -302,9 +303,9 @@ gdml_status gdml_pcg_solve_batched(gdml_ctx* const* ctxs, int32_t count, const d
 /* Tile autotuner for the matvec of this context's shapes.  FP64, DF64, TF32 and BF16
  * contexts: times every power-of-two K-split (1 .. 8 or more) of the second descriptor
  * contraction (FP64 DGEMM or tcgen05 GEMM) and keeps the fastest.  OZAKI contexts: times the
- * number of 256-entry K chunks each CTA of the two sliced GEMMs accumulates in registers
- * (GEMM 1: 1 or all; GEMM 2: 1, 2, 3, 4, 8, ... up to all, counting the chunks of both of its
- * K segments when they run as one product) and keeps the fastest pair.
+ * number of 512-entry K chunks each unit of the two residue products accumulates (the first: 1
+ * or all; the second: 1, 2, 3, 4, 8, ... up to all, as far as their buffers hold the K groups)
+ * and keeps the fastest pair; the results are the same for every choice.
  * *choice_out (host, may be NULL) receives the choice (OZAKI: g1 * 65536 + g2) so that a
  * caller can cache it and restore it later with gdml_set_tuning.  Synchronises the
  * context's stream.  Errors: GDML_ERR_ARG, GDML_ERR_OOM, GDML_ERR_CUDA. */

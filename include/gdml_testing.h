@@ -20,8 +20,8 @@ extern "C" {
 gdml_status gdml_test_tc_gemm(int32_t bf16, const double* A_dev, const double* B_dev, int32_t M, int32_t N,
                               int32_t K, double* C_dev, void* cuda_stream);
 
-/* C = A B^T through the sliced-BF16 tensor-core GEMM of OZAKI contexts (the
- * matvec's descriptor contractions, Sec. 2.1, at FP64-class accuracy).  A: M x K,
+/* C = A B^T through the sliced-BF16 tensor-core GEMM of OZAKI contexts (the matvec's
+ * descriptor contractions, Sec. 2.1, with a reduced number of levels; here any number).  A: M x K,
  * B: N x K, C: M x N, row-major FP64 device arrays, 1 <= M, N, K <= 2^24; every
  * 256-entry chunk of a row of A and B is split into 7 BF16 slices of 7 bits,
  * chunk products are accumulated exactly in FP32 per slice level, each CTA adds

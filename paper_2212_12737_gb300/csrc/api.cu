@@ -12,6 +12,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "oz.cuh"
+#include "rns.cuh"
 #include "tc.cuh"
 #include "../../include/gdml_testing.h"
 
@@ -92,7 +93,8 @@ struct gdml_ctx {
   double* Xc() const { return XcA; }
   double* XcB() const { return V64 + MB * D; }  // MB x D: the training side's centred descriptors
   TcMatvec tc;  // tensor-core matvec state (TF32/BF16 contexts)
-  OzMatvec oz;  // sliced-BF16 tensor-core matvec state (OZAKI contexts)
+  RnsMatvec rn;  // residue matvec state (OZAKI contexts)
+  OzMatvec oz;   // sliced-BF16 matvec of fewer levels (gdml_set_inner_levels), set up when asked for
 
   // preconditioner
   int64_t k = 0;  // rank built (0: none)
@@ -233,7 +235,8 @@ gdml_status matvec_any(gdml_ctx* c, const double* v, double* out, int add_lambda
   if (force_fp64 || c->precision == GDML_FP64) return matvec_fp64(c, v, out, add_lambda);
   if (c->precision == GDML_DF64) return matvec_df(c, v, out, add_lambda);
   if (c->precision == GDML_OZAKI) {
-    gdml_status s = oz_matvec(c->oz, c->G, c->G2, c->Xc(), v, out, add_lambda, c->lam, c->st, lev);
+    gdml_status s = lev == 7 ? rns_matvec(c->rn, c->G, c->Xc(), v, out, add_lambda, c->lam, c->st)
+                             : oz_matvec(c->oz, c->G, c->G2, c->Xc(), v, out, add_lambda, c->lam, c->st, lev);
     if (s != GDML_OK) return ctx_fail(c, s, "sliced tensor-core matvec: " + last_msg());
     return check_launch(c, "matvec_oz");
   }
@@ -633,6 +636,12 @@ gdml_status pcg_core(gdml_ctx* c, const double* b, double* x, double tol_abs, in
   return out;
 }
 
+// reads (and clears) the error words of both tensor-core matvecs of an OZAKI context
+gdml_status oz_check_all(gdml_ctx* c) {
+  const gdml_status s = rns_check(c->rn, c->st), o = oz_check(c->oz, c->st);
+  return s != GDML_OK ? s : o;
+}
+
 gdml_status validate(const gdml_ctx* c) {
   if (!c) return fail(GDML_ERR_ARG, "null context");
   return GDML_OK;
@@ -801,8 +810,8 @@ gdml_status setup_impl(gdml_ctx** out, const double* R_dev, int64_t M, int32_t N
     if (s != GDML_OK) return ctx_fail(C, s, "tensor-core setup: " + last_msg());
   }
   if (precision == GDML_OZAKI) {
-    gdml_status s = oz_setup(c->oz, M, N, (int)D, c->XcA, c->P64, 2 * MB, c->S, c->c, c->st, c->Ssym, c->pis,
-                             c->XcB());
+    gdml_status s = rns_setup(c->rn, M, N, (int)D, c->G, c->XcA, c->P64, 2 * MB, c->S, c->c, c->st, c->Ssym, c->pis,
+                              c->XcB());
     if (s != GDML_OK) return ctx_fail(C, s, "sliced tensor-core setup: " + last_msg());
   }
   CTRY(C, cudaStreamSynchronize(c->st));
@@ -1159,6 +1168,15 @@ gdml_status gdml_set_inner_levels(gdml_ctx* c, int32_t levels) {
   TRY(validate(c));
   if (c->precision != GDML_OZAKI) return ctx_fail(c, GDML_ERR_ARG, "inner levels apply to OZAKI contexts only");
   if (levels < 1 || levels > 7) return ctx_fail(c, GDML_ERR_ARG, "inner levels must be in 1..7");
+  if (levels < 7 && !c->oz.ready) {  // the sliced operands, which only this operator reads
+    gdml_status s = oz_setup(c->oz, c->M, c->N, c->D, c->XcA, c->P64, 2 * c->MB, c->S, c->c, c->st, c->Ssym, c->pis,
+                             c->XcB());
+    if (s != GDML_OK) {
+      oz_destroy(c->oz);
+      c->oz = OzMatvec();
+      return ctx_fail(c, s, "sliced tensor-core setup: " + last_msg());
+    }
+  }
   if (levels != c->inner_lev) drop_graphs(c);  // the captured loop bakes the GEMMs' level count in
   c->inner_lev = levels;
   return GDML_OK;
@@ -1249,7 +1267,7 @@ gdml_status gdml_pcg_solve(gdml_ctx* c, const double* y, double* alpha, double r
   c->hist_arm = false;
   CTRY(c, cudaStreamSynchronize(st));
   if (c->precision == GDML_TF32 || c->precision == GDML_BF16 || c->precision == GDML_OZAKI) {
-    gdml_status ts = c->precision == GDML_OZAKI ? oz_check(c->oz, st) : tc_check(c->tc, st);
+    gdml_status ts = c->precision == GDML_OZAKI ? oz_check_all(c) : tc_check(c->tc, st);
     if (ts != GDML_OK) return ctx_fail(c, ts, last_msg());
   }
   if (df_precond(c)) TRY(ws_check(c));
@@ -1349,7 +1367,7 @@ gdml_status gdml_test_precond_factor(gdml_ctx* c, double* L_out) {
 gdml_status gdml_test_set_wait_limit(uint32_t polls) {
   clear_msg();
   const uint32_t v = polls == 0xFFFFFFFFu ? tc_default_wait_limit() : polls;
-  for (auto fn : {set_wait_limit_oz, set_wait_limit_tc, set_wait_limit_wb, set_wait_limit_pc}) {
+  for (auto fn : {set_wait_limit_oz, set_wait_limit_rns, set_wait_limit_tc, set_wait_limit_wb, set_wait_limit_pc}) {
     cudaError_t e = fn(v);
     if (e != cudaSuccess) return fail(GDML_ERR_CUDA, std::string("set_wait_limit: ") + cudaGetErrorString(e));
   }
@@ -1558,7 +1576,7 @@ gdml_status gdml_autotune(gdml_ctx* c, int32_t* choice_out) {
   CTRY(c, cudaEventCreate(&e0));
   CTRY(c, cudaEventCreate(&e1));
   if (c->precision == GDML_OZAKI) {
-    // the sliced GEMMs' K chunks per CTA (GEMM 1: T = Xc W^T, GEMM 2: U = A W + beta Xc)
+    // the residue products' 512-entry K chunks per unit (T = Xc W^T, U = A W + beta Xc)
     auto time_mv = [&](float* ms) -> gdml_status {
       for (int w = 0; w < 2; ++w) TRY(matvec_any(c, v, out, 1, false));
       CTRY(c, cudaEventRecord(e0, c->st));
@@ -1568,16 +1586,16 @@ gdml_status gdml_autotune(gdml_ctx* c, int32_t* choice_out) {
       cudaEventElapsedTime(ms, e0, e1);
       return GDML_OK;
     };
-    const int n1 = (int)c->oz.W1.nchunks, n2 = (int)c->oz.nch2;
+    const int n1 = (int)c->rn.nch1, n2 = (int)c->rn.nch2;
     std::vector<int> cand2;
     for (int g = 1; g <= n2; g = g < 4 ? g + 1 : g * 2) cand2.push_back(g);
     if (cand2.back() != n2) cand2.push_back(n2);
-    int best1 = c->oz.g1, best2 = c->oz.g2;
+    int best1 = c->rn.g1, best2 = c->rn.g2;
     float best_ms = 1e30f;
     for (int g1 : {1, n1}) {
       for (int g2 : cand2) {
-        c->oz.g1 = g1;
-        c->oz.g2 = g2;
+        c->rn.g1 = g1;
+        c->rn.g2 = g2;
         float ms = 0.f;
         gdml_status ts = time_mv(&ms);
         if (ts != GDML_OK) {
@@ -1595,8 +1613,8 @@ gdml_status gdml_autotune(gdml_ctx* c, int32_t* choice_out) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    c->oz.g1 = best1;
-    c->oz.g2 = best2;
+    c->rn.g1 = best1;
+    c->rn.g2 = best2;
     drop_graphs(c);
     if (choice_out) *choice_out = best1 * 65536 + best2;
     return GDML_OK;
@@ -1631,12 +1649,15 @@ gdml_status gdml_autotune(gdml_ctx* c, int32_t* choice_out) {
 
 gdml_status gdml_set_tuning(gdml_ctx* c, int32_t splits) {
   TRY(validate(c));
-  if (c->precision == GDML_OZAKI) {  // g1 * 65536 + g2: K chunks per CTA of the two sliced GEMMs
+  if (c->precision == GDML_OZAKI) {  // g1 * 65536 + g2: K chunks per unit of the two residue products
     const int g1 = splits >> 16, g2 = splits & 0xFFFF;
-    if (g1 < 1 || g1 > c->oz.W1.nchunks || g2 < 1 || g2 > c->oz.nch2)
-      return ctx_fail(c, GDML_ERR_ARG, "chunks per CTA out of range");
-    c->oz.g1 = g1;
-    c->oz.g2 = g2;
+    // the range of recorded choices: they counted 256-entry chunks, of both of U's K segments where
+    // the first ends on a chunk
+    const int64_t n1 = cdiv(c->D, 256), n2 = cdiv(c->MB, 256), max2 = cdiv(c->MB, 128) % 2 == 0 ? 2 * n2 : n2;
+    if (g1 < 1 || g1 > n1 || g2 < 1 || g2 > max2)
+      return ctx_fail(c, GDML_ERR_ARG, "chunks per unit out of range");
+    c->rn.g1 = g1;
+    c->rn.g2 = g2;
     drop_graphs(c);
     return GDML_OK;
   }
@@ -1653,7 +1674,7 @@ gdml_status gdml_tc_check(gdml_ctx* c) {
   TRY(validate(c));
   if (df_precond(c)) TRY(ws_check(c));
   if (c->precision != GDML_TF32 && c->precision != GDML_BF16 && c->precision != GDML_OZAKI) return GDML_OK;
-  gdml_status s = c->precision == GDML_OZAKI ? oz_check(c->oz, c->st) : tc_check(c->tc, c->st);
+  gdml_status s = c->precision == GDML_OZAKI ? oz_check_all(c) : tc_check(c->tc, c->st);
   if (s != GDML_OK) return ctx_fail(c, s, last_msg());
   return GDML_OK;
 }
@@ -1670,6 +1691,7 @@ void gdml_destroy(gdml_ctx* c) {
   if (c->cap) cudaStreamDestroy(c->cap);
   tc_destroy(c->tc);
   oz_destroy(c->oz);
+  rns_destroy(c->rn);
   for (void* p : c->allocs)
     if (p) cudaFree(p);
   if (c->hsc) cudaFreeHost(c->hsc);

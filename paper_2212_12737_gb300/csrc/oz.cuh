@@ -1,6 +1,8 @@
-// FP64-accurate force-kernel matvec on the BF16 tensor cores (GDML_OZAKI contexts).
+// Sliced-BF16 products on the tensor cores (GDML_OZAKI contexts): the matvec with a reduced number of
+// slice levels (gdml_set_inner_levels; the full matvec is the residue form, rns.cuh) and the
+// preconditioner build's tall products.
 //
-// The two descriptor contractions of K v (the same algebra as the FP64 path),
+// The matvec's two descriptor contractions of K v (the same algebra as the FP64 path),
 //   GEMM 1:  T = Xc W^T                              (M x M, K = D)
 //   GEMM 2:  U = A W + beta Xc                       (M x D, K = M, two segments run as
 //                                                     one product over the concatenated K)

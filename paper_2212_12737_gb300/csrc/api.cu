@@ -871,7 +871,11 @@ gdml_status gdml_predict_forces(gdml_ctx* c, const double* R_query, int64_t Q, c
   TRY(s.get(&Sq, (size_t)(Q * MB)));
   TRY(s.get(&Tq, (size_t)(Q * MB)));
   TRY(s.get(&Pq, (size_t)(Q * 2 * MB)));
-  TRY(s.get(&Uq, (size_t)(Q * D)));
+  // few queries: the second contraction's K in groups, summed by the back-projection (one query of
+  // 210 descriptors against 1000 geometries has 14 tiles)
+  const int64_t utiles = cdiv(Q, 16) * cdiv(D, 16);
+  const int su = (int)std::max<int64_t>(1, std::min<int64_t>(2 * num_sms() / utiles, cdiv(2 * MB, 64)));
+  TRY(s.get(&Uq, (size_t)(su * Q * D)));
   TRY(s.get(&rs, (size_t)Q));
   double* W = c->V64;  // [W ; Xc] of the training side: W_b = J_b alpha_b (permuted copies with symmetries)
   launch_desc_jac(R_query, Q, N, D, Xq, Gq, st);
@@ -885,8 +889,8 @@ gdml_status gdml_predict_forces(gdml_ctx* c, const double* R_query, int64_t Q, c
   }
   launch_dgemm<double, double>(true, Q, MB, D, 1.0, Xqc, D, W, D, 0.0, Tq, MB, false, st);
   launch_beta_rows(Tq, Sq, c->tb, Q, MB, c->c, Pq + MB, 2 * MB, rs, st);
-  launch_dgemm<double, double>(false, Q, D, 2 * MB, 1.0, Pq, 2 * MB, c->V64, D, 0.0, Uq, D, false, st);
-  launch_backproj<double>(Uq, D, 1, Q * D, rs, Xqc, Gq, nullptr, Q, N, D, 0.0, 0, f, st);
+  launch_dgemm<double, double>(false, Q, D, 2 * MB, 1.0, Pq, 2 * MB, c->V64, D, 0.0, Uq, D, false, st, su, Q * D);
+  launch_backproj<double>(Uq, D, su, Q * D, rs, Xqc, Gq, nullptr, Q, N, D, 0.0, 0, f, st);
   return check_launch(c, "predict_forces");
 }
 

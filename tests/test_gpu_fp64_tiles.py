@@ -1,4 +1,5 @@
-"""FP64 products at the edges of their tiles: force prediction over the tile sizes (16, 32, 64) and K groups."""
+"""FP64 paths at the edges of their tiles: the blocked Cholesky (steps of 32 in blocks of 128), and
+force prediction over the products' tile sizes (16, 32, 64) and K groups."""
 import os
 
 import numpy as np
@@ -9,6 +10,7 @@ from oracle import kernel as ok
 from paper_2212_12737_gb300 import build, gdml, synth
 
 pytestmark = pytest.mark.gpu
+EPS = np.finfo(float).eps
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -22,6 +24,29 @@ def _lib():
 
 def dev(x):
     return torch.from_numpy(np.ascontiguousarray(x)).cuda()
+
+
+@pytest.mark.parametrize("k", [1, 31, 32, 33, 96, 127, 128, 129, 161, 300])
+def test_cholesky_backward_error(k):
+    """|A - L L^T| <= (2 k + 8) eps |L| |L|^T entry by entry: the factorisation's k + 1 roundings and
+    those of the pivot's root and reciprocal, and as many of the test's own product."""
+    rng = np.random.default_rng(k)
+    X = rng.standard_normal((k, k + 5))
+    A = X @ X.T * 10.0 ** rng.uniform(-2, 2, size=(k, 1))
+    A = (A + A.T) / 2 + k * 200.0 * np.eye(k)
+    L, eps = gdml.test_cholesky_jitter(dev(A))
+    L = L.cpu().numpy()
+    assert eps == 0.0
+    assert np.all(np.abs(np.tril(A - L @ L.T)) <= (2 * k + 8) * EPS * (np.abs(L) @ np.abs(L).T))
+
+
+def test_cholesky_reports_the_failing_column_of_any_step():
+    for bad in (0, 31, 32, 127, 128, 199):
+        A = np.eye(200)
+        A[bad, bad] = -1e9
+        with pytest.raises(gdml.GdmlError) as e:
+            gdml.test_cholesky_jitter(dev(A))
+        assert e.value.name == "ERR_NOT_SPD"
 
 
 @pytest.mark.parametrize("N,M,Q", [(3, 5, 1), (12, 300, 2), (12, 300, 17), (21, 400, 64), (9, 33, 700)])

@@ -320,7 +320,7 @@ gdml_status gdml_set_tuning(gdml_ctx* ctx, int32_t splits);
  * block or fail, or work recorded between pre-allocated buffers only.
  * The paper has no counterpart; this is a deployment variant of gdml_matvec.
  *  Limits: 1 <= M <= 128 geometries, 2 <= N <= 24 atoms (GDML_ERR_ARG beyond).
- *  Working memory: one static device array of 2.5 MB that every GPU loading
+ *  Working memory: one static device array of 1.5 MB that every GPU loading
  *    this library holds until process exit; every call overwrites what it uses,
  *    so nothing needs clearing between calls.
  *  The first call on each device looks the array's address up (with that

@@ -1,5 +1,6 @@
-"""FP64 paths at the edges of their tiles: the blocked Cholesky (steps of 32 in blocks of 128), and
-force prediction over the products' tile sizes (16, 32, 64) and K groups."""
+"""FP64 paths at the edges of their tiles: the blocked Cholesky (steps of 32 in blocks of 128), the
+products' tile sizes (16, 32, 64) and K groups behind force prediction, and the two-launch
+context-free matvec (geometries in 1 .. 16 groups, by the descriptor count)."""
 import os
 
 import numpy as np
@@ -59,3 +60,14 @@ def test_predicted_forces(N, M, Q):
     ctx.destroy()
     ref = ok.predict_forces(Rq, R, 4.0, alpha)
     assert np.linalg.norm(f - ref) <= 1e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("N,M", [(2, 128), (3, 1), (8, 9), (9, 100), (12, 33), (17, 64), (23, 128)])
+def test_noalloc_groups(N, M):
+    R = synth.geometries(synth.template(N, 7), M, 0.1, 8)
+    v = np.random.default_rng(N).standard_normal(R.size)
+    got = gdml.matvec_noalloc(dev(R), 3.0, 1e-6, dev(v)).cpu().numpy()
+    ref = ok.matvec(R, 3.0, v, 1e-6)
+    assert np.linalg.norm(got - ref) <= 1e-12 * np.linalg.norm(ref)
+    plain = gdml.matvec_noalloc(dev(R), 3.0, 1e-6, dev(v), add_lambda=False).cpu().numpy()
+    assert np.linalg.norm(got - plain - 1e-6 * v) <= 1e-12 * np.linalg.norm(ref)

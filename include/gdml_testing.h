@@ -36,8 +36,7 @@ gdml_status gdml_test_oz_gemm(const double* A_dev, const double* B_dev, int64_t 
 
 /* The tall product of the OZAKI preconditioner build (Eq. 5's L_k = K_nk L_kk^-T as K_nk
  * times the transposed triangular inverse, and the leverage-score row norms of Sec. 3's
- * estimate): C = A B^T on the sliced-BF16 tensor cores, accumulated over all of K inside
- * each output tile (FP64-class).  A: n x K FP64, COLUMN-major (entry (r, j) at A[j n + r]);
+ * estimate): C = A B^T by residue products on the BF16 tensor cores (FP64-class).  A: n x K FP64, COLUMN-major (entry (r, j) at A[j n + r]);
  * B: NB x K FP64, row-major with row stride ldb >= K; tri_b != 0 declares B lower
  * triangular (zero above its diagonal, which must hold: whole K blocks past each tile's
  * diagonal are skipped).  rowsq = 0: out (n x NB, column-major: C[r][c] at out[c n + r])

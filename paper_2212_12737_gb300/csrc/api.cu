@@ -335,9 +335,8 @@ gdml_status chol_jitter(gdml_ctx* c, const double* src, double* work, int64_t k,
 
 // L (k x n row-major = n x k col-major) <- Nystrom factor from columns S (Eq. 5).
 // FP64 / DF64 contexts: forward substitution on the FP64 pipe.  OZAKI contexts: the same
-// L_k = K_nk L_kk^-T as K_nk times the transposed triangular inverse of L_kk, on the sliced
-// BF16 tensor cores (FP64-class products, accumulated over all of k in each tile); only the
-// k x k inverse runs on the FP64 pipe.  On return `work` holds L_kk (lower, row-major).
+// L_k = K_nk L_kk^-T as K_nk times the transposed triangular inverse of L_kk, as residue
+// products on the tensor cores (rns_build.cu); only the k x k inverse runs on the FP64 pipe.  On return `work` holds L_kk (lower, row-major).
 gdml_status nystrom(gdml_ctx* c, const int64_t* S, int64_t k, double* L, double* Kkk, double* work,
                     double* eps_out) {
   TRY(get_cols(c, S, k, L));
@@ -351,8 +350,8 @@ gdml_status nystrom(gdml_ctx* c, const int64_t* S, int64_t k, double* L, double*
     set_identity(Linv, k, c->st);
     trsm_left_lower(work, k, Linv, k, c->st, true);  // L_kk^-1 (lower triangular)
     TRY(check_launch(c, "inducing-block inverse"));
-    gdml_status so = oz_gemm_tall(L, c->n, k, Linv, k, k, true, false, L, nullptr, c->st);
-    if (so != GDML_OK) return ctx_fail(c, so, "sliced K_nk L_kk^-T: " + last_msg());
+    gdml_status so = rns_gemm_tall(L, c->n, k, Linv, k, k, true, false, L, nullptr, c->st);
+    if (so != GDML_OK) return ctx_fail(c, so, "residue K_nk L_kk^-T: " + last_msg());
     return GDML_OK;
   }
   trsm_left_lower(work, k, L, c->n, c->st);  // rows of K_nk^T -> rows of L_k^T
@@ -362,12 +361,12 @@ gdml_status nystrom(gdml_ctx* c, const int64_t* S, int64_t k, double* L, double*
 // LC <- chol(lambda I + L^T L) (Eq. 4); with Cinv, also C^-1 = L_C^-T L_C^-1
 gdml_status woodbury_core(gdml_ctx* c, const double* L, int64_t k, double* LC, double* Cinv = nullptr,
                           double* Cfull = nullptr, const float* Lf = nullptr) {
-  if (Lf && c->precision == GDML_OZAKI) {  // C from the FP32 factor on the sliced tensor cores
-    gdml_status s = oz_syrk_lower(Lf, c->n, k, LC, k, c->st);
-    if (s != GDML_OK) return ctx_fail(c, s, "sliced syrk: " + last_msg());
-  } else if (c->precision == GDML_OZAKI) {  // C from the FP64 factor (columns = rows of L^T), sliced
-    gdml_status s = oz_syrk_lower_f64(L, k, c->n, c->n, LC, k, c->st);
-    if (s != GDML_OK) return ctx_fail(c, s, "sliced syrk: " + last_msg());
+  if (Lf && c->precision == GDML_OZAKI) {  // C from the FP32 factor by residue products
+    gdml_status s = rns_syrk_lower(Lf, k, c->n, c->n, LC, k, c->st);
+    if (s != GDML_OK) return ctx_fail(c, s, "residue syrk: " + last_msg());
+  } else if (c->precision == GDML_OZAKI) {  // C from the FP64 factor (columns = rows of L^T), likewise
+    gdml_status s = rns_syrk_lower(L, k, c->n, c->n, LC, k, c->st);
+    if (s != GDML_OK) return ctx_fail(c, s, "residue syrk: " + last_msg());
   } else if (Lf)  // DF64: C from the FP32-stored factor, exact products, double-float sums
     launch_dfsyrk(k, c->n, Lf, c->n, LC, k, c->st);
   else
@@ -391,10 +390,10 @@ gdml_status woodbury_core(gdml_ctx* c, const double* L, int64_t k, double* LC, d
     set_identity(X, k, c->st);
     trsm_left_lower(LC, k, X, k, c->st, true);  // X = L_C^-1 (lower triangular)
     transpose_square(X, k, Xt, c->st);
-    if (df_precond(c)) {  // X^T X on the sliced tensor cores (FP64-class), lower triangle mirrored
+    if (df_precond(c)) {  // X^T X by residue products, lower triangle mirrored
       TRY(check_launch(c, "woodbury inverse"));
-      gdml_status so = oz_syrk_lower_f64(Xt, k, k, k, Cinv, k, c->st);
-      if (so != GDML_OK) return ctx_fail(c, so, "sliced X^T X: " + last_msg());
+      gdml_status so = rns_syrk_lower(Xt, k, k, k, Cinv, k, c->st);
+      if (so != GDML_OK) return ctx_fail(c, so, "residue X^T X: " + last_msg());
       mirror_lower(Cinv, k, c->st);
     } else {
       launch_dgemm<double, double>(true, k, k, k, 1.0, Xt, k, Xt, k, 0.0, Cinv, k, false, c->st);  // X^T X
@@ -448,12 +447,12 @@ gdml_status rls_estimate(gdml_ctx* c, int64_t k, uint64_t seed, int64_t* S, doub
   TRY(woodbury_core(c, c->L, k, c->LC));          // chol(B^T B + lambda I)
   if (c->precision == GDML_OZAKI) {
     // tau_i = |L_C^-1 b_i|^2: the row square sums of B X^T with X = L_C^-1 (lower
-    // triangular, formed on the FP64 pipe), the product on the sliced tensor cores
+    // triangular, formed on the FP64 pipe), the product by residues
     set_identity(work, k, c->st);
     trsm_left_lower(c->LC, k, work, k, c->st, true);
     TRY(check_launch(c, "rls core inverse"));
-    gdml_status so = oz_gemm_tall(c->L, n, k, work, k, k, true, true, tau, nullptr, c->st);
-    if (so != GDML_OK) return ctx_fail(c, so, "sliced leverage scores: " + last_msg());
+    gdml_status so = rns_gemm_tall(c->L, n, k, work, k, k, true, true, tau, nullptr, c->st);
+    if (so != GDML_OK) return ctx_fail(c, so, "residue leverage scores: " + last_msg());
     return GDML_OK;
   }
   trsm_left_lower(c->LC, k, c->L, n, c->st);       // Z = L_C^-1 B^T
@@ -1349,7 +1348,7 @@ gdml_status gdml_test_oz_gemm_tall(const double* A_dev, int64_t n, int64_t K, co
   if (!A_dev || !B_dev || !out_dev || n < 1 || K < 1 || NB < 1 || ldb < K)
     return fail(GDML_ERR_ARG, "bad tall gemm test arguments");
   if (n > ((int64_t)1 << 31)) return fail(GDML_ERR_ARG, "tall gemm test: n too large");
-  return oz_gemm_tall(A_dev, n, K, B_dev, NB, ldb, tri_b != 0, rowsq != 0, out_dev, rowsq ? nullptr : out32_dev,
+  return rns_gemm_tall(A_dev, n, K, B_dev, NB, ldb, tri_b != 0, rowsq != 0, out_dev, rowsq ? nullptr : out32_dev,
                       static_cast<cudaStream_t>(stream));
 }
 

@@ -34,8 +34,6 @@ constexpr int kSmemData = 2 * kBGroup + kAStages * kATile;
 constexpr int kSmemTotal = kSmemData + 1024 + 256;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kKbPerChunk = oz::KC / oz::KB;
-constexpr int kWaiterWarp = 11;           // the accumulating GEMM's extra warp: mbarrier waits
-constexpr int kThreadsAcc = 32 * 12;
 constexpr int kStageLd = oz::BN + 1;  // padded row of the staged output tile (float2)
 // matvec GEMM: k-blocks of 64 K entries (one 128-byte swizzle span per tile).  The B group of
 // a k-block (7 slices, 56 KB) is double-buffered; the A slices stream through a 6-deep ring
@@ -206,30 +204,13 @@ __global__ void __launch_bounds__(256) oz_slice_rows_kernel(const double* __rest
   slice_write(xs, ex, sl, row, k, Rp, Kp);
 }
 
-// Same slicing for FP32 input rows (the FP32-stored Nystrom factor): hi = x, lo = 0.
-__global__ void __launch_bounds__(256) oz_slice_rows_f32_kernel(const float* __restrict__ X, int64_t ldx, int64_t K,
-                                                                int64_t rows, int64_t Rp, int64_t Kp,
-                                                                bf16* __restrict__ sl, int* __restrict__ e) {
-  __shared__ float red[8];
-  const int64_t row = blockIdx.x, q = blockIdx.y;
-  const int64_t k = q * oz::KC + threadIdx.x;
-  const float x = k < K ? X[row * ldx + k] : 0.f;
-  const int ex = chunk_exponent(fabsf(x), red);
-  if (threadIdx.x == 0) e[q * rows + row] = ex;
-  slice_write(make_float2(x, 0.f), ex, sl, row, k, Rp, Kp);
-}
-
-// an entry as a float pair (hi, lo) with hi + lo = x (FP64: rounded to 48 bits)
-__device__ __forceinline__ float2 as_pair(double x) { return split_d(x); }
-__device__ __forceinline__ float2 as_pair(float2 x) { return x; }
-
 // Slicing of a COLUMN-major source: operand row r (r < rows) is row r0 + r of the n x K
 // matrix whose column j starts at src + j ld, i.e. entry (r, j) = src[j ld + r0 + r].  One
 // CTA per RB rows (16, or 4 when 16 would leave most SMs idle) and one 256-entry chunk:
 // coalesced reads down the columns into a shared tile, a per-row exponent, then slice rows
 // written along K (coalesced).
-template <typename T, int RB = 16>
-__global__ void __launch_bounds__(256) oz_slice_cols_kernel(const T* __restrict__ src, int64_t ld, int64_t r0,
+template <int RB>
+__global__ void __launch_bounds__(256) oz_slice_cols_kernel(const float2* __restrict__ src, int64_t ld, int64_t r0,
                                                             int64_t rows, int64_t K, int64_t Rp, int64_t Kp,
                                                             bf16* __restrict__ sl, int* __restrict__ e) {
   static_assert(RB <= 16 && 256 % RB == 0, "rows per CTA");
@@ -244,7 +225,7 @@ __global__ void __launch_bounds__(256) oz_slice_cols_kernel(const T* __restrict_
       const int64_t j = q * oz::KC + jj;
       const int64_t row = rb + r;
       float2 x = make_float2(0.f, 0.f);
-      if (j < K && row < rows) x = as_pair(src[j * ld + r0 + row]);
+      if (j < K && row < rows) x = src[j * ld + r0 + row];
       tile[jj][r] = x;
     }
   }
@@ -267,15 +248,6 @@ __global__ void __launch_bounds__(256) oz_slice_cols_kernel(const T* __restrict_
     if (rb + r >= rows) break;
     slice_write(tile[tid][r], ex_s[r], sl, rb + r, q * oz::KC + tid, Rp, Kp);
   }
-}
-
-// sum of the square-sum partials of each row, in a fixed slot order
-__global__ void oz_rowsq_reduce_kernel(const double* __restrict__ sq, int slots, int64_t n, double* __restrict__ out) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double s = 0.0;
-  for (int k = 0; k < slots; ++k) s += sq[(int64_t)k * n + i];
-  out[i] = s;
 }
 
 // (h, l) = (ah, al) - (bh, bl)
@@ -853,303 +825,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-enum { ACC_ROWMAJOR = 0, ACC_COLMAJOR = 1, ACC_ROWSQ = 2 };
-struct AccOut {  // what the accumulating GEMM stores (see oz_gemm_acc_kernel)
-  int mode;
-  int lower_only;
-  int tri_b;
-  double* C;
-  float* C32;
-  double* sq;
-  int64_t ldc;
-};
-
-// Same sliced product accumulated over ALL K chunks inside the CTA, FP64 output:
-//   C[m][n] = sum_chunks 2^(eA + eB) sum_levels acc_level 2^-7(level + 2)
-// The MMA warp signals the end of each chunk on cdone; the 8 epilogue warps read the 7
-// level accumulators of their 32 columns, add the scaled chunk value into a running
-// double-float sum held in registers, and release the TMEM on tfree before the MMA
-// warp starts the next chunk (whose first MMA per level overwrites).
-//  o.lower_only: tiles wholly above the diagonal exit at once (symmetric products);
-//  o.tri_b: row c of B is zero beyond column c (lower triangular B), so the CTA of B rows
-//    [n0, n0 + 64) stops after K entry n0 + 63;
-//  o.mode: ACC_ROWMAJOR  C[m][n] at C[m ldc + n];
-//          ACC_COLMAJOR  C[m][n] at C[n ldc + m] (and as FP32 at C32[n ldc + m] if C32);
-//          ACC_ROWSQ     sq[(2 blockIdx.x + half) ldc + m] = sum over the half tile's 32
-//                        columns n of C[m][n]^2 (no C is stored).
-__global__ void __launch_bounds__(kThreadsAcc, 1)
-    oz_gemm_acc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int Ap,
-                       int Bp, int M, int N, int num_kb_all, const int* __restrict__ eA, const int* __restrict__ eB,
-                       const AccOut o, int* __restrict__ err) {
-  const int n0 = blockIdx.x * oz::BN, m0 = blockIdx.y * oz::BM;
-  if (o.lower_only && n0 >= m0 + oz::BM) return;
-  const int num_kb = o.tri_b ? min(num_kb_all, (n0 + oz::BN + oz::KB - 1) / oz::KB) : num_kb_all;
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sB = smem;
-  uint8_t* sA = smem + 2 * kBGroup;
-  uint64_t* bfull = reinterpret_cast<uint64_t*>(smem + kSmemData);
-  uint64_t* bempty = bfull + 2;
-  uint64_t* afull = bempty + 2;
-  uint64_t* aempty = afull + kAStages;
-  uint64_t* cdone = aempty + kAStages;
-  uint64_t* tfree = cdone + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfree + 1);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nchunks = (num_kb + kKbPerChunk - 1) / kKbPerChunk;
-
-  if (threadIdx.x == 0) {
-    for (int g = 0; g < 2; ++g) {
-      tc::mbar_init(&bfull[g], 1);
-      tc::mbar_init(&bempty[g], 1);
-    }
-    for (int s = 0; s < kAStages; ++s) {
-      tc::mbar_init(&afull[s], 1);
-      tc::mbar_init(&aempty[s], 1);
-    }
-    tc::mbar_init(cdone, 1);
-    tc::mbar_init(tfree, 8);  // one arrival per epilogue warp
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(tmem_slot)),
-                 "r"(kTmemCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-  // MMA thread: issued at least one MMA / learned of a failed wait.  A thread that failed
-  // before issuing anything commits nothing, so no asynchronous arrive outlives the CTA.
-  bool mma_any = false, mma_failed = false;
-
-  if (warp == 0 && lane == 0) {
-    // ---------------- TMA producer, A slices (all k-blocks)
-    for (int kb = 0; kb < num_kb; ++kb) {
-      bool ok = true;
-      for (int i = 0; i < oz::S; ++i) {
-        const int ai = kb * oz::S + i;
-        const int s = ai % kAStages;
-        const uint32_t ph = (uint32_t)(ai / kAStages) & 1u;
-        if (!mbar_wait_spin(&aempty[s], ph ^ 1u)) {
-          atomicExch(err, tc::ERR_TIMEOUT_EMPTY);
-          *abort_flag = 1;
-          ok = false;
-          break;
-        }
-        if (*abort_flag) {
-          ok = false;
-          break;
-        }
-        tc::mbar_expect_tx(&afull[s], kATile);
-        tc::tma_load_2d(sA + s * kATile, &mapA, &afull[s], kb * oz::KB, i * Ap + m0);
-      }
-      if (!ok) break;
-    }
-  } else if (warp == 2 && lane == 0) {
-    // ---------------- TMA producer, B slice groups
-    for (int kb = 0; kb < num_kb; ++kb) {
-      const int g = kb & 1;
-      const uint32_t gph = (uint32_t)(kb >> 1) & 1u;
-      if (!mbar_wait_spin(&bempty[g], gph ^ 1u)) {
-        atomicExch(err, tc::ERR_TIMEOUT_EMPTY);
-        *abort_flag = 1;
-        break;
-      }
-      if (*abort_flag) break;
-      tc::mbar_expect_tx(&bfull[g], kBGroup);
-      for (int j = 0; j < oz::S; ++j)
-        tc::tma_load_2d(sB + (g * oz::S + j) * kBTile, &mapB, &bfull[g], kb * oz::KB, j * Bp + n0);
-    }
-  } else if (warp == kWaiterWarp) {
-    // ---------------- waiter: every mbarrier wait on behalf of the MMA warp (see
-    // oz_gemm_kernel), one handoff per A tile at named barrier 2, num_kb * 7 in all
-    bool failed = false;
-    for (int kb = 0; kb < num_kb; ++kb) {
-      const int q = kb / kKbPerChunk;
-      const bool chunk_start = (kb % kKbPerChunk) == 0;
-      const int g = kb & 1;
-      const uint32_t gph = (uint32_t)(kb >> 1) & 1u;
-      int okw = 1;
-      if (lane == 0 && !failed) {
-        if (chunk_start && q > 0 && !mbar_wait_spin(tfree, (uint32_t)(q - 1) & 1u)) {  // chunk q-1 read out
-          atomicExch(err, tc::ERR_TIMEOUT_DONE);
-          *abort_flag = 1;
-          okw = 0;
-        } else if (!mbar_wait_spin(&bfull[g], gph)) {
-          atomicExch(err, tc::ERR_TIMEOUT_FULL);
-          *abort_flag = 1;
-          okw = 0;
-        }
-      }
-      failed = failed || !__shfl_sync(0xffffffffu, okw, 0);
-      for (int i = 0; i < oz::S; ++i) {
-        const int ai = kb * oz::S + i;
-        const int s = ai % kAStages;
-        const uint32_t ph = (uint32_t)(ai / kAStages) & 1u;
-        int oka = 1;
-        if (lane == 0 && !failed) {
-          if (!mbar_wait_spin(&afull[s], ph)) {
-            atomicExch(err, tc::ERR_TIMEOUT_FULL);
-            *abort_flag = 1;
-            oka = 0;
-          } else if (*abort_flag) {
-            oka = 0;
-          }
-        }
-        failed = failed || !__shfl_sync(0xffffffffu, oka, 0);
-        (void)handoff(failed);
-      }
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer (lane 0; the whole warp meets the waiter at barrier 2)
-    constexpr uint32_t idesc = tc::make_idesc(1, oz::BN);
-    constexpr uint32_t idesc2 = tc::make_idesc(1, 2 * oz::BN);
-    constexpr uint32_t idesc3 = tc::make_idesc(1, 3 * oz::BN);
-    constexpr uint32_t idesc4 = tc::make_idesc(1, 4 * oz::BN);
-    const uint64_t adesc0 = tc::make_sw128_desc(tc::smem_u32(sA));
-    const uint64_t bdesc0 = tc::make_sw128_desc(tc::smem_u32(sB));
-    bool& failed = mma_failed;
-    for (int kb = 0; kb < num_kb; ++kb) {
-      const bool chunk_start = (kb % kKbPerChunk) == 0;
-      const int g = kb & 1;
-      for (int i = 0; i < oz::S; ++i) {
-        failed = handoff(false) || failed;
-        tc::fence_after_sync();
-        const int ai = kb * oz::S + i;
-        const int s = ai % kAStages;
-        if (lane == 0) {
-          if (!failed) {
-            const uint64_t ad = adesc0 + (uint64_t)(s * (kATile >> 4));
-            const uint64_t bd = bdesc0 + (uint64_t)(g * oz::S * (kBTile >> 4));
-            // slice 0 is the first to reach every level, so in a chunk's first k-block its MMAs
-            // overwrite and all later ones accumulate; up to four pairs (i, j .. j + 3), i.e.
-            // adjacent levels and adjacent B slices, go into one MMA of N = 64 .. 256
-            const uint32_t first = (!chunk_start || i > 0) ? 1u : 0u;
-#pragma unroll
-            for (int j = 0; j < oz::S; j += kLevelsPerMma) {
-              if (i + j < oz::S) {
-                const int gl = min(kLevelsPerMma, oz::S - i - j);
-                const uint32_t id = gl == 1 ? idesc : gl == 2 ? idesc2 : gl == 3 ? idesc3 : idesc4;
-                const uint32_t d = tmem + (uint32_t)((i + j) * oz::BN);
-                const uint64_t bj = bd + (uint64_t)(j * (kBTile >> 4));
-                tc::mma_issue<true>(d, ad, bj, id, first);
-                tc::mma_issue<true>(d, ad + 2, bj + 2, id, 1u);
-                tc::mma_issue<true>(d, ad + 4, bj + 4, id, 1u);
-                tc::mma_issue<true>(d, ad + 6, bj + 6, id, 1u);
-              }
-            }
-            mma_any = true;
-          }
-          // also after a failure (the A producer never starves), unless the failure came
-          // before any MMA: then no asynchronous arrive may outlive the CTA
-          if (mma_any || !failed) tc::mma_commit(&aempty[s]);
-        }
-        __syncwarp();
-      }
-      if (lane == 0 && (mma_any || !failed)) {
-        tc::mma_commit(&bempty[g]);
-        if ((kb % kKbPerChunk) == kKbPerChunk - 1 || kb == num_kb - 1) tc::mma_commit(cdone);
-      }
-      __syncwarp();
-    }
-  } else if (warp >= 3) {
-    // ---------------- epilogue: running double-float sums of 32 columns per thread
-    const int quarter = warp & 3;
-    const int cbase = ((warp - 3) >> 2) * 32;
-    const int row = m0 + quarter * 32 + lane;
-    float rh[32], rl[32];
-#pragma unroll
-    for (int t = 0; t < 32; ++t) rh[t] = rl[t] = 0.f;
-    bool go = true;
-    for (int q = 0; q < nchunks && go; ++q) {
-      int okw = 1;
-      if (lane == 0) {
-        okw = tc::mbar_wait(cdone, (uint32_t)q & 1u) ? 1 : 0;
-        if (!okw) {
-          atomicExch(err, tc::ERR_TIMEOUT_DONE);
-          *abort_flag = 1;
-        }
-        if (*abort_flag) okw = 0;
-      }
-      okw = __shfl_sync(0xffffffffu, okw, 0);
-      if (!okw) {
-        go = false;
-        break;
-      }
-      tc::fence_after_sync();
-      const int ea = row < M ? eA[(int64_t)q * M + row] : 0;
-#pragma unroll
-      for (int c8 = 0; c8 < 32; c8 += 8) {
-        uint32_t v[oz::S][8];
-#pragma unroll
-        for (int L = 0; L < oz::S; ++L) tmem_ld8_nowait(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(L * oz::BN + cbase + c8), v[L]);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const float f4 = __uint_as_float(v[4][t]), f5 = __uint_as_float(v[5][t]), f6 = __uint_as_float(v[6][t]);
-          float tail = __fmul_rn(f6, pow2f(-oz::BITS * 8));
-          tail = __fadd_rn(tail, __fmul_rn(f5, pow2f(-oz::BITS * 7)));
-          tail = __fadd_rn(tail, __fmul_rn(f4, pow2f(-oz::BITS * 6)));
-          float hh = tail, ll = 0.f;
-          df_add_f(hh, ll, __fmul_rn(__uint_as_float(v[3][t]), pow2f(-oz::BITS * 5)));
-          df_add_f(hh, ll, __fmul_rn(__uint_as_float(v[2][t]), pow2f(-oz::BITS * 4)));
-          df_add_f(hh, ll, __fmul_rn(__uint_as_float(v[1][t]), pow2f(-oz::BITS * 3)));
-          df_add_f(hh, ll, __fmul_rn(__uint_as_float(v[0][t]), pow2f(-oz::BITS * 2)));
-          const int col = n0 + cbase + c8 + t;
-          const int ex = ea + (col < N ? eB[(int64_t)q * N + col] : 0);
-          df_add(rh[c8 + t], rl[c8 + t], scale2(hh, ex), scale2(ll, ex));
-        }
-      }
-      // this warp has read chunk q: release the accumulators
-      tc::fence_before_sync();
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(tfree)) : "memory");
-    }
-    if (go && row < M) {
-      if (o.mode == ACC_ROWMAJOR) {
-#pragma unroll
-        for (int t = 0; t < 32; ++t) {
-          const int col = n0 + cbase + t;
-          if (col < N) o.C[(int64_t)row * o.ldc + col] = (double)rh[t] + (double)rl[t];
-        }
-      } else if (o.mode == ACC_COLMAJOR) {  // lanes hold consecutive rows: coalesced per column
-#pragma unroll
-        for (int t = 0; t < 32; ++t) {
-          const int col = n0 + cbase + t;
-          if (col < N) {
-            const double v = (double)rh[t] + (double)rl[t];
-            o.C[(int64_t)col * o.ldc + row] = v;
-            if (o.C32) o.C32[(int64_t)col * o.ldc + row] = (float)v;
-          }
-        }
-      } else {  // ACC_ROWSQ
-        double sq = 0.0;
-#pragma unroll
-        for (int t = 0; t < 32; ++t) {
-          const double v = (double)rh[t] + (double)rl[t];
-          if (n0 + cbase + t < N) sq = fma(v, v, sq);
-        }
-        o.sq[((int64_t)blockIdx.x * 2 + (cbase >> 5)) * o.ldc + row] = sq;
-      }
-    }
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 1) {
-    // all MMAs have completed once the last chunk was signalled (or a wait gave up)
-    if (lane == 0 && (mma_any || !mma_failed) && nchunks > 0)
-      (void)tc::mbar_wait_bounded(cdone, (uint32_t)(nchunks - 1) & 1u);
-    __syncwarp();
-    tc::fence_after_sync();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
-  }
-}
-
 // ------------------------------------------------------------ nonlinear step and back-projection
 // beta_ab = c^2 S_ab (T_ab - t_b) in double-float (T from its chunk partials), sliced
 // row-wise into the A operand of segment 2, with the row sums of each 256-column chunk.
@@ -1582,10 +1257,10 @@ gdml_status oz_matvec(OzMatvec& oz, const double* G, const float2* G2, const dou
     { oz_proj_slice_df_kernel<<<(unsigned)M, oz::KC, 3 * oz.N * sizeof(float2), st>>>(G2, oz.Xc2, v, M, oz.N, D, (int)oz.W1.nchunks, oz.Wf, oz.t, oz.t2, oz.W1.Rp, oz.W1.Kp, (bf16*)oz.W1.slices, oz.W1.e); count_launch(); }
     if (cdiv(D, 16) * oz.WT2.nchunks >= 2 * num_sms()) {
       dim3 g((unsigned)cdiv(D, 16), (unsigned)oz.WT2.nchunks);
-      { oz_slice_cols_kernel<float2, 16><<<g, 256, 0, st>>>(oz.Wf, D, 0, D, MB, oz.WT2.Rp, oz.WT2.Kp, (bf16*)oz.WT2.slices, oz.WT2.e); count_launch(); }
+      { oz_slice_cols_kernel<16><<<g, 256, 0, st>>>(oz.Wf, D, 0, D, MB, oz.WT2.Rp, oz.WT2.Kp, (bf16*)oz.WT2.slices, oz.WT2.e); count_launch(); }
     } else {
       dim3 g((unsigned)cdiv(D, 4), (unsigned)oz.WT2.nchunks);
-      { oz_slice_cols_kernel<float2, 4><<<g, 256, 0, st>>>(oz.Wf, D, 0, D, MB, oz.WT2.Rp, oz.WT2.Kp, (bf16*)oz.WT2.slices, oz.WT2.e); count_launch(); }
+      { oz_slice_cols_kernel<4><<<g, 256, 0, st>>>(oz.Wf, D, 0, D, MB, oz.WT2.Rp, oz.WT2.Kp, (bf16*)oz.WT2.slices, oz.WT2.e); count_launch(); }
     }
   } else {
     launch_proj(G, Xc, v, M, oz.N, D, oz.W, D, oz.t, st);
@@ -1636,120 +1311,6 @@ void oz_destroy(OzMatvec& oz) {
   for (void* p : oz.allocs) cudaFree(p);
   oz.allocs.clear();
   oz.ready = false;
-}
-
-// C (lower triangle) = X X^T for the k rows of X, each of K entries, sliced by `slice`
-template <typename SliceFn>
-static gdml_status syrk_sliced(int64_t k, int64_t K, double* C, int64_t ldc, const SliceFn& slice, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(oz_gemm_acc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal) !=
-        cudaSuccess)
-      return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(sliced syrk)");
-    attr_set = true;
-  }
-  OzMatvec t;
-  OzOperand a;
-  // one operand serves as A and B (a second map with the B box height)
-  gdml_status s = make_operand(t, a, k, K, oz::BM, st);
-  CUtensorMap mapB;
-  if (s == GDML_OK && !make_kmajor_map(&mapB, a.slices, true, (uint64_t)a.Kp, (uint64_t)(oz::S * a.Rp),
-                                       (uint64_t)a.Kp, (uint32_t)oz::BN))
-    s = fail(GDML_ERR_CUDA, "cuTensorMapEncodeTiled failed (sliced syrk)");
-  if (s == GDML_OK) s = oz_alloc(t, &t.err, 1, st);
-  if (s == GDML_OK) {
-    slice(a);
-    dim3 grid((unsigned)cdiv(k, oz::BN), (unsigned)cdiv(k, oz::BM));
-    const AccOut o{ACC_ROWMAJOR, 1, 0, C, nullptr, nullptr, ldc};
-    { oz_gemm_acc_kernel<<<grid, kThreadsAcc, kSmemTotal, st>>>(a.map, mapB, (int)a.Rp, (int)a.Rp, (int)k, (int)k, (int)(a.Kp / oz::KB), a.e, a.e, o, t.err); count_launch(); }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) s = fail(GDML_ERR_CUDA, std::string("sliced syrk launch: ") + cudaGetErrorString(e));
-  }
-  if (s == GDML_OK) {
-    int h = 0;
-    if (cudaMemcpyAsync(&h, t.err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      s = fail(GDML_ERR_CUDA, "sliced syrk: synchronise");
-    else if (h)
-      s = fail(GDML_ERR_TIMEOUT, "sliced syrk: a tcgen05 pipeline wait timed out");
-  }
-  cudaStreamSynchronize(st);
-  oz_destroy(t);
-  return s;
-}
-
-gdml_status oz_syrk_lower(const float* L, int64_t n, int64_t k, double* C, int64_t ldc, cudaStream_t st) {
-  if (n <= 0 || k <= 0) return fail(GDML_ERR_ARG, "oz_syrk_lower: empty sizes");
-  // the k columns of L (stride n) are the rows of L^T
-  return syrk_sliced(k, n, C, ldc, [&](OzOperand& a) {
-    dim3 g((unsigned)k, (unsigned)a.nchunks);
-    { oz_slice_rows_f32_kernel<<<g, 256, 0, st>>>(L, n, n, k, a.Rp, a.Kp, (bf16*)a.slices, a.e); count_launch(); }
-  }, st);
-}
-
-gdml_status oz_syrk_lower_f64(const double* X, int64_t rows, int64_t K, int64_t ldx, double* C, int64_t ldc,
-                              cudaStream_t st) {
-  if (rows <= 0 || K <= 0) return fail(GDML_ERR_ARG, "oz_syrk_lower_f64: empty sizes");
-  return syrk_sliced(rows, K, C, ldc, [&](OzOperand& a) {
-    dim3 g((unsigned)rows, (unsigned)a.nchunks);
-    { oz_slice_rows_kernel<<<g, 256, 0, st>>>(X, ldx, K, rows, a.Rp, a.Kp, (bf16*)a.slices, a.e, nullptr, nullptr); count_launch(); }
-  }, st);
-}
-
-gdml_status oz_gemm_tall(const double* A, int64_t n, int64_t K, const double* B, int64_t NB, int64_t ldb, bool tri_b,
-                         bool rowsq, double* out, float* out32, cudaStream_t st) {
-  if (n <= 0 || K <= 0 || NB <= 0 || !A || !B || !out) return fail(GDML_ERR_ARG, "oz_gemm_tall: bad arguments");
-  if (NB > ((int64_t)1 << 24) || K > ((int64_t)1 << 24)) return fail(GDML_ERR_ARG, "oz_gemm_tall: sizes too large");
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(oz_gemm_acc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal) !=
-        cudaSuccess)
-      return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(sliced gemm)");
-    attr_set = true;
-  }
-  // rows of A per panel: the panel's slices (7 x P x Kp BF16) are the only copy of A made
-  const int64_t P = std::min<int64_t>(cdiv(n, oz::BM) * oz::BM, 65536);
-  const int64_t nbt = cdiv(NB, oz::BN);
-  OzMatvec t;
-  OzOperand a, b;
-  double* sq = nullptr;
-  gdml_status s = make_operand(t, b, NB, K, oz::BN, st);
-  if (s == GDML_OK) s = make_operand(t, a, P, K, oz::BM, st);
-  if (s == GDML_OK && rowsq) s = oz_alloc(t, &sq, (size_t)(2 * nbt * n), st);
-  if (s == GDML_OK) s = oz_alloc(t, &t.err, 1, st);
-  if (s == GDML_OK) {
-    slice_rows(B, ldb, b, st);
-    for (int64_t p0 = 0; p0 < n && s == GDML_OK; p0 += P) {
-      const int64_t rows = std::min(P, n - p0);
-      a.rows = rows;  // exponents of this panel are indexed [chunk][rows]
-      {
-        dim3 g((unsigned)cdiv(rows, 16), (unsigned)a.nchunks);
-        oz_slice_cols_kernel<double><<<g, 256, 0, st>>>(A, n, p0, rows, K, a.Rp, a.Kp, (bf16*)a.slices, a.e);
-        count_launch();
-      }
-      AccOut o{rowsq ? ACC_ROWSQ : ACC_COLMAJOR, 0, tri_b ? 1 : 0, rowsq ? nullptr : out + p0,
-               (!rowsq && out32) ? out32 + p0 : nullptr, rowsq ? sq + p0 : nullptr, n};
-      dim3 grid((unsigned)nbt, (unsigned)cdiv(rows, oz::BM));
-      { oz_gemm_acc_kernel<<<grid, kThreadsAcc, kSmemTotal, st>>>(a.map, b.map, (int)a.Rp, (int)b.Rp, (int)rows, (int)NB, (int)(a.Kp / oz::KB), a.e, b.e, o, t.err); count_launch(); }
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) s = fail(GDML_ERR_CUDA, std::string("sliced tall gemm launch: ") + cudaGetErrorString(e));
-    }
-    if (s == GDML_OK && rowsq) {
-      oz_rowsq_reduce_kernel<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(sq, (int)(2 * nbt), n, out);
-      count_launch();
-    }
-  }
-  if (s == GDML_OK) {
-    int h = 0;
-    if (cudaMemcpyAsync(&h, t.err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      s = fail(GDML_ERR_CUDA, "sliced tall gemm: synchronise");
-    else if (h)
-      s = fail(GDML_ERR_TIMEOUT, "sliced tall gemm: a tcgen05 pipeline wait timed out");
-  }
-  cudaStreamSynchronize(st);
-  oz_destroy(t);
-  return s;
 }
 
 cudaError_t set_wait_limit_oz(uint32_t polls) { return tc::set_wait_limit_here(polls); }

@@ -15,7 +15,13 @@ namespace gdml {
 namespace {
 
 using bf16 = __nv_bfloat16;
-constexpr float kMagic = 12582912.f;  // 1.5 2^23: adding it rounds |x| < 2^22 to an integer
+using rns::f2;
+using rns::kMagic;
+using rns::p_add;
+using rns::p_fma;
+using rns::p_mul;
+using rns::p_sub;
+using rns::residue2;
 
 // ------------------------------------------------------------ double-float helpers
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -80,14 +86,7 @@ __device__ __forceinline__ int row_scale(unsigned m, float sqrtK, int bits) {
   return bits - e;
 }
 
-// ------------------------------------------------------------ packed FP32 pairs
-// Two independent entries per instruction (f32x2); a - b as one fused multiply-add by -1 (exact).
-__device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
-__device__ __forceinline__ float2 p_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 p_sub(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f), a); }
-__device__ __forceinline__ float2 p_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 p_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-
+// ------------------------------------------------------------ packed FP32 pairs (rns.cuh)
 struct df2 {  // two double-float numbers h + l
   float2 h, l;
 };
@@ -135,19 +134,6 @@ __device__ __forceinline__ void digits2(df2 x, float2 (&d)[4]) {
   }
   // the last digit: h is below 2^13 and l below h's ulp
   d[0] = p_add(p_add(p_add(x.h, x.l), f2(kMagic)), f2(-kMagic));
-}
-
-// centred residues of two integers given by digits, modulo p_i, as packed BF16.  Every product and
-// sum is an integer below 2^24; the quotient's rounding error (< 0.002) leaves |r| <= p / 2 + 1/2.
-template <int NM>
-__device__ __forceinline__ uint32_t residue2(const rns::Crt<NM>& C, int i, const float2 (&d)[4]) {
-  float2 t = p_fma(d[1], f2(C.c1[i]), d[0]);
-  t = p_fma(d[2], f2(C.c2[i]), t);
-  t = p_fma(d[3], f2(C.c3[i]), t);
-  const float2 q = p_add(p_fma(t, f2(C.inv[i]), f2(kMagic)), f2(-kMagic));
-  const float2 r = p_fma(q, f2(-C.p[i]), t);
-  const __nv_bfloat162 b = __floats2bfloat162_rn(r.x, r.y);
-  return *reinterpret_cast<const uint32_t*>(&b);
 }
 
 // The fraction (x . y) / P of two neighbouring outputs, in units of 2^-43, from NM words of two
@@ -488,18 +474,39 @@ struct GemmArgs {
   int64_t ldo;
   uint16_t* out;
   int* err;
+  int units;
+  // the builds' products (BUILD)
+  int shape;    // RNS_FULL, RNS_TRI, RNS_LOWER
+  int row0;     // first row of A
+  int n_first;  // RNS_LOWER: column tiles of the first row of tiles
+  int tiles;    // RNS_LOWER: tiles
 };
 
 struct Unit {
   int mod, m0, n0, seg, kb0, nk;
   int64_t plane;
 };
+template <bool BUILD>
 __device__ __forceinline__ Unit unit_of(const GemmArgs& g, int u) {
   Unit x;
-  const int n = u % g.tn;
-  u /= g.tn;
-  const int m = u % g.tm;
-  u /= g.tm;
+  int n, m;
+  if (BUILD && g.shape == RNS_LOWER) {  // row m of tiles has n_first + m of them
+    n = u % g.tiles;
+    u /= g.tiles;
+    m = 0;
+    for (int w = g.n_first; n >= w; ++w, ++m) n -= w;
+  } else if (BUILD) {  // columns outermost, the longest K first (RNS_TRI)
+    const int rest = g.units / g.tn;
+    n = g.tn - 1 - u / rest;
+    u %= rest;
+    m = u % g.tm;
+    u /= g.tm;
+  } else {
+    n = u % g.tn;
+    u /= g.tn;
+    m = u % g.tm;
+    u /= g.tm;
+  }
   x.mod = u % g.nmod;
   const int sl = u / g.nmod;
   x.seg = sl / g.groups;
@@ -507,6 +514,8 @@ __device__ __forceinline__ Unit unit_of(const GemmArgs& g, int u) {
   x.nk = min(g.kb_group, g.nkb - x.kb0);
   x.m0 = m * (2 * kBM);
   x.n0 = n * g.bn;
+  // row c of B ends at its entry c
+  if (BUILD && g.shape == RNS_TRI) x.nk = max(0, min(x.nk, (x.n0 + g.bn + kKB - 1) / kKB - x.kb0));
   x.plane = (int64_t)sl * g.nmod + x.mod;
   return x;
 }
@@ -586,6 +595,7 @@ __device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr));
 }
 
+template <bool BUILD>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     rns_gemm_kernel(const __grid_constant__ GemmArgs g) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -600,7 +610,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int bn = g.bn, slots = g.slots;
   uint32_t rank;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  const int units = g.slabs * g.nmod * g.tm * g.tn;
+  const int units = g.units;
   const int u0 = blockIdx.x >> 1, du = gridDim.x >> 1;
   const int b_bytes = bn * 64;  // this CTA's half of a B tile
   uint8_t* smem_b = smem + slots * kATile;
@@ -645,9 +655,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     uint32_t ph = 1;
     bool ok = true;
     for (int u = u0; u < units && ok; u += du) {
-      const Unit x = unit_of(g, u);
+      const Unit x = unit_of<BUILD>(g, u);
       const CUtensorMap *mA = &g.a[x.seg], *mB = &g.b[x.seg];
-      const int ya = x.mod * g.Ra + x.m0 + (int)rank * kBM, yb = x.mod * g.Rb + x.n0 + (int)rank * (bn >> 1);
+      const int ya = x.mod * g.Ra + (BUILD ? g.row0 : 0) + x.m0 + (int)rank * kBM, yb = x.mod * g.Rb + x.n0 + (int)rank * (bn >> 1);
       int kx = x.kb0 * kKB;
       for (int kb = 0; kb < x.nk; ++kb, kx += kKB) {
         ok = wait_bar<false>(empty0 + 8u * slot, ph, limit, abort_flag);
@@ -681,7 +691,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     uint32_t ph = 0;
     bool ok = true;
     for (int u = u0; u < units && ok; u += du) {
-      const Unit x = unit_of(g, u);
+      const Unit x = unit_of<BUILD>(g, u);
       for (int k0 = 0; k0 < x.nk; k0 += kKbChunk) {
         const int len = min(kKbChunk, x.nk - k0);
         const uint32_t t = (uint32_t)(chunks & 1), acc = tmem + t * 256u;
@@ -720,7 +730,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const uint32_t tempty_leader = mapa(tempty0, 0);
     bool go = true;
     for (int u = u0; u < units && go; u += du) {
-      const Unit x = unit_of(g, u);
+      const Unit x = unit_of<BUILD>(g, u);
       const float2 np2 = f2(-g.p[x.mod]), inv2 = f2(g.inv[x.mod]);
       uint32_t acc[8][8];  // packed sums of residue + 256: columns 2w and 2w + 1 of group q
 #pragma unroll
@@ -1010,48 +1020,96 @@ static void gemm_shape(int64_t M, int64_t N, int64_t nkb, int64_t planes, int ca
 }
 
 // residues of A B^T (or of both segments' products) into out
-static gdml_status rns_gemm(const RnsOperand* A, const RnsOperand* B, int segs, int bn, int chunks,
-                            uint16_t* out, int64_t ldo, int* err, cudaStream_t st, int* slabs_out) {
+template <bool BUILD>
+static gdml_status launch_gemm(GemmArgs& g, int segs, int chunks, cudaStream_t st) {
   static bool attr_set = false;
   if (!attr_set) {
-    if (cudaFuncSetAttribute(rns_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
+    if (cudaFuncSetAttribute(rns_gemm_kernel<BUILD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
       return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(residue gemm)");
     attr_set = true;
-  }
-  GemmArgs g;
-  for (int s = 0; s < 2; ++s) {
-    g.a[s] = A[s < segs ? s : 0].map;
-    g.b[s] = B[s < segs ? s : 0].map;
   }
   for (int i = 0; i < rns::kMaxMod; ++i) {
     g.p[i] = (float)rns::kMods[i];
     g.inv[i] = 1.0f / (float)rns::kMods[i];
   }
   g.nmod = rns::kMvMods;
-  g.M = (int)A[0].rows;
-  g.N = (int)B[0].rows;
-  g.Ra = (int)A[0].rows;
-  g.Rb = (int)B[0].rows;
-  g.bn = bn;
-  g.tn = (int)cdiv(g.N, bn);
+  g.tn = (int)cdiv(g.N, g.bn);
   g.tm = (int)cdiv(g.M, 2 * kBM);
-  g.nkb = (int)(A[0].Kp / kKB);
   g.kb_group = chunks * kKbChunk;
   g.groups = (int)cdiv(g.nkb, g.kb_group);
   g.slabs = segs * g.groups;
-  g.slots = std::min(kMaxSlots, kRing / (kATile + bn * 64));
+  g.slots = std::min(kMaxSlots, kRing / (kATile + g.bn * 64));
+  int64_t tiles = (int64_t)g.tm * g.tn;
+  if (BUILD && g.shape == RNS_LOWER) {
+    g.n_first = g.row0 / (2 * kBM) + 1;
+    tiles = 0;
+    for (int m = 0; m < g.tm; ++m) tiles += g.n_first + m;
+    g.tiles = (int)tiles;
+  }
+  const int64_t units = (int64_t)g.slabs * g.nmod * tiles;
+  if (chunks > kMaxChunks) return fail(GDML_ERR_ARG, "residue gemm: too many K chunks per unit");
+  if (units > INT32_MAX / 2) return fail(GDML_ERR_ARG, "residue gemm: too many tiles");
+  g.units = (int)units;
+  const unsigned grid = 2u * (unsigned)std::min<int64_t>(units, std::max(num_sms() / 2, 1));
+  { rns_gemm_kernel<BUILD><<<grid, kThreads, kSmem, st>>>(g); count_launch(); }
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(GDML_ERR_CUDA, std::string("residue gemm launch: ") + cudaGetErrorString(e));
+  return GDML_OK;
+}
+
+static gdml_status rns_gemm(const RnsOperand* A, const RnsOperand* B, int segs, int bn, int chunks,
+                            uint16_t* out, int64_t ldo, int* err, cudaStream_t st, int* slabs_out) {
+  GemmArgs g{};
+  for (int s = 0; s < 2; ++s) {
+    g.a[s] = A[s < segs ? s : 0].map;
+    g.b[s] = B[s < segs ? s : 0].map;
+  }
+  g.M = g.Ra = (int)A[0].rows;
+  g.N = g.Rb = (int)B[0].rows;
+  g.bn = bn;
+  g.nkb = (int)(A[0].Kp / kKB);
   g.ldo = ldo;
   g.out = out;
   g.err = err;
-  const int64_t units = (int64_t)g.slabs * g.nmod * g.tm * g.tn;
-  if (chunks > kMaxChunks) return fail(GDML_ERR_ARG, "residue gemm: too many K chunks per unit");
-  if (units > INT32_MAX / 2) return fail(GDML_ERR_ARG, "residue gemm: too many tiles");
-  const unsigned grid = 2u * (unsigned)std::min<int64_t>(units, std::max(num_sms() / 2, 1));
-  { rns_gemm_kernel<<<grid, kThreads, kSmem, st>>>(g); count_launch(); }
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(GDML_ERR_CUDA, std::string("residue gemm launch: ") + cudaGetErrorString(e));
+  RNS_TRY(launch_gemm<false>(g, segs, chunks, st));
   if (slabs_out) *slabs_out = g.groups;
   return GDML_OK;
+}
+
+gdml_status rns_product(RnsProduct& q, int* err, cudaStream_t st) {
+  GemmArgs g{};
+  if (!make_kmajor_map(&g.a[0], q.A, true, (uint64_t)q.Kp, (uint64_t)(rns::kMvMods * q.Ra), (uint64_t)q.Kp, kBM) ||
+      !make_kmajor_map(&g.b[0], q.B, true, (uint64_t)q.Kp, (uint64_t)(rns::kMvMods * q.Rb), (uint64_t)q.Kp,
+                       (uint32_t)q.bn / 2))
+    return fail(GDML_ERR_CUDA, "cuTensorMapEncodeTiled failed (residue product)");
+  g.a[1] = g.a[0];
+  g.b[1] = g.b[0];
+  g.M = (int)q.M;
+  g.N = (int)q.N;
+  g.Ra = (int)q.Ra;
+  g.Rb = (int)q.Rb;
+  g.bn = q.bn;
+  g.nkb = (int)(q.Kp / kKB);
+  g.ldo = q.ldo;
+  g.out = q.out;
+  g.err = err;
+  g.shape = q.shape;
+  g.row0 = (int)q.row0;
+  return launch_gemm<true>(g, 1, q.chunks, st);
+}
+
+void rns_product_shape(RnsProduct& q, int cap) {
+  int bn = 256, g = 1;
+  gemm_shape(q.M, q.N, q.Kp / kKB, rns::kMvMods, cap, &bn, &g);
+  if (q.shape == RNS_LOWER && bn != 256) {  // square tiles: the diagonal's fall on the rows' last
+    bn = 256;
+    const int64_t nch = cdiv(q.Kp, rns::kChunk);
+    const int64_t units = cdiv(q.M, 2 * kBM) * cdiv(q.N, 256) * rns::kMvMods;
+    g = (int)cdiv(nch, std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cap, nch), num_sms() / 2 / units)));
+  }
+  q.bn = bn;
+  q.chunks = std::min(std::max(g, 1), kMaxChunks);
+  q.slabs = (int)cdiv(cdiv(q.Kp, rns::kChunk), q.chunks);
 }
 
 template <typename F>

@@ -38,6 +38,7 @@ constexpr int kMods[kMaxMod] = {361, 359, 358, 355, 353, 351, 349, 347, 343, 341
 
 constexpr int kMvMods = 14;  // the matvec's: P = 2^117.9
 constexpr int kMvBits = 57;  // both operands: 2^114 < P / 2
+constexpr int kChunk = 512;  // K entries whose products of residues sum exactly in FP32
 constexpr int kDigit = 14;  // residues are formed from digits of 14 bits, four per integer
 constexpr int kBad = -100000;  // scale of a row that holds a NaN or an infinity
 
@@ -103,6 +104,27 @@ struct Crt {
   }
 };
 
+// two independent entries per instruction (f32x2); a - b as one fused multiply-add by -1 (exact)
+constexpr float kMagic = 12582912.f;  // 1.5 2^23: adding it rounds |x| < 2^22 to an integer
+__device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 p_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 p_sub(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f), a); }
+__device__ __forceinline__ float2 p_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 p_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// centred residues of two integers given by digits, modulo p_i, as packed BF16.  Every product and
+// sum is an integer below 2^24; the quotient's rounding error (< 0.002) leaves |r| <= p / 2 + 1/2.
+template <int NM>
+__device__ __forceinline__ uint32_t residue2(const Crt<NM>& C, int i, const float2 (&d)[4]) {
+  float2 t = p_fma(d[1], f2(C.c1[i]), d[0]);
+  t = p_fma(d[2], f2(C.c2[i]), t);
+  t = p_fma(d[3], f2(C.c3[i]), t);
+  const float2 q = p_add(p_fma(t, f2(C.inv[i]), f2(kMagic)), f2(-kMagic));
+  const float2 r = p_fma(q, f2(-C.p[i]), t);
+  const __nv_bfloat162 b = __floats2bfloat162_rn(r.x, r.y);
+  return *reinterpret_cast<const uint32_t*>(&b);
+}
+
 }  // namespace rns
 
 // One operand as residues: NM planes of rows x Kp BF16 (K-major, zero padded), and the power of
@@ -162,5 +184,33 @@ void rns_destroy(RnsMatvec& r);
 // K chunks per unit: the value used for a requested one, given the slabs that the buffers hold
 int rns_chunks(int64_t nch, int g, int cap);
 cudaError_t set_wait_limit_rns(uint32_t polls);
+
+// ---- the products of the OZAKI preconditioner build: A B^T mod each p_i.  Operands: NM planes of
+// Ra (Rb) rows x Kp BF16 residues, Kp a multiple of 64, neither with the CRT factor folded in
+enum { RNS_FULL = 0, RNS_TRI = 1, RNS_LOWER = 2 };
+struct RnsProduct {
+  const __nv_bfloat16 *A = nullptr, *B = nullptr;
+  int64_t Ra = 0, Rb = 0, Kp = 0;
+  int64_t M = 0, N = 0;  // outputs: rows row0 .. row0 + M of A against rows 0 .. N of B
+  int64_t row0 = 0;      // a multiple of 256 (0 unless RNS_LOWER)
+  int shape = RNS_FULL;  // RNS_TRI: row c of B is zero past entry c; RNS_LOWER: only columns <= the row are wanted
+  uint16_t* out = nullptr;  // [slab][modulus][M][ldo]: sums over the slab's chunks of residue + 256
+  int64_t ldo = 0;          // a multiple of 16
+  int bn = 256, chunks = 1, slabs = 1;  // columns per tile, chunks per unit, K groups
+};
+// tile and K groups for a product of these sizes (at most `cap` groups unless a unit can't hold the chunks)
+void rns_product_shape(RnsProduct& q, int cap);
+gdml_status rns_product(RnsProduct& q, int* err, cudaStream_t st);
+
+// C = A B^T for a tall A (n x K, column-major: entry (r, j) at A[j n + r]) and B (NB x K, row-major,
+// row stride ldb; lower triangular when tri_b, so K entries past each row's diagonal are skipped).
+// rowsq = false: C stored column-major, out[c n + r] (and as FP32 at out32[c n + r] when out32 is not
+// null); out may alias A.  rowsq = true: out[r] = sum_c C[r][c]^2 (n doubles).  Synchronises the stream.
+gdml_status rns_gemm_tall(const double* A, int64_t n, int64_t K, const double* B, int64_t NB, int64_t ldb, bool tri_b,
+                          bool rowsq, double* out, float* out32, cudaStream_t st);
+// lower triangle of C = X X^T (k x k, FP64, row stride ldc) for X (k x K, row stride ldx).
+// Synchronises the stream.
+gdml_status rns_syrk_lower(const float* X, int64_t k, int64_t K, int64_t ldx, double* C, int64_t ldc, cudaStream_t st);
+gdml_status rns_syrk_lower(const double* X, int64_t k, int64_t K, int64_t ldx, double* C, int64_t ldc, cudaStream_t st);
 
 }  // namespace gdml

@@ -110,3 +110,22 @@ def test_long_training_side(M):
     ctx.destroy()
     f64.destroy()
     assert rel(got, ref) <= BOUND
+
+
+@pytest.mark.parametrize("N,M,k", [(5, 40, 1), (9, 60, 33), (9, 100, 255), (9, 100, 257), (8, 64, 520), (9, 650, 20)])
+def test_woodbury_core_from_residue_products(N, M, k):
+    """The core C = lambda I + L^T L of a built preconditioner by residue products (one tile, the
+    tiles' edges, three rows of tiles, K in groups, two K panels), through the apply
+    z = (r - L C^-1 L^T r) / lambda against FP64 with the same stored L.  C's entries err by about
+    2^-50 |L|^2, the apply's double-float sums by 2^-46: 2^6 2^-46 cond(C) bounds z's relative error."""
+    R = torch.from_numpy(synth.geometries(synth.template(N, 2), M, 0.1, 3)).cuda()
+    r = np.random.default_rng(k).standard_normal(3 * N * M)
+    ctx = gdml.kernel_setup(R, 3.0, 1e-3, precision="ozaki")
+    ctx.precond_build("uniform", k, seed=1)
+    L = ctx.precond_factor().cpu().numpy()
+    z = ctx.precond_apply(torch.from_numpy(r).cuda()).cpu().numpy()
+    ctx.destroy()
+    C = L.T @ L + 1e-3 * np.eye(L.shape[1])
+    ref = (r - L @ np.linalg.solve(C, L.T @ r)) / 1e-3
+    rel = np.linalg.norm(z - ref) / np.linalg.norm(ref)
+    assert rel <= 2.0 ** -40 * np.linalg.cond(C)

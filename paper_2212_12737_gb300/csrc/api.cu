@@ -271,22 +271,6 @@ gdml_status read_status(gdml_ctx* c, int* h) {
   return GDML_OK;
 }
 
-// K[:, cols] (n x ncols, column-major) for the Nystrom factor: in double-float with each
-// geometry's operands reused across the columns (DF64 / OZAKI contexts, whose preconditioner
-// is FP32-stored), else in FP64
-gdml_status get_cols(gdml_ctx* c, const int64_t* cols, int64_t ncols, double* out) {
-  if (c->Ssym > 1) {
-    if (!launch_kcol_sym(cols, ncols, c->X, c->G, c->S, c->P64, 2 * c->MB, c->M, c->MB, c->N, c->D, c->pis, c->pinv,
-                         c->Ssym, c->c, out, c->n, nullptr, c->st))
-      return ctx_fail(c, GDML_ERR_ARG, "kernel columns with symmetries: descriptor too long for shared memory");
-    return check_launch(c, "kcol (symmetries)");
-  }
-  if (!(c->X2 && launch_kcol_bulk_df(cols, ncols, c->X2, c->G2, c->S, c->P64, 2 * c->M, c->M, c->N, c->D, c->c, out,
-                                      c->n, c->st)))
-    launch_kcol(cols, ncols, c->X, c->G, c->S, c->P64, 2 * c->M, c->M, c->N, c->D, c->c, out, c->n, nullptr, c->st);
-  return check_launch(c, "kcol");
-}
-
 struct Scratch {
   gdml_ctx* c;
   std::vector<void*> ptrs;
@@ -300,6 +284,31 @@ struct Scratch {
     return s;
   }
 };
+
+
+// K[:, cols] (n x ncols, column-major) for the Nystrom factor: in double-float with each
+// geometry's operands reused across the columns (DF64 / OZAKI contexts, whose preconditioner
+// is FP32-stored), else in FP64
+gdml_status get_cols(gdml_ctx* c, const int64_t* cols, int64_t ncols, double* out) {
+  if (c->Ssym > 1) {
+    if (!launch_kcol_sym(cols, ncols, c->X, c->G, c->S, c->P64, 2 * c->MB, c->M, c->MB, c->N, c->D, c->pis, c->pinv,
+                         c->Ssym, c->c, out, c->n, nullptr, c->st))
+      return ctx_fail(c, GDML_ERR_ARG, "kernel columns with symmetries: descriptor too long for shared memory");
+    return check_launch(c, "kcol (symmetries)");
+  }
+  if (c->X2) {
+    Scratch s{c, {}};
+    float2* w = nullptr;
+    TRY(s.get(&w, (size_t)kcol_bulk_scratch(ncols, c->N, c->D)));
+    if (launch_kcol_bulk_df(cols, ncols, c->X2, c->G2, c->S, c->P64, 2 * c->M, c->M, c->N, c->D, c->c, out, c->n, w,
+                            c->st)) {
+      CTRY(c, cudaStreamSynchronize(c->st));  // (the scratch is freed)
+      return check_launch(c, "kcol");
+    }
+  }
+  launch_kcol(cols, ncols, c->X, c->G, c->S, c->P64, 2 * c->M, c->M, c->N, c->D, c->c, out, c->n, nullptr, c->st);
+  return check_launch(c, "kcol");
+}
 
 // In-place lower Cholesky of the k x k work matrix (copy of src) with the
 // jitter rule of Eq. 5's factorisation: eps = 1e-14 tr/k, x10 up to 1e-6 tr/k.

@@ -12,9 +12,11 @@
 //  center_like   query descriptors centred on the training centre (force prediction; dist_tab
 //             also makes the tables of query geometries against the training set)
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "rns.cuh"
 
 namespace gdml {
 
@@ -508,106 +510,217 @@ __global__ void __launch_bounds__(256) kcol_df_kernel(const int64_t* __restrict_
   }
 }
 
-// Many kernel columns at once (the Nystrom factor's K_nk, Eq. 5): the same double-float
-// arithmetic as kcol_df_kernel, with geometry a's x_a and g_a staged ONCE per CTA and reused by
-// a block of CB columns (W warps, one column at a time each), instead of once per (a, column).
-// grid (M, ceil(ncols / CB)).  Shared memory: 4 D float pairs for geometry a, plus per warp
-// N (w) + 2 D (x_a - x_b, u) float pairs.
-constexpr int kColBlock = 64;
-__global__ void __launch_bounds__(256) kcol_bulk_df_kernel(const int64_t* __restrict__ cols, int64_t ncols,
+// Many kernel columns at once (the Nystrom factor's K_nk, Eq. 5), in double-float like kcol_df_kernel:
+//   K[a, col] = J_a^T (A_ab w + coef (x_a - x_b)),  coef = -c^2 S_ab (x_a - x_b) . w,  w = J_b e_col.
+// Per entry the second term is a sum of N - 1 products, bound by the FP32 lanes, so it decides the
+// layout: a warp takes one atom of NA geometries a against 64 columns, two per lane in packed
+// arithmetic (the sums are compensated and combined in FP64), g_a and x_a as broadcasts from shared
+// memory, x_b from an array transposed to columns.  w has N - 1 entries (the pairs of one atom), so
+// the first term and coef take one pass over them per (a, column).
+// N = 42, M = 1001, 1500 columns: 26.7 ms as one warp per (a, column) gathering pairs from shared
+// memory, 5.1 ms so.
+constexpr int kColBlock = 128;   // columns per CTA
+constexpr int kColBatch = 2048;  // columns per launch (their transposed operands: (D + 2 N) float pairs each)
+
+// the columns' operands: XP[p][column pair] (hi, hi, lo, lo), W[j][column] = +-g_b on the pairs (i, j)
+// of the column's atom i, XG[j][column] = x_b there
+__global__ void kcol_prep_kernel(const int64_t* __restrict__ cols, int64_t ncols, int64_t LC,
+                                 const float2* __restrict__ X2, const float2* __restrict__ G2, int N, int D,
+                                 float4* __restrict__ XP, float2* __restrict__ W, float2* __restrict__ XG) {
+  const int64_t cp = blockIdx.x;
+  const int64_t ca = min(2 * cp, ncols - 1), cb = min(2 * cp + 1, ncols - 1);  // (padding repeats the last)
+  const int B = 3 * N;
+  const int64_t col[2] = {cols[ca], cols[cb]};
+  const float2 *x0 = X2 + col[0] / B * D, *x1 = X2 + col[1] / B * D;
+  for (int p = threadIdx.x; p < D; p += blockDim.x) {
+    const float2 u = x0[p], v = x1[p];
+    XP[p * (LC >> 1) + cp] = make_float4(u.x, v.x, u.y, v.y);
+  }
+  for (int e = threadIdx.x; e < 2 * N; e += blockDim.x) {
+    const int h = e >= N ? 1 : 0, j = e - h * N;
+    const int64_t b = col[h] / B;
+    const int l = (int)(col[h] - b * B), i = l / 3, q = l - 3 * i;
+    float2 w = make_float2(0.f, 0.f), x = w;
+    if (j != i) {
+      const int p = pair_idx(i, j);
+      const float2 g = G2[(b * D + p) * 3 + q];
+      w = i > j ? dfk_neg(g) : g;
+      x = X2[b * D + p];
+    }
+    W[j * LC + 2 * cp + h] = w;
+    XG[j * LC + 2 * cp + h] = x;
+  }
+}
+
+__device__ __forceinline__ double dfk_double(float2 a) { return (double)a.x + (double)a.y; }
+
+struct df2c {  // compensated sums of two columns
+  float2 h, l;
+};
+// s += g d, g the same for both columns
+__device__ __forceinline__ void mac2(df2c& s, float gh, float gl, float2 dh, float2 dl) {
+  using namespace rns;
+  const float2 p = p_mul(f2(gh), dh);
+  float2 e = p_fma(f2(gh), dh, p_mul(p, f2(-1.f)));
+  e = p_fma(f2(gh), dl, e);
+  e = p_fma(f2(gl), dh, e);
+  const float2 t = p_add(s.h, p), bb = p_sub(t, s.h);
+  s.l = p_add(s.l, p_add(p_add(p_sub(s.h, p_sub(t, bb)), p_sub(p, bb)), e));
+  s.h = t;
+}
+// (dh, dl) = a - x or x - a for the two columns x
+template <bool NEG>
+__device__ __forceinline__ void diff2(float ah, float al, float4 x, float2& dh, float2& dl) {
+  using namespace rns;
+  const float2 xh = make_float2(x.x, x.y), xl = make_float2(x.z, x.w);
+  const float2 uh = NEG ? xh : f2(ah), vh = NEG ? f2(ah) : xh, ul = NEG ? xl : f2(al), vl = NEG ? f2(al) : xl;
+  const float2 s = p_sub(uh, vh), bb = p_sub(s, uh);
+  const float2 e = p_add(p_sub(p_sub(uh, p_sub(s, bb)), p_add(vh, bb)), p_sub(ul, vl));
+  dh = p_add(s, e);
+  dl = p_sub(e, p_sub(dh, s));
+}
+
+template <int NA>
+__global__ void __launch_bounds__(256) kcol_bulk_df_kernel(const int64_t* __restrict__ cols, int64_t ncols, int64_t LC,
+                                                           const float4* __restrict__ XP, const float2* __restrict__ W,
+                                                           const float2* __restrict__ XG,
                                                            const float2* __restrict__ X2,
                                                            const float2* __restrict__ G2,
                                                            const double* __restrict__ S,
                                                            const double* __restrict__ A, int64_t ldA, int64_t M,
                                                            int N, int D, double c2, double* __restrict__ out,
                                                            int64_t ldo) {
-  extern __shared__ float2 shb[];
-  const int W = blockDim.x >> 5;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float2* sxa = shb;                                   // D: x_a
-  float2* sga = sxa + D;                               // 3 D: g_a
-  float2* wsp = sga + 3 * D + (size_t)warp * (N + 2 * D);  // N: +-g_b on the pairs (i, j), by partner j
-  float2* dab = wsp + N;                               // D: x_a - x_b
-  float2* u = dab + D;                                 // D
-  const int64_t a = blockIdx.x;
+  extern __shared__ float4 shb[];
+  __shared__ double s_coef[NA][kColBlock], s_aab[NA][kColBlock], s_self[NA][3][kColBlock];
+  __shared__ int s_atom[kColBlock];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int B = 3 * N;
-  {
-    const float2* Xa = X2 + a * D;
-    const float2* Ga = G2 + a * D * 3;
-    for (int e = threadIdx.x; e < 4 * D; e += blockDim.x) {
-      if (e < D)
-        sxa[e] = Xa[e];
-      else
-        sga[e - D] = Ga[e - D];
-    }
+  const int64_t a0 = (int64_t)blockIdx.x * NA, c0 = (int64_t)blockIdx.y * kColBlock;
+  // pair p of geometry a: (g_0, g_1), (g_2, x_a)
+  for (int e = tid; e < NA * D; e += 256) {
+    const int ai = e >= D ? 1 : 0, p = e - ai * D;
+    const int64_t r = min(a0 + ai, M - 1) * D + p;
+    const float2 g0 = G2[3 * r], g1 = G2[3 * r + 1], g2 = G2[3 * r + 2], x = X2[r];
+    shb[2 * e] = make_float4(g0.x, g0.y, g1.x, g1.y);
+    shb[2 * e + 1] = make_float4(g2.x, g2.y, x.x, x.y);
   }
   __syncthreads();
-  const int64_t c_end = min(ncols, (int64_t)(blockIdx.y + 1) * kColBlock);
-  for (int64_t c = (int64_t)blockIdx.y * kColBlock + warp; c < c_end; c += W) {
-    const int64_t col = cols[c];
-    const int64_t b = col / B;
-    const int l = (int)(col - b * B), i = l / 3, q = l - 3 * i;
-    const float2* Xb = X2 + b * D;
-    const float2* Gb = G2 + b * D * 3;
-    for (int j = lane; j < N; j += 32) {
-      float2 w = make_float2(0.f, 0.f);
-      if (j != i) {
-        const float2 g = Gb[3 * pair_idx(i, j) + q];
-        w = (i > j) ? dfk_neg(g) : g;
-      }
-      wsp[j] = w;
-    }
-    for (int p = lane; p < D; p += 32) dab[p] = dfk_add(sxa[p], dfk_neg(Xb[p]));  // x_a - x_b
-    __syncwarp();
-    const float2 sab = dfk_mul(dfk_split(c2), dfk_split(S[b * M + a]));
-    const float2 aab = dfk_split(A[b * ldA + a]);
-    float2 sd = make_float2(0.f, 0.f);
-    for (int j = lane; j < N; j += 32)
-      if (j != i) sd = dfk_add(sd, dfk_mul(dab[pair_idx(i, j)], wsp[j]));
-    for (int o = 16; o > 0; o >>= 1)
-      sd = dfk_add(sd, make_float2(__shfl_xor_sync(0xffffffffu, sd.x, o), __shfl_xor_sync(0xffffffffu, sd.y, o)));
-    const float2 coef = dfk_neg(dfk_mul(sab, sd));
-    for (int p = lane; p < D; p += 32) u[p] = dfk_mul(coef, dab[p]);
-    __syncwarp();
-    for (int j = lane; j < N; j += 32)
-      if (j != i) {
-        const int p = pair_idx(i, j);
-        u[p] = dfk_add(u[p], dfk_mul(aab, wsp[j]));
-      }
-    __syncwarp();
-    for (int l2 = lane; l2 < B; l2 += 32) {
-      const int i2 = l2 / 3, q2 = l2 - 3 * i2;
-      float2 s2 = make_float2(0.f, 0.f);
+  if (tid < NA * kColBlock) {  // one thread per (a, column)
+    const int ai = tid / kColBlock, cl = tid % kColBlock;
+    const int64_t c = c0 + cl, a = min(a0 + ai, M - 1);
+    const int64_t col = cols[min(c, ncols - 1)], b = col / B;
+    const int i = (int)(col - b * B) / 3;
+    const float4* sg = shb + 2 * ai * D;
+    float2 sd = make_float2(0.f, 0.f), self[3] = {sd, sd, sd};
+    if (c < LC)
       for (int j = 0; j < N; ++j) {
-        if (j == i2) continue;
-        const int p = pair_idx(i2, j);
-        const float2 gj = dfk_mul(sga[3 * p + q2], u[p]);
-        s2 = dfk_add(s2, (i2 > j) ? dfk_neg(gj) : gj);
+        if (j == i) continue;
+        const int p = pair_idx(i, j);
+        const float4 ga = sg[2 * p], gb = sg[2 * p + 1];
+        const float2 w = W[j * LC + c], x = XG[j * LC + c];
+        sd = dfk_add(sd, dfk_mul(dfk_add(make_float2(gb.z, gb.w), dfk_neg(x)), w));
+        const float2 v = i > j ? dfk_neg(w) : w;
+        self[0] = dfk_add(self[0], dfk_mul(make_float2(ga.x, ga.y), v));
+        self[1] = dfk_add(self[1], dfk_mul(make_float2(ga.z, ga.w), v));
+        self[2] = dfk_add(self[2], dfk_mul(make_float2(gb.x, gb.y), v));
       }
-      out[c * ldo + a * B + l2] = (double)s2.x + (double)s2.y;
+    const double aab = A[b * ldA + a];
+    s_coef[ai][cl] = -(c2 * S[b * M + a]) * dfk_double(sd);
+    s_aab[ai][cl] = aab;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) s_self[ai][q][cl] = aab * dfk_double(self[q]);
+    if (ai == 0) s_atom[cl] = i;
+  }
+  __syncthreads();
+  const int64_t hc = LC >> 1;
+  for (int task = warp; task < 2 * N; task += 8) {  // (64 columns, atom)
+    const int chunk = task >= N ? 1 : 0, i = task - chunk * N;
+    const int64_t cb = c0 + 64 * chunk;
+    if (cb >= ncols) break;
+    const float4* xp = XP + (cb >> 1) + lane;
+    df2c y[NA][3];
+#pragma unroll
+    for (int k = 0; k < NA; ++k)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) y[k][q] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    auto term = [&](int p, auto neg) {
+      const float4 x = xp[p * hc];
+#pragma unroll
+      for (int k = 0; k < NA; ++k) {
+        const float4 ga = shb[2 * (k * D + p)], gb = shb[2 * (k * D + p) + 1];
+        float2 dh, dl;
+        diff2<decltype(neg)::value>(gb.z, gb.w, x, dh, dl);
+        mac2(y[k][0], ga.x, ga.y, dh, dl);
+        mac2(y[k][1], ga.z, ga.w, dh, dl);
+        mac2(y[k][2], gb.x, gb.y, dh, dl);
+      }
+    };
+    // J_a^T has +g on the pairs' first atoms, -g on their second
+#pragma unroll 2
+    for (int j = 0; j < i; ++j) term(pair_idx(i, j), std::true_type{});
+#pragma unroll 2
+    for (int j = i + 1; j < N; ++j) term(pair_idx(i, j), std::false_type{});
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const int cl = 64 * chunk + 2 * lane + v;
+      if (c0 + cl >= ncols) break;
+      const int ic = s_atom[cl];
+      const double w = ic == i ? 0.0 : (i > ic ? -1.0 : 1.0) * dfk_double(W[i * LC + c0 + cl]);
+      const int p = ic == i ? 0 : pair_idx(i, ic);
+#pragma unroll
+      for (int k = 0; k < NA; ++k) {
+        if (a0 + k >= M) break;
+        const float4 ga = shb[2 * (k * D + p)], gb = shb[2 * (k * D + p) + 1];
+        const float2 g[3] = {make_float2(ga.x, ga.y), make_float2(ga.z, ga.w), make_float2(gb.x, gb.y)};
+        double* o = out + (c0 + cl) * ldo + (a0 + k) * B + 3 * i;
+        const double coef = s_coef[k][cl], aw = s_aab[k][cl] * w;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const double t = ic == i ? s_self[k][q][cl] : aw * dfk_double(g[q]);
+          o[q] = fma(coef, dfk_double(v ? make_float2(y[k][q].h.y, y[k][q].l.y) : make_float2(y[k][q].h.x, y[k][q].l.x)), t);
+        }
+      }
     }
-    __syncwarp();  // wsp, dab and u are rewritten for the warp's next column
   }
 }
 
-bool launch_kcol_bulk_df(const int64_t* cols, int64_t ncols, const float2* X2, const float2* G2, const double* S,
-                         const double* A, int64_t ldA, int64_t M, int N, int D, double c, double* out, int64_t ldo,
-                         cudaStream_t st) {
-  const size_t fixed = 4 * (size_t)D * sizeof(float2), per_warp = ((size_t)N + 2 * (size_t)D) * sizeof(float2);
-  const size_t budget = 200 * 1024;
-  if (fixed + per_warp > budget || ncols < 1 || M > 2147483647 || cdiv(ncols, kColBlock) > 65535) return false;
-  const int W = (int)std::min<size_t>(8, (budget - fixed) / per_warp);
-  const size_t smem = fixed + W * per_warp;
+int64_t kcol_bulk_scratch(int64_t ncols, int N, int D) {
+  return std::min<int64_t>(kColBatch, cdiv(ncols, kColBlock) * kColBlock) * (D + 2 * (int64_t)N);
+}
+
+template <int NA>
+static bool kcol_bulk(const int64_t* cols, int64_t ncols, const float2* X2, const float2* G2, const double* S,
+                      const double* A, int64_t ldA, int64_t M, int N, int D, double c, double* out, int64_t ldo,
+                      float2* scratch, cudaStream_t st) {
+  const size_t smem = 2 * NA * (size_t)D * sizeof(float4);
   static size_t attr = 0;
-  if (smem > 48 * 1024 && smem > attr) {
-    if (cudaFuncSetAttribute(kcol_bulk_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+  if (smem > 32 * 1024 && smem > attr) {
+    if (cudaFuncSetAttribute(kcol_bulk_df_kernel<NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
       return false;
     attr = smem;
   }
-  dim3 g((unsigned)M, (unsigned)cdiv(ncols, kColBlock));
-  { kcol_bulk_df_kernel<<<g, 32 * W, smem, st>>>(cols, ncols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo); count_launch(); }
+  for (int64_t c0 = 0; c0 < ncols; c0 += kColBatch) {
+    const int64_t nc = std::min<int64_t>(kColBatch, ncols - c0), LC = cdiv(nc, kColBlock) * kColBlock;
+    float4* XP = reinterpret_cast<float4*>(scratch);
+    float2 *W = scratch + LC * D, *XG = W + LC * N;
+    { kcol_prep_kernel<<<(unsigned)(LC / 2), 128, 0, st>>>(cols + c0, nc, LC, X2, G2, N, D, XP, W, XG); count_launch(); }
+    const dim3 g((unsigned)cdiv(M, NA), (unsigned)(LC / kColBlock));
+    { kcol_bulk_df_kernel<NA><<<g, 256, smem, st>>>(cols + c0, nc, LC, XP, W, XG, X2, G2, S, A, ldA, M, N, D, c * c, out + c0 * ldo, ldo); count_launch(); }
+  }
   return true;
+}
+
+// Two geometries per CTA halve the loads of x_b; one where their 32 bytes per pair and geometry leave no
+// room for two (D > 3400) or where two would leave SMs without a CTA
+bool launch_kcol_bulk_df(const int64_t* cols, int64_t ncols, const float2* X2, const float2* G2, const double* S,
+                         const double* A, int64_t ldA, int64_t M, int N, int D, double c, double* out, int64_t ldo,
+                         float2* scratch, cudaStream_t st) {
+  const size_t one = 2 * (size_t)D * sizeof(float4), most = 212 * 1024;
+  if (one > most || ncols < 1 || M > 2147483647) return false;
+  if (2 * one <= most && cdiv(M, 2) * cdiv(ncols, kColBlock) >= num_sms())
+    return kcol_bulk<2>(cols, ncols, X2, G2, S, A, ldA, M, N, D, c, out, ldo, scratch, st);
+  return kcol_bulk<1>(cols, ncols, X2, G2, S, A, ldA, M, N, D, c, out, ldo, scratch, st);
 }
 
 bool launch_kcol_df(const int64_t* cols, int64_t ncols, const float2* X2, const float2* G2, const double* S,

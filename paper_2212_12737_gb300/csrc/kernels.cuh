@@ -27,11 +27,13 @@ void launch_dist_tab(const double* X, int64_t M, int D, double c, double* S, dou
 bool launch_kcol_df(const int64_t* cols, int64_t ncols, const float2* X2, const float2* G2, const double* S,
                     const double* A, int64_t ldA, int64_t M, int N, int D, double c, double* out, int64_t ldo,
                     const int* stop_flag, cudaStream_t st);
-// many kernel columns at once in double-float (the Nystrom factor's K_nk); false (nothing
-// launched) when geometry a's operands and the per-warp scratch do not fit in 200 KB
+// many kernel columns at once in double-float (the Nystrom factor's K_nk), with a scratch of
+// kcol_bulk_scratch float pairs; false (nothing launched) when a geometry's operands do not fit in
+// shared memory (D > 6784)
+int64_t kcol_bulk_scratch(int64_t ncols, int N, int D);  // float pairs
 bool launch_kcol_bulk_df(const int64_t* cols, int64_t ncols, const float2* X2, const float2* G2, const double* S,
                          const double* A, int64_t ldA, int64_t M, int N, int D, double c, double* out, int64_t ldo,
-                         cudaStream_t st);
+                         float2* scratch, cudaStream_t st);
 // permutational symmetries (pis, pinv: S x D descriptor-entry permutations of the group)
 void launch_sym_gather(const double* in, int64_t M, int D, const int* pis, int S, const double* xcB, double* out,
                        double* t, cudaStream_t st);

@@ -82,6 +82,26 @@ __device__ __forceinline__ void pair_of(int p, int& i, int& j) {
   i = ii;
   j = p - ii * (ii - 1) / 2;
 }
+// Programmatic dependent launch: grid_wait returns once the kernels before this one in the stream have
+// completed, grid_trigger lets the next one start (when every CTA has called it or has ended)
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// launches a kernel that may start before the one ahead of it in the stream has ended (it calls grid_wait)
+template <typename... P, typename... A>
+void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 __device__ __forceinline__ int pair_idx(int i, int j) {  // requires i != j
   return i > j ? i * (i - 1) / 2 + j : j * (j - 1) / 2 + i;
 }

@@ -424,7 +424,6 @@ __global__ void __launch_bounds__(256) kcol_df_kernel(const int64_t* __restrict_
                                                       int64_t ldA, int64_t M, int N, int D, double c2,
                                                       double* __restrict__ out, int64_t ldo,
                                                       const int* __restrict__ stop_flag) {
-  if (stop_flag && *stop_flag) return;
   extern __shared__ float2 shf[];
   const int W = blockDim.x >> 5;
   float2* wsp = shf;        // N: +-g_b on the pairs (i, j), indexed by partner j
@@ -434,12 +433,12 @@ __global__ void __launch_bounds__(256) kcol_df_kernel(const int64_t* __restrict_
   float2* u = sxa + D;                                 // D
   float2* sga = u + D;                                 // 3 D: g_a
   const int64_t c = blockIdx.y;
-  const int64_t col = cols[c];
   const int B = 3 * N;
   const int64_t a = (int64_t)blockIdx.x * W + warp;
   const bool live = a < M;
   float2 sab = make_float2(0.f, 0.f), aab = sab;
-  // geometry a's operands do not depend on the pivot: their loads go first
+  // geometry a's operands do not depend on the pivot: their loads go first, before the step that
+  // selects it has ended
   if (live) {  // eight independent loads in flight per lane, then the shared-memory stores
     const float2* Xa = X2 + a * D;
     const float2* Ga = G2 + a * D * 3;
@@ -460,6 +459,10 @@ __global__ void __launch_bounds__(256) kcol_df_kernel(const int64_t* __restrict_
       }
     }
   }
+  grid_wait();
+  if (stop_flag && *stop_flag) return;
+  grid_trigger();  // (after the wait: the next kernel may rely on what came before this one)
+  const int64_t col = cols[c];
   const int64_t b = col / B;
   const int l = (int)(col - b * B), i = l / 3, q = l - 3 * i;
   const float2* Xb = X2 + b * D;
@@ -739,7 +742,10 @@ bool launch_kcol_df(const int64_t* cols, int64_t ncols, const float2* X2, const 
     attr = wsmem;
   }
   dim3 g((unsigned)cdiv(M, W), (unsigned)ncols);
-  { kcol_df_kernel<<<g, 32 * W, wsmem, st>>>(cols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag); count_launch(); }
+  if (stop_flag)  // Algorithm 1's step: follows the previous one without waiting for it to drain
+    { launch_after(kcol_df_kernel, g, 32 * W, wsmem, st, cols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag); count_launch(); }
+  else
+    { kcol_df_kernel<<<g, 32 * W, wsmem, st>>>(cols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag); count_launch(); }
   return true;
 }
 

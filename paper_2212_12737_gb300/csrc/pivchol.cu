@@ -412,18 +412,25 @@ __global__ void __launch_bounds__(kArgThreads) pc_finish_select_df_kernel(
 // Algorithm 1 step m in one TMA-staged pass: the Schur sums s_i = sum_{j<m} L[i + j n] prow[j]
 // of ws_gemv_n_kernel's SCHUR mode, followed row by row (as each chunk's sums are combined)
 // by pc_finish_select_df_kernel's work: l_{i,m}, column m of L, the residual diagonal, the
-// argmax and the trace.  The last CTA to finish selects the pivot of step m + 1, performs
-// the swap and gathers that pivot's row of L into prow (every CTA has read prow by then).
+// argmax and the trace.  The last CTA to finish selects the pivot of step m + 1 and performs the swap.
+// Bounded by HBM while it streams; what comes before and after is a chain of latencies, at n = 63,000,
+// k = 2,000 at the end 36 us of a step's 111 (160 ms for the build; 140 ms so), therefore
+//  - it starts beside the step's kernel column (see launch_after) and waits for it only at the end;
+//  - lanes fetch the pivot row's entries straight from L, 32 / CPW tiles ahead (gathered by the last CTA
+//    of the step before: up to 8 us);
+//  - the rows' state is loaded before the stream, and the argmax carries the row with its position;
+//  - the leading `keep` columns stay in L2 (64 MB of them: 4 ms of the build; 96 MB: 1 ms).
 template <int NT>
 __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
-    const __grid_constant__ CUtensorMap map, int64_t n, int64_t m, int64_t nch, int select, float* __restrict__ L,
-    float* __restrict__ prow, const double* __restrict__ col, double* __restrict__ d,
+    const __grid_constant__ CUtensorMap map, int64_t n, int64_t m, int64_t nch, int64_t keep, int select, float* __restrict__ L,
+    const double* __restrict__ col, double* __restrict__ d,
     unsigned char* __restrict__ chosen, int64_t* __restrict__ perm, int64_t* __restrict__ posof,
     int64_t* __restrict__ pivots, double* __restrict__ trace, PivState* __restrict__ ps,
-    ArgMaxPart* __restrict__ part, unsigned* __restrict__ ticket, int* __restrict__ err, int evict_first) {
+    ArgMaxPart* __restrict__ part, unsigned* __restrict__ ticket, int* __restrict__ err) {
   constexpr int RC = 128 * NT, COLS = 32 / NT, CPW = 4 / NT;
   constexpr int kW = kWsWarps + 1;
-  if (ps->stop) return;
+  grid_trigger();  // (the next column's CTAs may start once all of these have)
+  if (__ldcg(&ps->stop)) return;  // (up to grid_wait, state is read past L1, which may hold the last step's)
   extern __shared__ uint8_t ws_smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(ws_smem_raw) + kWsAlign - 1) &
                                              ~uintptr_t(kWsAlign - 1));
@@ -437,11 +444,11 @@ __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
   __shared__ int64_t sp[kW];
   __shared__ double ss[kW];
   __shared__ bool last;
-  __shared__ int64_t s_piv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntiles = (int)((m + COLS - 1) / COLS);
-  const int64_t piv = ps->piv;
-  const double lmm = ps->lmm, ilmm = ps->ilmm;
+  const int64_t piv = __ldcg(&ps->piv);
+  const double lmm = __ldcg(&ps->lmm), ilmm = __ldcg(&ps->ilmm);
+  const int64_t other = select && threadIdx.x == 0 ? __ldcg(perm + m + 1) : 0;
   if (threadIdx.x == 0) {
     ws_init(full, empty, cbar, abort_flag);
     issued_s = 0;
@@ -451,8 +458,7 @@ __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
   double sum = 0.0;
   if (warp == kWsWarps) {
     if (lane == 0)
-      issued_s = evict_first ? ws_produce<NT, true>(&map, ring, full, empty, abort_flag, nch, ntiles, err)
-                             : ws_produce<NT, false>(&map, ring, full, empty, abort_flag, nch, ntiles, err);
+      issued_s = ws_produce<NT, true>(&map, ring, full, empty, abort_flag, nch, ntiles, (int)(keep / COLS), err);
   } else {
     WsRing rp;
     uint32_t ci = 0;
@@ -463,13 +469,31 @@ __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
       for (int t = 0; t < NT; ++t)
 #pragma unroll
         for (int q = 0; q < 2; ++q) h2[t][q] = l2[t][q] = make_float2(0.f, 0.f);
+      const int64_t i = ch * RC + threadIdx.x;  // 256 consumer threads, one row each
+      const bool mine = (int)threadIdx.x < RC && i < n;
+      bool chs = true;
+      double di = 0.0;
+      int64_t pi = 0;
+      if (mine) {
+        chs = __ldcg(chosen + i) != 0;
+        di = __ldcg(d + i);
+        pi = __ldcg(posof + i);
+      }
+      // entry (pivot, column) of the tiles s0 .. s0 + 32 / CPW: lane l holds tile l / CPW, column l % CPW
+      auto fetch = [&](int s0) {
+        const int64_t j = (int64_t)(s0 + lane / CPW) * COLS + warp * CPW + lane % CPW;
+        return j < m ? __ldcg(L + piv + j * n) : 0.f;
+      };
+      float xcur = 0.f, xnext = fetch(0);
       for (int s = 0; s < ntiles; ++s) {
+        const int sb = s % (32 / CPW);
+        if (sb == 0) {
+          xcur = xnext;
+          xnext = fetch(s + 32 / CPW);
+        }
         float xv[CPW];
 #pragma unroll
-        for (int c = 0; c < CPW; ++c) {
-          const int64_t j = (int64_t)s * COLS + warp * CPW + c;
-          xv[c] = j < m ? prow[j] : 0.f;
-        }
+        for (int c = 0; c < CPW; ++c) xv[c] = __shfl_sync(0xffffffffu, xcur, sb * CPW + c);
         if (!ws_consume_wait(&full[rp.slot], rp.phase, abort_flag, err)) {
           go = false;
           break;
@@ -505,14 +529,11 @@ __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
           cmb[warp * 256 + 128 * t + 4 * lane + 2 * q] = make_float2(h2[t][q].x, l2[t][q].x);
           cmb[warp * 256 + 128 * t + 4 * lane + 2 * q + 1] = make_float2(h2[t][q].y, l2[t][q].y);
         }
+      grid_wait();  // the kernel column
+      const double ci_ = mine ? __ldcg(col + i) : 0.0;
       if (!ws_consumer_sync(&cbar[0], ci & 1u, abort_flag, err)) break;
-      const int64_t i0 = ch * RC;
-      const int rr = threadIdx.x;  // 256 consumer threads, one row each
-      if (rr < RC && i0 + rr < n) {
-        const int64_t i = i0 + rr;
-        const bool chs = chosen[i] != 0;
-        const double ci_ = col[i], di = d[i];
-        const int64_t pi = posof[i];
+      if (mine) {
+        const int rr = threadIdx.x;
         float hh = cmb[rr].x, ll = cmb[rr].y;
 #pragma unroll
         for (int w = 1; w < kWsWarps; ++w) df_add_pair_pc(hh, ll, cmb[w * 256 + rr].x, cmb[w * 256 + rr].y);
@@ -524,7 +545,7 @@ __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
           const double dn = __dsub_rn(di, __dmul_rn(lr, lr));
           d[i] = dn;
           sum += dn;
-          best = better(best, ArgMax{dn, pi});
+          best = better(best, ArgMax{dn, (pi << 32) | i});  // (n <= 2^30)
         } else if (i == piv) {
           L[i + m * n] = (float)lmm;
         }
@@ -532,6 +553,7 @@ __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
       if (!ws_consumer_sync(&cbar[1], ci & 1u, abort_flag, err)) break;
     }
   }
+  grid_wait();
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag) ws_drain(full, issued_s);
   // CTA reduction (the producer warp holds neutral values), then the grid's through part[]
@@ -568,10 +590,18 @@ __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
   {
     ArgMax bt{-1.0 / 0.0, INT64_MAX};
     double st = 0.0;
-    volatile ArgMaxPart* vp = part;
-    for (unsigned q = threadIdx.x; q < gridDim.x; q += blockDim.x) {
-      bt = better(bt, ArgMax{vp[q].v, vp[q].pos});
-      st += vp[q].sum;
+    for (unsigned q0 = threadIdx.x; q0 < gridDim.x; q0 += 2 * blockDim.x) {
+      const unsigned q1 = q0 + blockDim.x;
+      const ArgMaxPart* p0 = part + q0;
+      const ArgMaxPart* p1 = part + (q1 < gridDim.x ? q1 : q0);
+      const ArgMax a0{__ldcg(&p0->v), __ldcg(&p0->pos)}, a1{__ldcg(&p1->v), __ldcg(&p1->pos)};
+      const double s0 = __ldcg(&p0->sum), s1 = __ldcg(&p1->sum);
+      bt = better(bt, a0);
+      st += s0;
+      if (q1 < gridDim.x) {
+        bt = better(bt, a1);
+        st += s1;
+      }
     }
     for (int o = 16; o > 0; o >>= 1) {
       const ArgMax ob{__shfl_xor_sync(0xffffffffu, bt.v, o), (int64_t)__shfl_xor_sync(0xffffffffu, (long long)bt.pos, o)};
@@ -594,49 +624,29 @@ __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
       sw += __shfl_xor_sync(0xffffffffu, sw, o);
     }
     if (lane == 0) {
-      const ArgMax b = bw;
       *ticket = 0u;
       if (trace) trace[m] = sw;
-      s_piv = -1;
       if (select) {
-        const int64_t m1 = m + 1;
-        if (!(b.v > 0.0) || b.pos >= n) {
+        const int64_t m1 = m + 1, pos = bw.pos >> 32, p = bw.pos & 0xffffffff;
+        if (!(bw.v > 0.0) || pos >= n) {
           ps->stop = 1;
           ps->rank = m1;
         } else {
-          const int64_t p = perm[b.pos];
-          const int64_t other = perm[m1];
-          perm[b.pos] = other;
+          const double l = sqrt(bw.v);
+          perm[pos] = other;
           perm[m1] = p;
-          posof[other] = b.pos;
+          posof[other] = pos;
           posof[p] = m1;
           pivots[m1] = p;
           chosen[p] = 1;
-          ps->lmm = sqrt(d[p]);
-          ps->ilmm = 1.0 / ps->lmm;
+          ps->lmm = l;
+          ps->ilmm = 1.0 / l;
           ps->piv = p;
           ps->rank = m1 + 1;
-          s_piv = p;
         }
       }
     }
   }
-  __syncthreads();
-  const int64_t p = s_piv;
-  if (p >= 0)  // the next pivot's row of L, columns 0..m (column m written above, fenced)
-    for (int64_t j0 = threadIdx.x; j0 <= m; j0 += 8 * (int64_t)blockDim.x) {
-      float pv[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int64_t j = j0 + (int64_t)u * blockDim.x;
-        pv[u] = j <= m ? L[p + j * n] : 0.f;
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int64_t j = j0 + (int64_t)u * blockDim.x;
-        if (j <= m) prow[j] = pv[u];
-      }
-    }
 }
 
 int pivchol_schur_groups() { return kSchurMaxGroups; }
@@ -653,23 +663,21 @@ void pivchol_run_df(const PivCholArgs& a, float* L, cudaStream_t st) {
   // step 0's pivot
   { pc_argmax_kernel<<<arg_blocks(), kArgThreads, 0, st>>>(0, a.n, 1, a.d, a.perm, a.chosen, a.pivots, nullptr,
                                                        a.ps, a.part, a.ticket, a.posof); count_launch(); }
-  if (plan.ok) {  // two launches per step: the kernel column, then Schur sums + finish
+  if (plan.ok) {  // two launches per step: the kernel column, and Schur sums + finish beside it
     static bool attr = false;
     if (!attr) {
       cudaFuncSetAttribute(pc_schur_finish_ws_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWsSmemN);
       cudaFuncSetAttribute(pc_schur_finish_ws_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWsSmemN);
       attr = true;
     }
+    const int64_t keep = ((int64_t)64 << 20) / (4 * a.n);
     for (int64_t m = 0; m < a.k; ++m) {
       a.get_col(a.pivots + m, a.col, &a.ps->stop, st);
       const int select = m + 1 < a.k ? 1 : 0;
-      // once the first m columns no longer fit in L2 they are streamed evict-first, so the
-      // kernel column's operands (X, G as float pairs) and the per-row state stay resident
-      const int ef = (double)m * (double)a.n * 4.0 > 96.0 * 1024 * 1024 ? 1 : 0;
       if (plan.rc == 256)
-        { pc_schur_finish_ws_kernel<2><<<plan.grid, kWsThreads, kWsSmemN, st>>>(plan.map, a.n, m, plan.nch, select, L, a.prow, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err, ef); count_launch(); }
+        { launch_after(pc_schur_finish_ws_kernel<2>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
       else
-        { pc_schur_finish_ws_kernel<1><<<plan.grid, kWsThreads, kWsSmemN, st>>>(plan.map, a.n, m, plan.nch, select, L, a.prow, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err, ef); count_launch(); }
+        { launch_after(pc_schur_finish_ws_kernel<1>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
     }
     return;
   }

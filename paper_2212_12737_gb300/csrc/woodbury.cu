@@ -543,7 +543,7 @@ __global__ void __launch_bounds__(kWsThreads, 2)
   }
   __syncthreads();
   if (warp == kWsWarps) {
-    if (lane == 0) issued_s = ws_produce<NT, true>(&map, ring, full, empty, abort_flag, nch, ntiles, err);
+    if (lane == 0) issued_s = ws_produce<NT, false>(&map, ring, full, empty, abort_flag, nch, ntiles, 0, err);
   } else {
     WsRing rp;
     uint32_t ci = 0;

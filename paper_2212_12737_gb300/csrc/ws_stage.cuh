@@ -14,8 +14,8 @@ namespace gdml {
 // ---------------------------------------------------------------------------
 // TMA-staged passes.  One producer thread keeps a ring of 16 KB column tiles of
 // L in flight (cp.async.bulk.tensor, zero fill past n and k; an L2 evict-first
-// hint where L is streamed once: the apply's passes, and the Schur sums once the
-// columns no longer fit in L2); eight consumer warps do the double-float
+// hint where L is streamed once: the apply's passes, and the Schur sums but for the
+// leading columns, which stay in L2 from step to step); eight consumer warps do the double-float
 // arithmetic out of shared memory.  The bytes in flight per SM then no longer
 // depend on how many loads each warp holds in registers.
 // The L u pass and the Schur sums cut the rows into chunks of RC = 128 NT rows
@@ -155,16 +155,15 @@ struct WsRing {
 };
 
 // The producer: tile (chunk, s) = rows [chunk RC, chunk RC + RC) x columns [s COLS, s COLS + COLS).
-// Returns the number of tiles issued.
-template <int NT, bool EVICT_FIRST>
+// With KEEP the first `keep` tiles of a chunk keep their lines in L2, the others are evict-first.  Returns the
+// number of tiles issued.
+template <int NT, bool KEEP>
 __device__ uint32_t ws_produce(const CUtensorMap* map, uint8_t* ring, uint64_t* full, uint64_t* empty,
-                               volatile int* abort_flag, int64_t nch, int ntiles, int* err) {
+                               volatile int* abort_flag, int64_t nch, int ntiles, int keep, int* err) {
   constexpr int RC = 128 * NT, COLS = 32 / NT;
-  uint64_t policy;
-  if (EVICT_FIRST)
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-  else
-    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
+  uint64_t first, normal = 0;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
+  if (KEEP) asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(normal));
   WsRing rp;
   uint32_t issued = 0;
   for (int64_t ch = blockIdx.x; ch < nch; ch += gridDim.x)
@@ -176,7 +175,7 @@ __device__ uint32_t ws_produce(const CUtensorMap* map, uint8_t* ring, uint64_t* 
       }
       if (*abort_flag) return issued;
       tc::mbar_expect_tx(&full[rp.slot], kWsTile);
-      ws_tma_load(ring + rp.slot * kWsTile, map, &full[rp.slot], (int)(ch * RC), s * COLS, policy);
+      ws_tma_load(ring + rp.slot * kWsTile, map, &full[rp.slot], (int)(ch * RC), s * COLS, KEEP && s < keep ? normal : first);
     }
   return issued;
 }

@@ -86,9 +86,10 @@ __device__ __forceinline__ void pair_of(int p, int& i, int& j) {
 // completed, grid_trigger lets the next one start (when every CTA has called it or has ended)
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// launches a kernel that may start before the one ahead of it in the stream has ended (it calls grid_wait)
+// launches a kernel that with `early` may start before the one ahead of it in the stream has ended (it
+// calls grid_wait)
 template <typename... P, typename... A>
-void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+void launch_after(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -98,7 +99,7 @@ void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cuda
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 

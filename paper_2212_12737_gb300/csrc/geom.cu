@@ -742,10 +742,8 @@ bool launch_kcol_df(const int64_t* cols, int64_t ncols, const float2* X2, const 
     attr = wsmem;
   }
   dim3 g((unsigned)cdiv(M, W), (unsigned)ncols);
-  if (stop_flag)  // Algorithm 1's step: follows the previous one without waiting for it to drain
-    { launch_after(kcol_df_kernel, g, 32 * W, wsmem, st, cols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag); count_launch(); }
-  else
-    { kcol_df_kernel<<<g, 32 * W, wsmem, st>>>(cols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag); count_launch(); }
+  // stop_flag: Algorithm 1's step, which follows the previous one without waiting for it to drain
+  { launch_after(stop_flag != nullptr, kcol_df_kernel, g, 32 * W, wsmem, st, cols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag); count_launch(); }
   return true;
 }
 

@@ -675,9 +675,9 @@ void pivchol_run_df(const PivCholArgs& a, float* L, cudaStream_t st) {
       a.get_col(a.pivots + m, a.col, &a.ps->stop, st);
       const int select = m + 1 < a.k ? 1 : 0;
       if (plan.rc == 256)
-        { launch_after(pc_schur_finish_ws_kernel<2>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
+        { launch_after(true, pc_schur_finish_ws_kernel<2>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
       else
-        { launch_after(pc_schur_finish_ws_kernel<1>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
+        { launch_after(true, pc_schur_finish_ws_kernel<1>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
     }
     return;
   }

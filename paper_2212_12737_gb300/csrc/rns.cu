@@ -180,18 +180,22 @@ __device__ __forceinline__ df2 p_scale(df2 x, int e0, int e1) {
 }
 
 // ------------------------------------------------------------ operand kernels
-// Largest bits of |x| over the CTA's 256 threads
+// Largest bits of |x| over the CTA's threads (256 at most)
 __device__ __forceinline__ unsigned cta_max_bits(unsigned m, unsigned* red) {
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   m = red[0];
-#pragma unroll
-  for (int w = 1; w < 8; ++w) m = max(m, red[w]);
+  for (int w = 1; w < (int)blockDim.x >> 5; ++w) m = max(m, red[w]);
   return m;
 }
 
 __device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+
+// The columns' largest magnitudes are kept in kColCopies arrays, row a's CTA raising the (a mod
+// kColCopies)-th: with one array the CTAs of a round, which all see it cleared, queue up behind one
+// another's atomics (projection at M = 1,000, D = 210: 22.8 us, 8.6 with 16).
+constexpr int kColCopies = 16;
 
 // *p = max(*p, b) among all CTAs.  Most entries do not raise it: a plain look first (a stale value is
 // only smaller) spares L2 the atomics, which all fall on the same few lines
@@ -247,6 +251,7 @@ __global__ void __launch_bounds__(256) rns_rows_kernel(const double* __restrict_
   constexpr rns::Crt<NM> C{};
   const int64_t row = blockIdx.x;
   unsigned m = 0;
+  colmax += (row % kColCopies) * ((K + 1) & ~1);
   for (int k = threadIdx.x; k < K; k += 256) {
     const unsigned b = abs_bits(__double2float_ru(fabs(X[row * K + k])));
     raise_max(&colmax[k], b);
@@ -291,14 +296,25 @@ __global__ void __launch_bounds__(512) rns_proj_kernel(const float4* __restrict_
   float2* sv = sh + Dp;
   const float4* Ga = G3 + a * 3 * H;
   const float4* Xa = Xc2 + a * H;
+  colmax += (a % kColCopies) * Dp;
+  // the first descriptors' operands in one round of loads with v
+  const int q0 = min(tid, H - 1);
+  float4 g[3] = {Ga[q0], Ga[H + q0], Ga[2 * H + q0]}, x = Xa[q0];
+  uint2 pr = ij[q0], cm = __ldcg(reinterpret_cast<const uint2*>(colmax) + q0);
+  grid_trigger();
   for (int l = tid; l < B; l += nt) sv[l] = split_d(v[a * B + l]);
   __syncthreads();
   df2 t{f2(0.f), f2(0.f)};
   unsigned m = 0;
   for (int q = tid; q < H; q += nt) {  // descriptors 2q, 2q + 1
-    const float4 g[3] = {Ga[q], Ga[H + q], Ga[2 * H + q]};
-    const float4 x = Xa[q];
-    const uint2 pr = ij[q];  // 3 i | 3 j << 16 of each
+    if (q != tid) {
+      g[0] = Ga[q];
+      g[1] = Ga[H + q];
+      g[2] = Ga[2 * H + q];
+      x = Xa[q];
+      pr = ij[q];  // 3 i | 3 j << 16 of each
+      cm = __ldcg(reinterpret_cast<const uint2*>(colmax) + q);
+    }
     const float2 *vi0 = sv + (pr.x & 0xffffu), *vj0 = sv + (pr.x >> 16), *vi1 = sv + (pr.y & 0xffffu),
                  *vj1 = sv + (pr.y >> 16);
     df2 w{f2(0.f), f2(0.f)};
@@ -312,7 +328,6 @@ __global__ void __launch_bounds__(512) rns_proj_kernel(const float4* __restrict_
     sw[q] = wf;
     Wf[a * H + q] = wf;
     const unsigned b0 = abs_bits(w.h.x), b1 = abs_bits(w.h.y);
-    const uint2 cm = __ldcg(reinterpret_cast<const uint2*>(colmax) + q);
     if (b0 > cm.x) atomicMax(&colmax[2 * q], b0);
     if (b1 > cm.y) atomicMax(&colmax[2 * q + 1], b1);
     m = max(m, max(b0, b1));
@@ -353,6 +368,8 @@ __global__ void __launch_bounds__(256) rns_cols_kernel(const T* __restrict__ W, 
   __shared__ float2 tile[32][33];
   const int64_t b0 = (int64_t)blockIdx.x * 32;
   const int d0 = blockIdx.y * 32;
+  grid_trigger();
+  grid_wait();
   {
     const int c = threadIdx.x & 31;
 #pragma unroll
@@ -362,7 +379,13 @@ __global__ void __launch_bounds__(256) rns_cols_kernel(const T* __restrict__ W, 
     }
   }
   const int c = threadIdx.x >> 3, r = (threadIdx.x & 7) * 4;
-  const int s = d0 + c < D ? row_scale(colmax[d0 + c], sqrtf((float)MB) * 1.0001f, bits) : 0;
+  unsigned m = 0;
+  if (d0 + c < D)
+#pragma unroll
+    for (int i = 0; i < kColCopies / 8; ++i) m = max(m, colmax[((threadIdx.x & 7) + 8 * i) * ((D + 1) & ~1) + d0 + c]);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int s = row_scale(m, sqrtf((float)MB) * 1.0001f, bits);
   __syncthreads();
   if (d0 + c >= D || b0 + r >= Kp) return;
   if (b0 == 0 && r == 0) sc[d0 + c] = s;
@@ -642,6 +665,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     *abort_flag = 1;
   };
 
+  grid_trigger();
+  grid_wait();
   const uint32_t limit = tc::g_wait_limit;
   const uint32_t full0 = tc::smem_u32(full), empty0 = tc::smem_u32(empty);
   const uint32_t tfull0 = tc::smem_u32(tfull), tempty0 = tc::smem_u32(tempty);
@@ -799,10 +824,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 // beta_ab = c^2 S_ab (T_ab - t_b) in double-float (T from its residues) and its row residues.  One
 // CTA per row a, two columns per thread and step in packed arithmetic.  STAGE: beta is kept in shared
 // memory between the row's maximum and its residues; else (rows of more than kBetaStage columns) it
-// is formed twice.
+// is formed twice.  Four CTAs of 256 threads per SM (64 registers, 50 bytes of spills more than at 80)
+// against three; rows that fit the chip as CTAs of 128 threads run in one round (see row_threads).
 constexpr int64_t kBetaStage = 24 * 1024;
 template <int NM, bool STAGE>
-__global__ void __launch_bounds__(256, 3) rns_beta_kernel(const uint16_t* __restrict__ Tp, int slabs, int chunks,
+__global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* __restrict__ Tp, int slabs, int chunks,
                                                           int64_t M, int64_t MB, int64_t ldT,
                                                           const int* __restrict__ sA, const int* __restrict__ sW,
                                                           const float2* __restrict__ S2, const float2* __restrict__ t2,
@@ -818,6 +844,8 @@ __global__ void __launch_bounds__(256, 3) rns_beta_kernel(const uint16_t* __rest
   const int64_t plane = M * ldT;
   const float4* Sa = reinterpret_cast<const float4*>(S2 + a * ldT);
   const unsigned n = (unsigned)MB;
+  grid_trigger();
+  grid_wait();
   auto beta2 = [&](unsigned b) {  // columns b, b + 1 (b even)
     uint32_t w[NM];
 #pragma unroll
@@ -832,7 +860,7 @@ __global__ void __launch_bounds__(256, 3) rns_beta_kernel(const uint16_t* __rest
     return r;
   };
   unsigned m = 0;
-  for (unsigned b = 2 * tid; b < n; b += 512) {
+  for (unsigned b = 2 * tid; b < n; b += 2 * blockDim.x) {
     const df2 r = beta2(b);
     if (STAGE) sb[b >> 1] = as_f4(r);
     m = max(m, max(abs_bits(r.h.x), abs_bits(r.h.y)));
@@ -842,7 +870,7 @@ __global__ void __launch_bounds__(256, 3) rns_beta_kernel(const uint16_t* __rest
   if (tid == 0) sc[a] = s;
   bf16* da = d + a * Kp;
   const int64_t dplane = M * Kp;
-  for (unsigned b = 4 * tid; b < n; b += 1024) {
+  for (unsigned b = 4 * tid; b < n; b += 4 * blockDim.x) {
     const df2 zero{f2(0.f), f2(0.f)};
     float2 dx[4], dy[4];
     digits2(p_scale(STAGE ? as_df2(sb[b >> 1]) : beta2(b), s, s), dx);
@@ -862,7 +890,7 @@ __global__ void __launch_bounds__(256, 3) rns_beta_kernel(const uint16_t* __rest
 // with respect to its first atom i > j carries the minus sign).  CTA 0 clears the column maxima for
 // the next matvec.
 template <int NM>
-__global__ void __launch_bounds__(256, 3) rns_backproj_kernel(const uint16_t* __restrict__ Up, int slabs, int chunks,
+__global__ void __launch_bounds__(256, 4) rns_backproj_kernel(const uint16_t* __restrict__ Up, int slabs, int chunks,
                                                               int64_t M, int D, int Dp, int64_t ldU,
                                                               const int* __restrict__ sA, const int* __restrict__ sWT,
                                                               const int* __restrict__ sB, const int* __restrict__ sXT,
@@ -876,14 +904,15 @@ __global__ void __launch_bounds__(256, 3) rns_backproj_kernel(const uint16_t* __
   const int64_t a = blockIdx.x;
   const int tid = threadIdx.x, H = Dp >> 1;
   constexpr rns::Crt<NM> C{};
+  grid_wait();
   const int ea = C.pexp - 43 - sA[a], eb = C.pexp - 43 - sB[a];
   if (a == 0)
-    for (int p = tid; p < Dp; p += 256) colmax[p] = 0u;
+    for (int p = tid; p < kColCopies * Dp; p += blockDim.x) colmax[p] = 0u;
   const int64_t plane = M * ldU;
   const uint16_t* Ua = Up + a * ldU;
   const float4* Ga = G3 + a * 3 * H;
   const df2 pm{f2(C.pih), f2(C.pil)};
-  for (unsigned p = 2 * tid; p <= (unsigned)D; p += 512) {
+  for (unsigned p = 2 * tid; p <= (unsigned)D; p += 2 * blockDim.x) {
     uint32_t w[2][NM];
 #pragma unroll
     for (int sg = 0; sg < 2; ++sg)
@@ -911,7 +940,7 @@ __global__ void __launch_bounds__(256, 3) rns_backproj_kernel(const uint16_t* __
     }
   }
   __syncthreads();
-  const int sub = tid & (lanes - 1), per = 256 / lanes;
+  const int sub = tid & (lanes - 1), per = (int)blockDim.x / lanes;
   const float2* w3 = reinterpret_cast<const float2*>(w4);
   for (int i0 = 0; i0 < N; i0 += per) {  // every lane group runs the same trip count
     const int i = i0 + tid / lanes;
@@ -1021,7 +1050,7 @@ static void gemm_shape(int64_t M, int64_t N, int64_t nkb, int64_t planes, int ca
 
 // residues of A B^T (or of both segments' products) into out
 template <bool BUILD>
-static gdml_status launch_gemm(GemmArgs& g, int segs, int chunks, cudaStream_t st) {
+static gdml_status launch_gemm(GemmArgs& g, int segs, int chunks, bool pdl, cudaStream_t st) {
   static bool attr_set = false;
   if (!attr_set) {
     if (cudaFuncSetAttribute(rns_gemm_kernel<BUILD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
@@ -1051,14 +1080,14 @@ static gdml_status launch_gemm(GemmArgs& g, int segs, int chunks, cudaStream_t s
   if (units > INT32_MAX / 2) return fail(GDML_ERR_ARG, "residue gemm: too many tiles");
   g.units = (int)units;
   const unsigned grid = 2u * (unsigned)std::min<int64_t>(units, std::max(num_sms() / 2, 1));
-  { rns_gemm_kernel<BUILD><<<grid, kThreads, kSmem, st>>>(g); count_launch(); }
+  { launch_after(pdl, rns_gemm_kernel<BUILD>, grid, kThreads, kSmem, st, g); count_launch(); }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(GDML_ERR_CUDA, std::string("residue gemm launch: ") + cudaGetErrorString(e));
   return GDML_OK;
 }
 
 static gdml_status rns_gemm(const RnsOperand* A, const RnsOperand* B, int segs, int bn, int chunks,
-                            uint16_t* out, int64_t ldo, int* err, cudaStream_t st, int* slabs_out) {
+                            uint16_t* out, int64_t ldo, int* err, bool pdl, cudaStream_t st, int* slabs_out) {
   GemmArgs g{};
   for (int s = 0; s < 2; ++s) {
     g.a[s] = A[s < segs ? s : 0].map;
@@ -1071,7 +1100,7 @@ static gdml_status rns_gemm(const RnsOperand* A, const RnsOperand* B, int segs, 
   g.ldo = ldo;
   g.out = out;
   g.err = err;
-  RNS_TRY(launch_gemm<false>(g, segs, chunks, st));
+  RNS_TRY(launch_gemm<false>(g, segs, chunks, pdl, st));
   if (slabs_out) *slabs_out = g.groups;
   return GDML_OK;
 }
@@ -1095,7 +1124,7 @@ gdml_status rns_product(RnsProduct& q, int* err, cudaStream_t st) {
   g.err = err;
   g.shape = q.shape;
   g.row0 = (int)q.row0;
-  return launch_gemm<true>(g, 1, q.chunks, st);
+  return launch_gemm<true>(g, 1, q.chunks, false, st);
 }
 
 void rns_product_shape(RnsProduct& q, int cap) {
@@ -1155,7 +1184,7 @@ gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, co
   RNS_TRY(rns_alloc(r, &r.G3, (size_t)(3 * M * r.Dp), st));
   RNS_TRY(rns_alloc(r, &r.Xc2, (size_t)(M * r.Dp), st));
   RNS_TRY(rns_alloc(r, &r.ij, (size_t)r.Dp, st));
-  RNS_TRY(rns_alloc(r, &r.colmax, (size_t)r.Dp, st));
+  RNS_TRY(rns_alloc(r, &r.colmax, (size_t)(kColCopies * r.Dp), st));
   RNS_TRY(rns_alloc(r, &r.t2, (size_t)r.ldT, st));
   RNS_TRY(rns_alloc(r, &r.S2, (size_t)(M * r.ldT), st));
   RNS_TRY(rns_alloc(r, &r.Tp, (size_t)(r.cap1 * NM * M * r.ldT), st));
@@ -1193,6 +1222,30 @@ gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, co
   return GDML_OK;
 }
 
+// Threads per row of the beta and back-projection kernels (64 registers, `smem` bytes a row): 128 where a
+// row has no work for more, or where that makes all M rows resident at once and 256 do not; else 256.
+// Back-projection of M = 1,000 rows, D = 210: 13.3 us, 20.3 with 256 threads in three CTAs per SM; beta of
+// 1,000 columns 18.9 and 20.2; of 6,000 columns (48 KB a row, so four CTAs either way) 128 threads took 16 us longer.
+static int row_threads(int64_t M, int64_t pairs, size_t smem) {
+  const int64_t sms = num_sms(), fit = std::min<int64_t>(8, (int64_t)(227 * 1024 / (smem + 2048)));
+  if (pairs <= 128) return 128;
+  return M > std::min<int64_t>(4, fit) * sms && M <= fit * sms ? 128 : 256;
+}
+
+// Whether the matvec's kernels may start while the one before them drains (each waits for it before it
+// reads): about 1.5 us of launch and start-up per kernel.  Outside capture only, and where a kernel's rows
+// are resident at once: M = 200, D = 36 28.3 us, 38.6 without; M = 1,000, D = 210 92.9 and 98.9; but M = 5,000,
+// D = 861 1,660 and 1,588, and a captured solve at M = 1,000 8.96 and 8.85 ms.
+static bool chained(int64_t M, cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (M > 8 * (int64_t)num_sms()) return false;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
+}
+
 gdml_status rns_matvec(RnsMatvec& r, const double* G, const double* Xc, const double* v, double* out, int add_lambda,
                        double lam, cudaStream_t st) {
   constexpr int NM = rns::kMvMods;
@@ -1200,36 +1253,39 @@ gdml_status rns_matvec(RnsMatvec& r, const double* G, const double* Xc, const do
   if (!r.ready) return fail(GDML_ERR_STATE, "residue matvec not set up");
   const int64_t M = r.M, MB = r.MB;
   const int D = r.D;
+  const bool pdl = chained(M, st);
   const float rootD = std::sqrt((float)D) * 1.0001f, rootMB = std::sqrt((float)MB) * 1.0001f;
   const dim3 gc((unsigned)cdiv(MB, 32), (unsigned)cdiv(D, 32));
   if (r.S > 1) {  // w_b = J_b v_b, then row b S + q = P_q w_b with t = xc_(bS+q) . w_(bS+q)
     launch_proj(G, Xc, v, M, r.N, D, r.W, D, r.t, st);
     launch_sym_gather(r.W, M, D, r.pis, r.S, r.XcB, r.WB, r.t, st);
     { rns_rows_kernel<NM><<<(unsigned)MB, 256, 0, st>>>(r.WB, MB, D, r.W1.Kp, bits, r.W1.d, r.W1.s, r.colmax, r.t, r.t2); count_launch(); }
-    { rns_cols_kernel<NM, double><<<gc, 256, 0, st>>>(r.WB, MB, D, D, r.colmax, r.WT2.Kp, D + 1, bits, r.WT2.d, r.WT2.s); count_launch(); }
+    { launch_after(pdl, rns_cols_kernel<NM, double>, gc, 256, 0, st, r.WB, MB, D, D, r.colmax, r.WT2.Kp, D + 1, bits, r.WT2.d, r.WT2.s); count_launch(); }
   } else {
     const size_t sm = (size_t)(3 * r.N + r.Dp) * sizeof(float2);
     RNS_TRY(big_smem(rns_proj_kernel<NM>, sm));
     const int nt = (int)std::min<int64_t>(512, std::max<int64_t>(64, cdiv(cdiv(D, 2), 32) * 32));
     { rns_proj_kernel<NM><<<(unsigned)M, nt, sm, st>>>((const float4*)r.G3, (const float4*)r.Xc2, (const uint2*)r.ij, v, M, r.N, r.Dp, rootD, (float4*)r.Wf, r.t2, r.W1.Kp, bits, r.W1.d, r.W1.s, r.colmax); count_launch(); }
-    { rns_cols_kernel<NM, float2><<<gc, 256, 0, st>>>(r.Wf, MB, D, r.Dp, r.colmax, r.WT2.Kp, D + 1, bits, r.WT2.d, r.WT2.s); count_launch(); }
+    { launch_after(pdl, rns_cols_kernel<NM, float2>, gc, 256, 0, st, r.Wf, MB, D, r.Dp, r.colmax, r.WT2.Kp, D + 1, bits, r.WT2.d, r.WT2.s); count_launch(); }
   }
   int s1 = 0, s2 = 0;
-  RNS_TRY(rns_gemm(&r.Xc1, &r.W1, 1, r.bn1, rns_chunks(r.nch1, r.g1, r.cap1), r.Tp, r.ldT, r.err, st, &s1));
+  RNS_TRY(rns_gemm(&r.Xc1, &r.W1, 1, r.bn1, rns_chunks(r.nch1, r.g1, r.cap1), r.Tp, r.ldT, r.err, pdl, st, &s1));
+  const int nr = row_threads(M, cdiv(MB, 2), MB <= kBetaStage ? (size_t)r.ldT * sizeof(float2) : 0);
   if (MB <= kBetaStage) {
     const size_t sm = (size_t)r.ldT * sizeof(float2);
     RNS_TRY(big_smem(rns_beta_kernel<NM, true>, sm));
-    { rns_beta_kernel<NM, true><<<(unsigned)M, 256, sm, st>>>(r.Tp, s1, (int)r.nch1, M, MB, r.ldT, r.Xc1.s, r.W1.s, r.S2, r.t2, rootMB, r.B2.Kp, bits, r.B2.d, r.B2.s); count_launch(); }
+    { launch_after(pdl, rns_beta_kernel<NM, true>, (unsigned)M, nr, sm, st, r.Tp, s1, (int)r.nch1, M, MB, r.ldT, r.Xc1.s, r.W1.s, r.S2, r.t2, rootMB, r.B2.Kp, bits, r.B2.d, r.B2.s); count_launch(); }
   } else {
-    { rns_beta_kernel<NM, false><<<(unsigned)M, 256, 0, st>>>(r.Tp, s1, (int)r.nch1, M, MB, r.ldT, r.Xc1.s, r.W1.s, r.S2, r.t2, rootMB, r.B2.Kp, bits, r.B2.d, r.B2.s); count_launch(); }
+    { launch_after(pdl, rns_beta_kernel<NM, false>, (unsigned)M, nr, 0, st, r.Tp, s1, (int)r.nch1, M, MB, r.ldT, r.Xc1.s, r.W1.s, r.S2, r.t2, rootMB, r.B2.Kp, bits, r.B2.d, r.B2.s); count_launch(); }
   }
   const RnsOperand a[2] = {r.A2, r.B2}, b[2] = {r.WT2, r.XT2};
-  RNS_TRY(rns_gemm(a, b, 2, r.bn2, rns_chunks(r.nch2, r.g2, r.cap2), r.Up, r.ldU, r.err, st, &s2));
-  int lanes = 4;  // per atom in the last step: as many as 256 threads give, up to 16
-  while (lanes < 16 && 2 * lanes * r.N <= 256) lanes *= 2;
+  RNS_TRY(rns_gemm(a, b, 2, r.bn2, rns_chunks(r.nch2, r.g2, r.cap2), r.Up, r.ldU, r.err, pdl, st, &s2));
   const size_t sm = 3 * (size_t)r.Dp * sizeof(float2);
+  const int nb = row_threads(M, cdiv(D + 1, 2), sm);
+  int lanes = 4;  // per atom in the last step: as many as the threads give, up to 16
+  while (lanes < 16 && 2 * lanes * r.N <= nb) lanes *= 2;
   RNS_TRY(big_smem(rns_backproj_kernel<NM>, sm));
-  { rns_backproj_kernel<NM><<<(unsigned)M, 256, sm, st>>>(r.Up, s2, (int)r.nch2, M, D, r.Dp, r.ldU, r.A2.s, r.WT2.s, r.B2.s, r.XT2.s, r.JX, (const float4*)r.G3, v, r.N, lam, add_lambda, lanes, r.colmax, out); count_launch(); }
+  { launch_after(pdl, rns_backproj_kernel<NM>, (unsigned)M, nb, sm, st, r.Up, s2, (int)r.nch2, M, D, r.Dp, r.ldU, r.A2.s, r.WT2.s, r.B2.s, r.XT2.s, r.JX, (const float4*)r.G3, v, r.N, lam, add_lambda, lanes, r.colmax, out); count_launch(); }
   if (cudaGetLastError() != cudaSuccess) return fail(GDML_ERR_CUDA, "residue matvec kernels");
   return GDML_OK;
 }

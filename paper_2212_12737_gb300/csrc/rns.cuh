@@ -157,7 +157,7 @@ struct RnsMatvec {
   float2* G3 = nullptr;     // [M][3][Dp] Jacobian factors
   uint32_t* ij = nullptr;   // Dp: 3 i | 3 j << 16 of pair p
   float2* Wf = nullptr;     // [M][Dp] the projection (S = 1)
-  unsigned* colmax = nullptr;  // D: largest |W| of each descriptor (float bits), zero between matvecs
+  unsigned* colmax = nullptr;  // copies x Dp: largest |W| of each descriptor (float bits), zero between matvecs
   float2* Xc2 = nullptr;    // [M][Dp] the centred descriptors
   float2* t2 = nullptr;     // t_b = xc_b . w_b over the mantissa of P
   float2* S2 = nullptr;     // M x ldT: c^2 S_ab times the mantissa of P

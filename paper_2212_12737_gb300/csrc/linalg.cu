@@ -14,102 +14,142 @@ namespace gdml {
 // Two levels of blocking: steps of NB = 32 columns factorise a block of NO = 128, whose update of the
 // rest is one product.  An SM's FP64 pipe does under two multiply-adds per cycle, so the work of the
 // serial kernels (the diagonal block on one SM, ~NB^3 / 3; a panel's rows at NB^2 / 2 each) decides:
-// with steps of 64 the diagonal block took 105 us and a panel 150-190 us.  A warp of 32 rows per CTA
-// spreads a panel over all SMs.  Two factorisations and two triangular inverses at k = 1500: 62 ms
-// with one level of 64, 31 ms so.
+// with steps of 64 the diagonal block took 105 us and a panel 150-190 us.  32 rows per CTA
+// spread a panel over all SMs.  Two factorisations and two triangular inverses at k = 1500: 62 ms
+// with one level of 64, 21 ms so.
 constexpr int NB = 32;
 constexpr int NO = 128;
 
-// Unblocked Cholesky of the nb x nb diagonal block at (j0, j0), in place (lower): one warp, lane r
-// holds row r.
-__global__ void __launch_bounds__(32) potrf_diag_kernel(double* __restrict__ A, int64_t lda, int64_t j0, int nb,
-                                                        int* __restrict__ status) {
+// A warp's FP64 operation takes 64 cycles on its quarter of an SM, so all three kernels below use four
+// warps per 32 rows: one warp each took 53, 31 and 24 us (23, 16 and 19 us so).
+constexpr int kGroup = 4;  // lanes (potrf: warps) that share a row: every fourth column each
+constexpr int kOwn = NB / kGroup;
+
+// Unblocked Cholesky of the nb x nb diagonal block at (j0, j0), in place (lower): lane r of every warp
+// holds row r, warp w its columns w, w + 4, ...; the column of each step goes through shared memory.
+__global__ void __launch_bounds__(32 * kGroup) potrf_diag_kernel(double* __restrict__ A, int64_t lda, int64_t j0,
+                                                                 int nb, int* __restrict__ status) {
+  __shared__ double colv[2][NB];
+  __shared__ int s_bad;
   if (*status) return;
-  const int r = threadIdx.x;
+  const int r = threadIdx.x & 31, w = threadIdx.x >> 5;
   double* row = A + (j0 + r) * lda + j0;
-  double a[NB];
+  double a[kOwn];
 #pragma unroll
-  for (int c = 0; c < NB; ++c) a[c] = (r < nb && c <= r) ? row[c] : (c == r ? 1.0 : 0.0);
-  int bad = 0;
+  for (int q = 0; q < kOwn; ++q) {
+    const int c = kGroup * q + w;
+    a[q] = (r < nb && c <= r) ? row[c] : (c == r ? 1.0 : 0.0);
+  }
+  if (threadIdx.x == 0) s_bad = 0;
+  __syncthreads();
 #pragma unroll
   for (int c = 0; c < NB; ++c) {
-    const double d = __shfl_sync(0xffffffffu, a[c], c);
-    if (!(d > 0.0) || !isfinite(d)) {  // (warp-uniform)
-      bad = c + 1;
-      break;
+    double* v = colv[c & 1];
+    if (w == c % kGroup) {
+      const double d = __shfl_sync(0xffffffffu, a[c / kGroup], c);
+      const bool ok = d > 0.0 && isfinite(d);
+      if (!ok && r == 0) s_bad = c + 1;
+      // 1 / l and l = d / l by a correction of each other (one square root, no division)
+      const double inv = rsqrt(ok ? d : 1.0), l0 = d * inv;
+      const double l = fma(fma(-l0, l0, d), 0.5 * inv, l0);
+      a[c / kGroup] = r == c ? l : a[c / kGroup] * inv;
+      v[r] = a[c / kGroup];
     }
-    const double l = sqrt(d), inv = 1.0 / l;
-    a[c] = r == c ? l : a[c] * inv;
+    __syncthreads();
+    if (s_bad) break;
+    const double x = v[r];
 #pragma unroll
-    for (int cc = c + 1; cc < NB; ++cc) a[cc] = fma(-a[c], __shfl_sync(0xffffffffu, a[c], cc), a[cc]);
+    for (int q = c / kGroup; q < kOwn; ++q) {
+      const int cc = kGroup * q + w;
+      if (cc > c) a[q] = fma(-x, v[cc], a[q]);
+    }
   }
-  if (bad) {
-    if (r == 0) *status = (int)(j0 + bad);
+  if (s_bad) {
+    if (threadIdx.x == 0) *status = (int)(j0 + s_bad);
     return;
   }
   if (r < nb)
 #pragma unroll
-    for (int c = 0; c < NB; ++c)
-      if (c < nb) row[c] = c <= r ? a[c] : 0.0;
+    for (int q = 0; q < kOwn; ++q) {
+      const int c = kGroup * q + w;
+      if (c < nb) row[c] = c <= r ? a[q] : 0.0;
+    }
 }
 
-// Rows r in [r0, rend): solve x L_jj^T = A[r, j0:j0+nb]  (one thread per row, one warp per CTA).
-__global__ void __launch_bounds__(32) trsm_right_kernel(double* __restrict__ A, int64_t lda, int64_t j0, int nb,
-                                                        int64_t r0, int64_t rend, const int* __restrict__ status) {
-  __shared__ double L[NB][NB + 1];
-  __shared__ double rows[NB][NB + 1];
-  if (*status) return;
-  const int t = threadIdx.x;
-  const int64_t base = r0 + blockIdx.x * (int64_t)NB;
-  for (int r = 0; r < NB; ++r) {
-    const bool in = r < nb && t < nb;
-    L[r][t] = in ? A[(j0 + r) * lda + j0 + t] : (r == t ? 1.0 : 0.0);
-    rows[r][t] = base + r < rend && t < nb ? A[(base + r) * lda + j0 + t] : 0.0;
-  }
-  __syncwarp();
-  const double inv = 1.0 / L[t][t];
-  double x[NB];
-#pragma unroll
-  for (int c = 0; c < NB; ++c) x[c] = rows[t][c];
+// x <- x L^-T for the row x spread over four neighbouring lanes (lane g: entries g, g + 4, ...); inv: the
+// reciprocals of L's diagonal
+__device__ __forceinline__ void solve_row(double (&x)[kOwn], const double (&L)[NB][NB + 1], const double* inv) {
+  const int g = threadIdx.x & (kGroup - 1), first = (threadIdx.x & 31) & ~(kGroup - 1);
 #pragma unroll
   for (int c = 0; c < NB; ++c) {  // column by column: the updates of the later ones are independent
-    x[c] *= __shfl_sync(0xffffffffu, inv, c);
+    if (g == c % kGroup) x[c / kGroup] *= inv[c];
+    const double xc = __shfl_sync(0xffffffffu, x[c / kGroup], first + c % kGroup);
 #pragma unroll
-    for (int cc = c + 1; cc < NB; ++cc) x[cc] = fma(-x[c], L[cc][c], x[cc]);
+    for (int q = c / kGroup; q < kOwn; ++q) {
+      const int cc = kGroup * q + g;
+      if (cc > c) x[q] = fma(-xc, L[cc][c], x[q]);
+    }
   }
+}
+
+// Rows r in [r0, rend): solve x L_jj^T = A[r, j0:j0+nb]  (four lanes per row, 32 rows per CTA).
+__global__ void __launch_bounds__(32 * kGroup) trsm_right_kernel(double* __restrict__ A, int64_t lda, int64_t j0,
+                                                                 int nb, int64_t r0, int64_t rend,
+                                                                 const int* __restrict__ status) {
+  __shared__ double L[NB][NB + 1];
+  __shared__ double inv[NB];
+  if (*status) return;
+  const int t = threadIdx.x;
+  for (int r = t >> 5; r < NB; r += kGroup) {
+    const int c = t & 31;
+    const double l = r < nb && c < nb ? A[(j0 + r) * lda + j0 + c] : (r == c ? 1.0 : 0.0);
+    L[r][c] = l;
+    if (r == c) inv[r] = 1.0 / l;
+  }
+  const int64_t row = r0 + blockIdx.x * (int64_t)NB + t / kGroup;
+  const int g = t & (kGroup - 1);
+  double* a = A + row * lda + j0;
+  double x[kOwn];
 #pragma unroll
-  for (int c = 0; c < NB; ++c) rows[t][c] = x[c];
-  __syncwarp();
-  for (int r = 0; r < NB; ++r)
-    if (base + r < rend && t < nb) A[(base + r) * lda + j0 + t] = rows[r][t];
+  for (int q = 0; q < kOwn; ++q) x[q] = row < rend && kGroup * q + g < nb ? a[kGroup * q + g] : 0.0;
+  __syncthreads();
+  solve_row(x, L, inv);
+  if (row < rend)
+#pragma unroll
+    for (int q = 0; q < kOwn; ++q)
+      if (kGroup * q + g < nb) a[kGroup * q + g] = x[q];
 }
 
 // Left forward substitution on a block of rows of B (k x nrhs, row-major, ld):
-// B[j0:j0+nb, col] <- L_jj^-1 B[j0:j0+nb, col]; one thread per column, one warp per CTA.
-__global__ void __launch_bounds__(32) trsm_left_diag_kernel(const double* __restrict__ Lkk, int64_t ldl, int64_t j0,
-                                                            int nb, double* __restrict__ Bm, int64_t ldb,
-                                                            int64_t nrhs) {
+// B[j0:j0+nb, col] <- L_jj^-1 B[j0:j0+nb, col]; four lanes per column, 32 columns per CTA.
+__global__ void __launch_bounds__(32 * kGroup) trsm_left_diag_kernel(const double* __restrict__ Lkk, int64_t ldl,
+                                                                     int64_t j0, int nb, double* __restrict__ Bm,
+                                                                     int64_t ldb, int64_t nrhs) {
   __shared__ double L[NB][NB + 1];
+  __shared__ double B[NB][NB + 1];
+  __shared__ double inv[NB];
   const int t = threadIdx.x;
-  for (int r = 0; r < NB; ++r)
-    L[r][t] = r < nb && t < nb ? Lkk[(j0 + r) * ldl + j0 + t] : (r == t ? 1.0 : 0.0);
-  __syncwarp();
-  const double inv = 1.0 / L[t][t];
-  const int64_t col = blockIdx.x * (int64_t)NB + t;
-  const bool in = col < nrhs;
-  double x[NB];
-#pragma unroll
-  for (int r = 0; r < NB; ++r) x[r] = in && r < nb ? Bm[(j0 + r) * ldb + col] : 0.0;
-#pragma unroll
-  for (int r = 0; r < NB; ++r) {
-    x[r] *= __shfl_sync(0xffffffffu, inv, r);
-#pragma unroll
-    for (int rr = r + 1; rr < NB; ++rr) x[rr] = fma(-L[rr][r], x[r], x[rr]);
+  const int64_t c0 = blockIdx.x * (int64_t)NB;
+  for (int r = t >> 5; r < NB; r += kGroup) {
+    const int c = t & 31;
+    const double l = r < nb && c < nb ? Lkk[(j0 + r) * ldl + j0 + c] : (r == c ? 1.0 : 0.0);
+    L[r][c] = l;
+    if (r == c) inv[r] = 1.0 / l;
+    B[r][c] = r < nb && c0 + c < nrhs ? Bm[(j0 + r) * ldb + c0 + c] : 0.0;
   }
-  if (in)
+  __syncthreads();
+  const int g = t & (kGroup - 1), col = t / kGroup;
+  double x[kOwn];
 #pragma unroll
-    for (int r = 0; r < NB; ++r)
-      if (r < nb) Bm[(j0 + r) * ldb + col] = x[r];
+  for (int q = 0; q < kOwn; ++q) x[q] = B[kGroup * q + g][col];
+  solve_row(x, L, inv);
+#pragma unroll
+  for (int q = 0; q < kOwn; ++q) B[kGroup * q + g][col] = x[q];
+  __syncthreads();
+  for (int r = t >> 5; r < nb; r += kGroup) {
+    const int c = t & 31;
+    if (c0 + c < nrhs) Bm[(j0 + r) * ldb + c0 + c] = B[r][c];
+  }
 }
 
 __global__ void add_diag_kernel(double* A, int64_t lda, int64_t k, double eps) {
@@ -125,10 +165,10 @@ void cholesky_inplace(double* A, int64_t k, int* status, cudaStream_t st) {
     const int64_t o1 = std::min<int64_t>(k, o0 + NO);
     for (int64_t j0 = o0; j0 < o1; j0 += NB) {
       const int nb = (int)std::min<int64_t>(NB, o1 - j0);
-      { potrf_diag_kernel<<<1, 32, 0, st>>>(A, k, j0, nb, status); count_launch(); }
+      { potrf_diag_kernel<<<1, 32 * kGroup, 0, st>>>(A, k, j0, nb, status); count_launch(); }
       const int64_t r0 = j0 + nb;
       if (r0 >= k) break;
-      { trsm_right_kernel<<<(unsigned)cdiv(k - r0, NB), NB, 0, st>>>(A, k, j0, nb, r0, k, status); count_launch(); }
+      { trsm_right_kernel<<<(unsigned)cdiv(k - r0, NB), 32 * kGroup, 0, st>>>(A, k, j0, nb, r0, k, status); count_launch(); }
       // the block's remaining columns: A[r0:, r0:o1] -= L[r0:, j0:r0] L[r0:o1, j0:r0]^T
       if (r0 < o1)
         launch_dgemm<double, double>(true, k - r0, o1 - r0, nb, -1.0, A + r0 * k + j0, k, A + r0 * k + j0, k, 1.0,
@@ -157,7 +197,7 @@ void trsm_left_lower(const double* Lkk, int64_t k, double* Bm, int64_t nrhs, cud
     for (int64_t j0 = o0; j0 < o1; j0 += NB) {
       const int nb = (int)std::min<int64_t>(NB, o1 - j0);
       const int64_t ncols = cols(j0 + nb);
-      { trsm_left_diag_kernel<<<(unsigned)cdiv(ncols, NB), NB, 0, st>>>(Lkk, k, j0, nb, Bm, nrhs, ncols); count_launch(); }
+      { trsm_left_diag_kernel<<<(unsigned)cdiv(ncols, NB), 32 * kGroup, 0, st>>>(Lkk, k, j0, nb, Bm, nrhs, ncols); count_launch(); }
       if (j0 + nb < o1) update(j0 + nb, o1, j0, j0 + nb);
     }
     if (o1 < k) update(o1, k, o0, o1);

@@ -47,7 +47,7 @@ def parse():
                     help="system on which every form is solved to the end (FP64 takes minutes at n = 630,000)")
     ap.add_argument("--precision", default="ozaki", choices=["fp64", "tf32", "bf16", "df64", "ozaki"],
                     help="headline form (df64: double-float contractions on the FP32 lanes; ozaki: exact "
-                         "BF16 slices on the tensor cores; both FP64-class, FP64 true-residual restarts)")
+                         "BF16 residues on the tensor cores; both FP64-class, FP64 true-residual restarts)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-forms", action="store_true", help="skip the per-precision comparison solves")
     ap.add_argument("--only", default="solve", choices=["solve", "matvec", "apply", "passes", "build"],
@@ -66,9 +66,9 @@ def parse():
     return ap.parse_args()
 
 
-# tensor-core products per FP64-equivalent product: the sliced form multiplies
-# 28 BF16 slice pairs (7 slices per operand, pairs i + j <= 8) for each one
-SLICE_PAIRS = {"fp64": 1, "df64": 1, "tf32": 1, "bf16": 1, "ozaki": 28}
+# tensor-core products per FP64-equivalent product: the OZAKI form multiplies residues
+# modulo 14 numbers for each one
+TC_PRODUCTS = {"fp64": 1, "df64": 1, "tf32": 1, "bf16": 1, "ozaki": 14}
 
 
 # ----------------------------------------------------------------- helpers
@@ -557,19 +557,19 @@ def run_gpu(args):
     elif args.precision == "tf32":
         peak, peak_src, bound = torch_peak(torch.float32, tf32=True, size=8192), \
             "of measured (torch TF32 matmul 8192^3, this run)", "tensor"
-    else:  # ozaki (28 BF16 slice-pair products per contraction on tcgen05) and bf16
+    else:  # ozaki (14 BF16 residue products per contraction on tcgen05) and bf16
         peak = peaks.get("bf16_tflops", 1900.0)
         peak_src, bound = ("of measured (MEASURED_PEAKS.json bf16_tflops, burst: the matvec is timed alone)"
                            if peaks else "of fallback"), "tensor"
 
-    mv_flop = 6.0 * M * M * D * SLICE_PAIRS[args.precision]
+    mv_flop = 6.0 * M * M * D * TC_PRODUCTS[args.precision]
     roof_matvec = {"kernel": f"force-kernel matvec, {args.precision}: one launch unit = projection + "
-                             f"{'sliced ' if args.precision == 'ozaki' else ''}contractions + beta + back-projection",
+                             f"{'residue ' if args.precision == 'ozaki' else ''}contractions + beta + back-projection",
                    "bound": bound, "achieved": mv_flop / mv_sec / 1e12, "peak": peak, "unit": "TFLOP/s",
                    "frac": mv_flop / mv_sec / 1e12 / peak, "peak_source": peak_src,
                    "traffic": NCU_TRAFFIC.get((args.workload, args.precision, "matvec")),
                    "algorithmic_flop_per_launch": mv_flop,
-                   "algorithmic_flop_note": ("28 BF16 slice-pair products x 6 M^2 D" if args.precision == "ozaki"
+                   "algorithmic_flop_note": ("14 BF16 residue products x 6 M^2 D" if args.precision == "ozaki"
                                              else "6 M^2 D"),
                    "fp64_equivalent_tflops": 6.0 * M * M * D / mv_sec / 1e12, "ms": mv_sec * 1e3}
     hbm = peaks.get("hbm_gbs", 6800.0)
@@ -595,7 +595,7 @@ def run_gpu(args):
             sec = op_rate(c2, lambda: c2.matvec(v, out), reps=5 if prec in ("fp64", "df64") else 20)
             c2.destroy()
             forms[prec] = {"matvec_ms": sec * 1e3, "matvec_tflops_fp64_equivalent": 6.0 * M * M * D / sec / 1e12,
-                           "matvec_tflops_executed": 6.0 * M * M * D * SLICE_PAIRS[prec] / sec / 1e12}
+                           "matvec_tflops_executed": 6.0 * M * M * D * TC_PRODUCTS[prec] / sec / 1e12}
         # whole solves of every form on the 63,000-unknown system (minutes in FP64 at n = 630,000)
         w2 = synth.workload(args.forms_workload)
         R2, y2 = torch.from_numpy(w2.R).to(dev), torch.from_numpy(w2.y).to(dev)
@@ -631,7 +631,7 @@ def run_gpu(args):
             "warmup": args.warmup, "ms_per_step": t_dev * 1e3, "higher_is_better": False, "scaling": "weak",
             "vs_baseline": None,
             "dtype": {"fp64": "f64", "df64": "f32x2 (double-float) contractions + f64",
-                      "ozaki": "bf16 x7 exact slices (FP32 accumulate) + f32x2 + f64", "tf32": "tf32 + f64",
+                      "ozaki": "bf16 residues mod 14 numbers (exact FP32 sums) + f32x2 + f64", "tf32": "tf32 + f64",
                       "bf16": "bf16 + f64"}[args.precision], "data": "synthetic",
             "config": {"workload": f"{args.workload}: N={N} atoms, M={M} geometries, n={n}, D={D}, "
                                    f"{w.select} k={k}, sigma={w.sigma}, lambda={w.lam}, rtol={RTOL}",

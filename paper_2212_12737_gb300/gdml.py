@@ -393,7 +393,7 @@ def test_oz_gemm(A: torch.Tensor, B: torch.Tensor, chunks_per_cta: int = 0, leve
 
 
 def test_oz_gemm_tall(A: torch.Tensor, B: torch.Tensor, tri_b: bool = False, rowsq: bool = False):
-    """The OZAKI build's tall sliced GEMM: C = A B^T with A (n x K) and B (NB x K) FP64 (B lower
+    """The OZAKI build's tall residue GEMM: C = A B^T with A (n x K) and B (NB x K) FP64 (B lower
     triangular when tri_b).  Returns C (n x NB) and its FP32 copy, or the row square sums of C
     (n,) when rowsq."""
     lib = load()

@@ -86,6 +86,15 @@ __device__ __forceinline__ void pair_of(int p, int& i, int& j) {
 // completed, grid_trigger lets the next one start (when every CTA has called it or has ended)
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// whether launches into the stream are not being captured (early starts gained nothing in captured loops)
+inline bool not_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
+}
 // launches a kernel that with `early` may start before the one ahead of it in the stream has ended (it
 // calls grid_wait)
 template <typename... P, typename... A>

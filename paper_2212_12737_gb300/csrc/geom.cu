@@ -460,9 +460,9 @@ __global__ void __launch_bounds__(256) kcol_df_kernel(const int64_t* __restrict_
     }
   }
   grid_wait();
-  if (stop_flag && *stop_flag) return;
+  if (stop_flag && __ldcg(stop_flag)) return;
   grid_trigger();  // (after the wait: the next kernel may rely on what came before this one)
-  const int64_t col = cols[c];
+  const int64_t col = __ldcg(cols + c);
   const int64_t b = col / B;
   const int l = (int)(col - b * B), i = l / 3, q = l - 3 * i;
   const float2* Xb = X2 + b * D;

@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(256) rns_cols_kernel(const T* __restrict__ W, 
   unsigned m = 0;
   if (d0 + c < D)
 #pragma unroll
-    for (int i = 0; i < kColCopies / 8; ++i) m = max(m, colmax[((threadIdx.x & 7) + 8 * i) * ((D + 1) & ~1) + d0 + c]);
+    for (int i = 0; i < kColCopies / 8; ++i) m = max(m, __ldcg(colmax + ((threadIdx.x & 7) + 8 * i) * ((D + 1) & ~1) + d0 + c));
 #pragma unroll
   for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   const int s = row_scale(m, sqrtf((float)MB) * 1.0001f, bits);
@@ -1237,13 +1237,7 @@ static int row_threads(int64_t M, int64_t pairs, size_t smem) {
 // are resident at once: M = 200, D = 36 28.3 us, 38.6 without; M = 1,000, D = 210 92.9 and 98.9; but M = 5,000,
 // D = 861 1,660 and 1,588, and a captured solve at M = 1,000 8.96 and 8.85 ms.
 static bool chained(int64_t M, cudaStream_t st) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (M > 8 * (int64_t)num_sms()) return false;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return false;
-  }
-  return cap == cudaStreamCaptureStatusNone;
+  return M <= 8 * (int64_t)num_sms() && not_capturing(st);
 }
 
 gdml_status rns_matvec(RnsMatvec& r, const double* G, const double* Xc, const double* v, double* out, int add_lambda,

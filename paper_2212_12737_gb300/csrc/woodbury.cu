@@ -1104,7 +1104,7 @@ void woodbury_apply_df(const float* L, int64_t n, int64_t k, const double* C, co
   }
   // Outside capture the launches of this path may start while the one before them drains: each waits for it
   // before it reads anything but L and the k x k matrices, and lets the next one start only then, so that at
-  // most two are under way; vectors that a launch of the chain rewrites are read past L1.  Seven launches of
+  // most two are under way; vectors that a launch of the chain rewrites are read past L1.  Eight launches of
   // 3 to 11 us: n = 34,965, k = 77 45.1 -> 32.4 us.
   df_pass_t(L, n, k, rs, part, t, t2, plan, err, st);
   // u = C^-1 t, refined once with the residual t - C u (see woodbury_apply)

@@ -136,37 +136,52 @@ __device__ __forceinline__ void digits2(df2 x, float2 (&d)[4]) {
   d[0] = p_add(p_add(p_add(x.h, x.l), f2(kMagic)), f2(-kMagic));
 }
 
-// The fraction (x . y) / P of two neighbouring outputs, in units of 2^-43, from NM words of two
-// 16-bit sums (each over `chunks` chunks of residue + 256).
-template <int NM>
-__device__ __forceinline__ df2 crt_fraction(const rns::Crt<NM>& C, const uint32_t (&w)[NM], uint32_t chunks) {
-  uint64_t a1[2] = {0, 0};
-  uint32_t a2[2] = {0, 0}, a0[2] = {0, 0};
+// The fraction (x . y) / P of two neighbouring outputs, in units of 2^-43, from words of two 16-bit
+// sums (each over at most rns::kSumChunks chunks of residue + 256, so that neither field carries into
+// the other); several groups of chunks are added here, in wider sums.
+struct CrtSum {
+  uint64_t a1[2] = {0, 0}, a0[2] = {0, 0};
+  uint32_t a2[2] = {0, 0};
+  template <int NM>
+  __device__ __forceinline__ void add(const rns::Crt<NM>& C, const uint32_t (&w)[NM]) {
+    uint32_t s0[2] = {0, 0};  // (14 fields times 12 bits stay below 2^32)
 #pragma unroll
-  for (int i = 0; i < NM; ++i) {
-    const uint32_t u[2] = {w[i] & 0xffffu, w[i] >> 16};
+    for (int i = 0; i < NM; ++i) {
+      const uint32_t u[2] = {w[i] & 0xffffu, w[i] >> 16};
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        s0[v] += u[v] * C.w0[i];
+        a1[v] += (uint64_t)u[v] * C.w1[i];
+        a2[v] += u[v] * C.w2[i];
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 2; ++v) a0[v] += s0[v];
+  }
+  template <int NM>
+  __device__ __forceinline__ df2 fraction(const rns::Crt<NM>& C, uint32_t chunks) const {
+    // minus the offset of 256 per residue and chunk
+    const uint64_t off = ((uint64_t)(chunks * C.o2) << 32) + (uint64_t)chunks * C.o1;
+    float g2[2], g1[2], g0[2];
 #pragma unroll
     for (int v = 0; v < 2; ++v) {
-      a0[v] += u[v] * C.w0[i];
-      a1[v] += (uint64_t)u[v] * C.w1[i];
-      a2[v] += u[v] * C.w2[i];
+      const int64_t f = (int64_t)((((uint64_t)a2[v] << 32) + a1[v]) - off) + (((int64_t)a0[v] - (int64_t)(chunks * C.o0)) >> 12);
+      // three digits of 21, 22 and 21 bits, each exact in FP32
+      g2[v] = __int_as_float(0x4b400000 + (int)(f >> 43));
+      g1[v] = __uint_as_float(0x4b000000u | ((uint32_t)(f >> 21) & 0x3fffffu));
+      g0[v] = __uint_as_float(0x4b000000u | ((uint32_t)f & 0x1fffffu));
     }
+    const float2 h2 = p_add(make_float2(g2[0], g2[1]), f2(-kMagic)), h1 = p_add(make_float2(g1[0], g1[1]), f2(-8388608.f)),
+                 h0 = p_add(make_float2(g0[0], g0[1]), f2(-8388608.f));
+    df2 r = p_fast_two_sum(p_mul(h2, f2(4194304.f)), h1);  // units of 2^21 2^-64
+    return p_fast_two_sum(r.h, p_fma(h0, f2(4.76837158203125e-7f), r.l));
   }
-  // minus the offset of 256 per residue and chunk
-  const uint64_t off = ((uint64_t)(chunks * C.o2) << 32) + (uint64_t)chunks * C.o1;
-  float g2[2], g1[2], g0[2];
-#pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    const int64_t f = (int64_t)((((uint64_t)a2[v] << 32) + a1[v]) - off) + (((int64_t)a0[v] - (int64_t)(chunks * C.o0)) >> 12);
-    // three digits of 21, 22 and 21 bits, each exact in FP32
-    g2[v] = __int_as_float(0x4b400000 + (int)(f >> 43));
-    g1[v] = __uint_as_float(0x4b000000u | ((uint32_t)(f >> 21) & 0x3fffffu));
-    g0[v] = __uint_as_float(0x4b000000u | ((uint32_t)f & 0x1fffffu));
-  }
-  const float2 h2 = p_add(make_float2(g2[0], g2[1]), f2(-kMagic)), h1 = p_add(make_float2(g1[0], g1[1]), f2(-8388608.f)),
-               h0 = p_add(make_float2(g0[0], g0[1]), f2(-8388608.f));
-  df2 r = p_fast_two_sum(p_mul(h2, f2(4194304.f)), h1);  // units of 2^21 2^-64
-  return p_fast_two_sum(r.h, p_fma(h0, f2(4.76837158203125e-7f), r.l));
+};
+template <int NM>
+__device__ __forceinline__ df2 crt_fraction(const rns::Crt<NM>& C, const uint32_t (&w)[NM], uint32_t chunks) {
+  CrtSum s;
+  s.add(C, w);
+  return s.fraction(C, chunks);
 }
 
 // (h, l) 2^e for each entry
@@ -484,7 +499,8 @@ constexpr int kRing = 224 * 1024;
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 32 * (2 + kEpiWarps);  // warp 0 TMA, 1 MMA, 2.. epilogue
 constexpr int kSmem = kRing + 1024 + 256;
-constexpr int kMaxChunks = 96;  // per unit: a 16-bit sum of residues + 256 (at most 437 each) holds 149
+constexpr int kMaxChunks = 96;  // per unit
+static_assert(kMaxChunks <= rns::kSumChunks, "a unit's 16-bit sums");
 static_assert(kSmem <= 227 * 1024, "shared memory per CTA");
 
 struct GemmArgs {
@@ -888,9 +904,10 @@ __global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* __rest
 // w_p = g_p u_p into shared memory, two consecutive descriptors per thread and step; then `lanes`
 // lanes per atom sum shares of its N - 1 pair terms, all three coordinates (the derivative of x_p
 // with respect to its first atom i > j carries the minus sign).  CTA 0 clears the column maxima for
-// the next matvec.
-template <int NM>
-__global__ void __launch_bounds__(256, 4) rns_backproj_kernel(const uint16_t* __restrict__ Up, int slabs, int chunks,
+// the next matvec.  A product's slabs are added as packed 16-bit sums; WIDE (more than kSumChunks chunks
+// in all, MB > 76,288): `per_sum` slabs at a time, and these in the reconstruction's wider sums.
+template <int NM, bool WIDE>
+__global__ void __launch_bounds__(256, 4) rns_backproj_kernel(const uint16_t* __restrict__ Up, int slabs, int per_sum, int chunks,
                                                               int64_t M, int D, int Dp, int64_t ldU,
                                                               const int* __restrict__ sA, const int* __restrict__ sWT,
                                                               const int* __restrict__ sB, const int* __restrict__ sXT,
@@ -914,23 +931,31 @@ __global__ void __launch_bounds__(256, 4) rns_backproj_kernel(const uint16_t* __
   const df2 pm{f2(C.pih), f2(C.pil)};
   for (unsigned p = 2 * tid; p <= (unsigned)D; p += 2 * blockDim.x) {
     uint32_t w[2][NM];
-#pragma unroll
-    for (int sg = 0; sg < 2; ++sg)
-#pragma unroll
-      for (int i = 0; i < NM; ++i)
-        w[sg][i] = *reinterpret_cast<const uint32_t*>(Ua + (int64_t)(sg * slabs * NM + i) * plane + p);
-    const unsigned q = p >> 1, qg = min(q, (unsigned)H - 1u);
-    const float4 g[3] = {Ga[qg], Ga[H + qg], Ga[2 * H + qg]};
-    for (int sl = 1; sl < slabs; ++sl)
+    CrtSum sum[2];
+    auto load = [&](int s0, int s1) {  // slabs s0 .. s1 - 1
 #pragma unroll
       for (int sg = 0; sg < 2; ++sg)
 #pragma unroll
         for (int i = 0; i < NM; ++i)
-          w[sg][i] += *reinterpret_cast<const uint32_t*>(Ua + (int64_t)((sg * slabs + sl) * NM + i) * plane + p);
+          w[sg][i] = *reinterpret_cast<const uint32_t*>(Ua + (int64_t)((sg * slabs + s0) * NM + i) * plane + p);
+      for (int sl = s0 + 1; sl < s1; ++sl)
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg)
+#pragma unroll
+          for (int i = 0; i < NM; ++i)
+            w[sg][i] += *reinterpret_cast<const uint32_t*>(Ua + (int64_t)((sg * slabs + sl) * NM + i) * plane + p);
+    };
+    const unsigned q = p >> 1, qg = min(q, (unsigned)H - 1u);
+    const float4 g[3] = {Ga[qg], Ga[H + qg], Ga[2 * H + qg]};
+    for (int s0 = 0; s0 < slabs; s0 += WIDE ? per_sum : slabs) {
+      load(s0, WIDE ? min(s0 + per_sum, slabs) : slabs);
+      sum[0].add(C, w[0]);
+      sum[1].add(C, w[1]);
+    }
     // (the scales of columns 0 .. D, padded to an even count)
     const int2 e0 = *reinterpret_cast<const int2*>(sWT + p), e1 = *reinterpret_cast<const int2*>(sXT + p);
-    const df2 x = p_scale(crt_fraction<NM>(C, w[0], (uint32_t)chunks), ea - e0.x, ea - e0.y);
-    const df2 y = p_scale(crt_fraction<NM>(C, w[1], (uint32_t)chunks), eb - e1.x, eb - e1.y);
+    const df2 x = p_scale(sum[0].fraction(C, (uint32_t)chunks), ea - e0.x, ea - e0.y);
+    const df2 y = p_scale(sum[1].fraction(C, (uint32_t)chunks), eb - e1.x, eb - e1.y);
     if (p == (unsigned)D) rs = make_float2(y.h.x, y.l.x);
     if (p + 1 == (unsigned)D) rs = make_float2(y.h.y, y.l.y);
     if (p < (unsigned)D) {
@@ -1154,7 +1179,8 @@ gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, co
   constexpr int NM = rns::kMvMods;
   if (Ssym < 1 || (Ssym > 1 && (!pis || !XcB))) return fail(GDML_ERR_ARG, "residue setup: bad symmetry arguments");
   const int64_t MB = M * Ssym;
-  if (MB > (int64_t)1 << 24 || D > (1 << 20)) return fail(GDML_ERR_ARG, "system too large for the residue path");
+  // (beta's kernel adds all K groups of T as packed 16-bit sums)
+  if (MB > (int64_t)1 << 24 || D > rns::kSumChunks * rns::kChunk) return fail(GDML_ERR_ARG, "system too large for the residue path");
   r.M = M;
   r.MB = MB;
   r.N = N;
@@ -1278,8 +1304,11 @@ gdml_status rns_matvec(RnsMatvec& r, const double* G, const double* Xc, const do
   const int nb = row_threads(M, cdiv(D + 1, 2), sm);
   int lanes = 4;  // per atom in the last step: as many as the threads give, up to 16
   while (lanes < 16 && 2 * lanes * r.N <= nb) lanes *= 2;
-  RNS_TRY(big_smem(rns_backproj_kernel<NM>, sm));
-  { launch_after(pdl, rns_backproj_kernel<NM>, (unsigned)M, nb, sm, st, r.Up, s2, (int)r.nch2, M, D, r.Dp, r.ldU, r.A2.s, r.WT2.s, r.B2.s, r.XT2.s, r.JX, (const float4*)r.G3, v, r.N, lam, add_lambda, lanes, r.colmax, out); count_launch(); }
+  const bool wide = r.nch2 > rns::kSumChunks;
+  const int per_sum = rns::kSumChunks / rns_chunks(r.nch2, r.g2, r.cap2);
+  auto* backproj = wide ? rns_backproj_kernel<NM, true> : rns_backproj_kernel<NM, false>;
+  RNS_TRY(big_smem(backproj, sm));
+  { launch_after(pdl, backproj, (unsigned)M, nb, sm, st, r.Up, s2, per_sum, (int)r.nch2, M, D, r.Dp, r.ldU, r.A2.s, r.WT2.s, r.B2.s, r.XT2.s, r.JX, (const float4*)r.G3, v, r.N, lam, add_lambda, lanes, r.colmax, out); count_launch(); }
   if (cudaGetLastError() != cudaSuccess) return fail(GDML_ERR_CUDA, "residue matvec kernels");
   return GDML_OK;
 }

@@ -39,6 +39,7 @@ constexpr int kMods[kMaxMod] = {361, 359, 358, 355, 353, 351, 349, 347, 343, 341
 constexpr int kMvMods = 14;  // the matvec's: P = 2^117.9
 constexpr int kMvBits = 57;  // both operands: 2^114 < P / 2
 constexpr int kChunk = 512;  // K entries whose products of residues sum exactly in FP32
+constexpr int kSumChunks = 149;  // chunks whose residues + 256 (at most 437 each) a 16-bit sum holds
 constexpr int kDigit = 14;  // residues are formed from digits of 14 bits, four per integer
 constexpr int kBad = -100000;  // scale of a row that holds a NaN or an infinity
 

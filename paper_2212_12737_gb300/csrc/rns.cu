@@ -377,8 +377,8 @@ __global__ void __launch_bounds__(512) rns_proj_kernel(const float4* __restrict_
 // column's largest magnitude.  One CTA per 32 rows x 32 columns through shared memory; a thread
 // writes four consecutive entries of an operand row per modulus (8 bytes, 64 per row).
 template <int NM, typename T>
-__global__ void __launch_bounds__(256) rns_cols_kernel(const T* __restrict__ W, int64_t MB, int D, int ldW,
-                                                       const unsigned* __restrict__ colmax, int64_t Kp, int64_t rows,
+__global__ void __launch_bounds__(256) rns_cols_kernel(const T* W, int64_t MB, int D, int ldW,
+                                                       const unsigned* colmax, int64_t Kp, int64_t rows,
                                                        int bits, bf16* __restrict__ d, int* __restrict__ sc) {
   __shared__ float2 tile[32][33];
   const int64_t b0 = (int64_t)blockIdx.x * 32;
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(256) rns_cols_kernel(const T* __restrict__ W, 
 #pragma unroll
     for (int r0 = 0; r0 < 32; r0 += 8) {
       const int r = r0 + (threadIdx.x >> 5);
-      tile[c][r] = b0 + r < MB && d0 + c < D ? as_pair(W[(b0 + r) * ldW + d0 + c]) : make_float2(0.f, 0.f);
+      tile[c][r] = b0 + r < MB && d0 + c < D ? as_pair(__ldcg(W + (b0 + r) * ldW + d0 + c)) : make_float2(0.f, 0.f);
     }
   }
   const int c = threadIdx.x >> 3, r = (threadIdx.x & 7) * 4;
@@ -844,10 +844,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 // against three; rows that fit the chip as CTAs of 128 threads run in one round (see row_threads).
 constexpr int64_t kBetaStage = 24 * 1024;
 template <int NM, bool STAGE>
-__global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* __restrict__ Tp, int slabs, int chunks,
+__global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* Tp, int slabs, int chunks,
                                                           int64_t M, int64_t MB, int64_t ldT,
-                                                          const int* __restrict__ sA, const int* __restrict__ sW,
-                                                          const float2* __restrict__ S2, const float2* __restrict__ t2,
+                                                          const int* __restrict__ sA, const int* sW,
+                                                          const float2* __restrict__ S2, const float2* t2,
                                                           float rootMB, int64_t Kp, int bits, bf16* __restrict__ d,
                                                           int* __restrict__ sc) {
   extern __shared__ float4 sb[];
@@ -865,12 +865,12 @@ __global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* __rest
   auto beta2 = [&](unsigned b) {  // columns b, b + 1 (b even)
     uint32_t w[NM];
 #pragma unroll
-    for (int i = 0; i < NM; ++i) w[i] = *reinterpret_cast<const uint32_t*>(Ta + i * plane + b);
-    const df2 S = as_df2(Sa[b >> 1]), t = as_df2(reinterpret_cast<const float4*>(t2)[b >> 1]);
-    const int2 e2 = *reinterpret_cast<const int2*>(sW + b);
+    for (int i = 0; i < NM; ++i) w[i] = __ldcg(reinterpret_cast<const uint32_t*>(Ta + i * plane + b));
+    const df2 S = as_df2(Sa[b >> 1]), t = as_df2(__ldcg(reinterpret_cast<const float4*>(t2) + (b >> 1)));
+    const int2 e2 = __ldcg(reinterpret_cast<const int2*>(sW + b));
     for (int sl = 1; sl < slabs; ++sl)
 #pragma unroll
-      for (int i = 0; i < NM; ++i) w[i] += *reinterpret_cast<const uint32_t*>(Ta + (sl * NM + i) * plane + b);
+      for (int i = 0; i < NM; ++i) w[i] += __ldcg(reinterpret_cast<const uint32_t*>(Ta + (sl * NM + i) * plane + b));
     df2 r = p_df_mul(S, p_df_sub(p_scale(crt_fraction<NM>(C, w, (uint32_t)chunks), ea - e2.x, ea - e2.y), t));
     if (b + 1 >= n) r.h.y = r.l.y = 0.f;
     return r;
@@ -907,14 +907,14 @@ __global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* __rest
 // the next matvec.  A product's slabs are added as packed 16-bit sums; WIDE (more than kSumChunks chunks
 // in all, MB > 76,288): `per_sum` slabs at a time, and these in the reconstruction's wider sums.
 template <int NM, bool WIDE>
-__global__ void __launch_bounds__(256, 4) rns_backproj_kernel(const uint16_t* __restrict__ Up, int slabs, int per_sum, int chunks,
+__global__ void __launch_bounds__(256, 4) rns_backproj_kernel(const uint16_t* Up, int slabs, int per_sum, int chunks,
                                                               int64_t M, int D, int Dp, int64_t ldU,
-                                                              const int* __restrict__ sA, const int* __restrict__ sWT,
-                                                              const int* __restrict__ sB, const int* __restrict__ sXT,
+                                                              const int* __restrict__ sA, const int* sWT,
+                                                              const int* sB, const int* __restrict__ sXT,
                                                               const float2* __restrict__ JX,
                                                               const float4* __restrict__ G3,
                                                               const double* __restrict__ v, int N, double lam,
-                                                              int add_lambda, int lanes, unsigned* __restrict__ colmax,
+                                                              int add_lambda, int lanes, unsigned* colmax,
                                                               double* __restrict__ out) {
   extern __shared__ float4 w4[];  // [3][Dp] pairs: the terms g_pc u_p
   __shared__ float2 rs;
@@ -922,7 +922,7 @@ __global__ void __launch_bounds__(256, 4) rns_backproj_kernel(const uint16_t* __
   const int tid = threadIdx.x, H = Dp >> 1;
   constexpr rns::Crt<NM> C{};
   grid_wait();
-  const int ea = C.pexp - 43 - sA[a], eb = C.pexp - 43 - sB[a];
+  const int ea = C.pexp - 43 - sA[a], eb = C.pexp - 43 - __ldcg(sB + a);
   if (a == 0)
     for (int p = tid; p < kColCopies * Dp; p += blockDim.x) colmax[p] = 0u;
   const int64_t plane = M * ldU;
@@ -937,13 +937,13 @@ __global__ void __launch_bounds__(256, 4) rns_backproj_kernel(const uint16_t* __
       for (int sg = 0; sg < 2; ++sg)
 #pragma unroll
         for (int i = 0; i < NM; ++i)
-          w[sg][i] = *reinterpret_cast<const uint32_t*>(Ua + (int64_t)((sg * slabs + s0) * NM + i) * plane + p);
+          w[sg][i] = __ldcg(reinterpret_cast<const uint32_t*>(Ua + (int64_t)((sg * slabs + s0) * NM + i) * plane + p));
       for (int sl = s0 + 1; sl < s1; ++sl)
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg)
 #pragma unroll
           for (int i = 0; i < NM; ++i)
-            w[sg][i] += *reinterpret_cast<const uint32_t*>(Ua + (int64_t)((sg * slabs + sl) * NM + i) * plane + p);
+            w[sg][i] += __ldcg(reinterpret_cast<const uint32_t*>(Ua + (int64_t)((sg * slabs + sl) * NM + i) * plane + p));
     };
     const unsigned q = p >> 1, qg = min(q, (unsigned)H - 1u);
     const float4 g[3] = {Ga[qg], Ga[H + qg], Ga[2 * H + qg]};
@@ -953,7 +953,7 @@ __global__ void __launch_bounds__(256, 4) rns_backproj_kernel(const uint16_t* __
       sum[1].add(C, w[1]);
     }
     // (the scales of columns 0 .. D, padded to an even count)
-    const int2 e0 = *reinterpret_cast<const int2*>(sWT + p), e1 = *reinterpret_cast<const int2*>(sXT + p);
+    const int2 e0 = __ldcg(reinterpret_cast<const int2*>(sWT + p)), e1 = *reinterpret_cast<const int2*>(sXT + p);
     const df2 x = p_scale(sum[0].fraction(C, (uint32_t)chunks), ea - e0.x, ea - e0.y);
     const df2 y = p_scale(sum[1].fraction(C, (uint32_t)chunks), eb - e1.x, eb - e1.y);
     if (p == (unsigned)D) rs = make_float2(y.h.x, y.l.x);
@@ -1259,7 +1259,7 @@ static int row_threads(int64_t M, int64_t pairs, size_t smem) {
 }
 
 // Whether the matvec's kernels may start while the one before them drains (each waits for it before it
-// reads): about 1.5 us of launch and start-up per kernel.  Outside capture only, and where a kernel's rows
+// reads, and reads what a kernel of the same matvec wrote past L1, never as read-only data): about 1.5 us of launch and start-up per kernel.  Outside capture only, and where a kernel's rows
 // are resident at once: M = 200, D = 36 28.3 us, 38.6 without; M = 1,000, D = 210 92.9 and 98.9; but M = 5,000,
 // D = 861 1,660 and 1,588, and a captured solve at M = 1,000 8.96 and 8.85 ms.
 static bool chained(int64_t M, cudaStream_t st) {

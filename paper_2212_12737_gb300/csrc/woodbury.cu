@@ -260,7 +260,7 @@ __device__ __forceinline__ void dot_col(const float4 (&a)[4], const float2 (&rv)
 // end.  VEC: n % 4 == 0 (aligned float4 loads).
 template <bool VEC>
 __global__ void __launch_bounds__(256, 2) gemv_t_df_kernel(const float* __restrict__ L, int64_t n, int64_t k,
-                                                           const float2* __restrict__ rs, double* __restrict__ part) {
+                                                           const float2* rs, double* __restrict__ part) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t i0 = (int64_t)blockIdx.y * kDfRows;
   const int64_t rem = n - i0;
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(256, 2) gemv_t_df_kernel(const float* __restri
 // warps' partials are combined in a fixed order through shared memory.
 template <bool VEC>
 __global__ void __launch_bounds__(256, 2) gemv_n_df_kernel(const float* __restrict__ L, int64_t n, int64_t k,
-                                                           const float2* __restrict__ us, float2* __restrict__ zp) {
+                                                           const float2* us, float2* __restrict__ zp) {
   __shared__ float2 part[8][kDfRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t i0 = (int64_t)blockIdx.x * kDfRows;
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(256, 2) gemv_n_df_kernel(const float* __restri
 }
 
 // z[i] = (r[i] - sum_g zp[g][i]) / lambda (groups in a fixed order)
-__global__ void gemv_n_df_finish_kernel(const float2* __restrict__ zp, int64_t n, const double* __restrict__ r,
+__global__ void gemv_n_df_finish_kernel(const float2* zp, int64_t n, const double* __restrict__ r,
                                         double inv_lam, double* __restrict__ z) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   grid_wait();
@@ -708,9 +708,8 @@ __device__ __forceinline__ void df_term(float& h, float& l, float ah, float al, 
 // are reduced by a fixed shuffle tree and then across the 8 warps in order.
 template <bool EVEN>
 __global__ void __launch_bounds__(256) symv_df_kernel(const float2* __restrict__ A, int64_t k,
-                                                      const float2* __restrict__ x, int mode,
-                                                      const double* __restrict__ t, double* __restrict__ y,
-                                                      float2* __restrict__ y2) {
+                                                      const float2* x, int mode, const double* t,
+                                                      double* y, float2* __restrict__ y2) {
   __shared__ float2 red[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t i = blockIdx.x;
@@ -750,9 +749,9 @@ __global__ void __launch_bounds__(256) symv_df_kernel(const float2* __restrict__
     v = s;
     y[i] = v;
   } else if (mode == 1) {
-    v = t[i] - s;
+    v = __ldcg(t + i) - s;
   } else {
-    v = y[i] + s;
+    v = __ldcg(y + i) + s;
     y[i] = v;
   }
   const float vh = (float)v;
@@ -866,18 +865,18 @@ static void symv_df(const float2* A, int64_t k, const float2* x, int mode, const
 // t[j] = sum of the chunk partials (as reduce_chunks_kernel), also split into t2[j]; PAIRS:
 // the partials are double-float pairs (float2) rather than doubles
 template <bool PAIRS>
-__device__ __forceinline__ void reduce_row_df(const double* __restrict__ part, int64_t nchunks,
+__device__ __forceinline__ void reduce_row_df(const double* part, int64_t nchunks,
                                               double* __restrict__ t, float2* __restrict__ t2, int64_t j, int lane) {
   double s = 0.0;
   if (PAIRS) {
     const float2* pj = reinterpret_cast<const float2*>(part) + j * nchunks;
     for (int64_t c = lane; c < nchunks; c += 32) {
-      const float2 v = pj[c];
+      const float2 v = __ldcg(pj + c);
       s += (double)v.x + (double)v.y;
     }
   } else {
     const double* pj = part + j * nchunks;
-    for (int64_t c = lane; c < nchunks; c += 32) s += pj[c];
+    for (int64_t c = lane; c < nchunks; c += 32) s += __ldcg(pj + c);
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) {
@@ -888,7 +887,7 @@ __device__ __forceinline__ void reduce_row_df(const double* __restrict__ part, i
 }
 
 template <bool PAIRS>
-__global__ void __launch_bounds__(256) reduce_chunks_df_kernel(const double* __restrict__ part, int64_t nchunks,
+__global__ void __launch_bounds__(256) reduce_chunks_df_kernel(const double* part, int64_t nchunks,
                                                                int64_t k, double* __restrict__ t,
                                                                float2* __restrict__ t2) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1104,7 +1103,7 @@ void woodbury_apply_df(const float* L, int64_t n, int64_t k, const double* C, co
   }
   // Outside capture the launches of this path may start while the one before them drains: each waits for it
   // before it reads anything but L and the k x k matrices, and lets the next one start only then, so that at
-  // most two are under way; vectors that a launch of the chain rewrites are read past L1.  Eight launches of
+  // most two are under way; what a launch of the chain writes is read past L1, never as read-only data.  Eight launches of
   // 3 to 11 us: n = 34,965, k = 77 45.1 -> 32.4 us.
   df_pass_t(L, n, k, rs, part, t, t2, plan, err, st);
   // u = C^-1 t, refined once with the residual t - C u (see woodbury_apply)

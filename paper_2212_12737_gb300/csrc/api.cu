@@ -979,15 +979,18 @@ static gdml_status precond_build_impl(gdml_ctx* c, int32_t method, int64_t k, ui
     a.part = part;
     a.ticket = ticket;
     a.col = col;
-    a.get_col = [c](const int64_t* cols, double* out, const int* stop, cudaStream_t st) {
+    a.get_col = [c](const int64_t* cols, double* out, PivState* ps, unsigned step, cudaStream_t st) {
+      const int* stop = &ps->stop;
       if (c->Ssym > 1) {  // checked to fit at setup
         (void)launch_kcol_sym(cols, 1, c->X, c->G, c->S, c->P64, 2 * c->MB, c->M, c->MB, c->N, c->D, c->pis, c->pinv,
                               c->Ssym, c->c, out, c->n, stop, st);
-        return;
+        return false;
       }
-      if (!c->X2 || !launch_kcol_df(cols, 1, c->X2, c->G2, c->S, c->P64, 2 * c->M, c->M, c->N, c->D, c->c, out,
-                                    c->n, stop, st))
-        launch_kcol(cols, 1, c->X, c->G, c->S, c->P64, 2 * c->M, c->M, c->N, c->D, c->c, out, c->n, stop, st);
+      if (c->X2 && launch_kcol_df(cols, 1, c->X2, c->G2, c->S, c->P64, 2 * c->M, c->M, c->N, c->D, c->c, out, c->n,
+                                  stop, st, step ? &ps->step : nullptr, step))
+        return step > 0;
+      launch_kcol(cols, 1, c->X, c->G, c->S, c->P64, 2 * c->M, c->M, c->N, c->D, c->c, out, c->n, stop, st);
+      return false;
     };
     if (df_precond(c)) {
       TRY(s.get(&a.schur, (size_t)(pivchol_schur_groups() * n)));

@@ -418,12 +418,16 @@ __device__ __forceinline__ float2 dfk_mul(float2 a, float2 b) {  // a b
 // FP64 form of this kernel was bound by it; the column is accurate to ~1e-14 of its terms,
 // the class of the double-float Schur sums it meets in Algorithm 1.  S and A are symmetric:
 // column b is read as row b.  One warp per geometry a, W warps per CTA.
-__global__ void __launch_bounds__(256) kcol_df_kernel(const int64_t* __restrict__ cols,
+//
+// Algorithm 1 (released not null): the grid starts beside the step before and waits for it here; its first
+// thread then releases `step`, so that the Schur step that starts beside THIS grid, and acquires it, sees
+// what the step before wrote (a grid sees what it waited for; one that a trigger started does not).
+__global__ void __launch_bounds__(256) kcol_df_kernel(const int64_t* cols,
                                                       const float2* __restrict__ X2, const float2* __restrict__ G2,
                                                       const double* __restrict__ S, const double* __restrict__ A,
                                                       int64_t ldA, int64_t M, int N, int D, double c2,
                                                       double* __restrict__ out, int64_t ldo,
-                                                      const int* __restrict__ stop_flag) {
+                                                      const int* stop_flag, unsigned* released, unsigned step) {
   extern __shared__ float2 shf[];
   const int W = blockDim.x >> 5;
   float2* wsp = shf;        // N: +-g_b on the pairs (i, j), indexed by partner j
@@ -460,8 +464,10 @@ __global__ void __launch_bounds__(256) kcol_df_kernel(const int64_t* __restrict_
     }
   }
   grid_wait();
+  if (released && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(released), "r"(step) : "memory");
   if (stop_flag && __ldcg(stop_flag)) return;
-  grid_trigger();  // (after the wait: the next kernel may rely on what came before this one)
+  grid_trigger();  // (after the wait and the release: the next kernel needs not poll)
   const int64_t col = __ldcg(cols + c);
   const int64_t b = col / B;
   const int l = (int)(col - b * B), i = l / 3, q = l - 3 * i;
@@ -728,7 +734,7 @@ bool launch_kcol_bulk_df(const int64_t* cols, int64_t ncols, const float2* X2, c
 
 bool launch_kcol_df(const int64_t* cols, int64_t ncols, const float2* X2, const float2* G2, const double* S,
                     const double* A, int64_t ldA, int64_t M, int N, int D, double c, double* out, int64_t ldo,
-                    const int* stop_flag, cudaStream_t st) {
+                    const int* stop_flag, cudaStream_t st, unsigned* released, unsigned step) {
   const size_t per_warp = 5 * (size_t)D * sizeof(float2), fixed = ((size_t)N + D) * sizeof(float2);
   int W = (int)std::min<size_t>(8, (200 * 1024 - std::min<size_t>(fixed, 200 * 1024)) / per_warp);
   if (W < 1 || ncols > 65535) return false;
@@ -743,7 +749,7 @@ bool launch_kcol_df(const int64_t* cols, int64_t ncols, const float2* X2, const 
   }
   dim3 g((unsigned)cdiv(M, W), (unsigned)ncols);
   // stop_flag: Algorithm 1's step, which follows the previous one without waiting for it to drain
-  { launch_after(stop_flag != nullptr, kcol_df_kernel, g, 32 * W, wsmem, st, cols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag); count_launch(); }
+  { launch_after(stop_flag != nullptr, kcol_df_kernel, g, 32 * W, wsmem, st, cols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag, released, step); count_launch(); }
   return true;
 }
 

@@ -26,7 +26,7 @@ void launch_dist_tab(const double* X, int64_t M, int D, double c, double* S, dou
 // or ncols > 65535
 bool launch_kcol_df(const int64_t* cols, int64_t ncols, const float2* X2, const float2* G2, const double* S,
                     const double* A, int64_t ldA, int64_t M, int N, int D, double c, double* out, int64_t ldo,
-                    const int* stop_flag, cudaStream_t st);
+                    const int* stop_flag, cudaStream_t st, unsigned* released = nullptr, unsigned step = 0);
 // many kernel columns at once in double-float (the Nystrom factor's K_nk), with a scratch of
 // kcol_bulk_scratch float pairs; false (nothing launched) when a geometry's operands do not fit in
 // shared memory (D > 6784)
@@ -186,7 +186,7 @@ struct PivState {
   int64_t piv;
   int64_t rank;
   int stop;
-  int pad;
+  unsigned step;  // the kernel column of step - 1 has seen everything the step before it wrote (kcol_df_kernel)
 };
 struct ArgMaxPart {
   double v;
@@ -204,7 +204,8 @@ struct PivCholArgs {
   ArgMaxPart* part;
   unsigned* ticket;
   double* col;
-  std::function<void(const int64_t*, double*, const int*, cudaStream_t)> get_col;
+  // the kernel column of *col, unless ps->stop; with step > 0 it may release ps->step = step (true: it does)
+  std::function<bool(const int64_t* col, double* out, PivState* ps, unsigned step, cudaStream_t)> get_col;
   // DF64 form only: pivot-row gather (k floats) and Schur partials (pivchol_schur_groups() * n pairs)
   float* prow = nullptr;
   float2* schur = nullptr;

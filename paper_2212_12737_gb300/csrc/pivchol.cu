@@ -409,28 +409,38 @@ __global__ void __launch_bounds__(kArgThreads) pc_finish_select_df_kernel(
     }
 }
 
-// Algorithm 1 step m in one TMA-staged pass: the Schur sums s_i = sum_{j<m} L[i + j n] prow[j]
-// of ws_gemv_n_kernel's SCHUR mode, followed row by row (as each chunk's sums are combined)
-// by pc_finish_select_df_kernel's work: l_{i,m}, column m of L, the residual diagonal, the
+// Bounded wait until *p has reached `step`; what its releaser saw is then visible here
+__device__ __forceinline__ bool acquire_step(const unsigned* p, unsigned step) {
+  const uint32_t limit = tc::g_wait_limit;
+  for (uint32_t it = 0; it < limit; ++it) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    if (v >= step) return true;
+  }
+  return false;
+}
+
+// Algorithm 1 step m in one TMA-staged pass: the Schur sums s_i = sum_{j<m} L[i + j n] L[piv + j n],
+// followed row by row (as each chunk's sums are combined) by pc_finish_select_df_kernel's work: l_{i,m}, column m of L, the residual diagonal, the
 // argmax and the trace.  The last CTA to finish selects the pivot of step m + 1 and performs the swap.
 // Bounded by HBM while it streams; what comes before and after is a chain of latencies, at n = 63,000,
 // k = 2,000 at the end 36 us of a step's 111 (160 ms for the build; 140 ms so), therefore
-//  - it starts beside the step's kernel column (see launch_after) and waits for it only at the end;
+//  - it starts beside the step's kernel column (see launch_after) and waits for it only at the end.  What
+//    it reads before that (the pivot, the rows' state, columns of L, these also by TMA) the step before
+//    wrote, which the kernel column waited for: it releases ps->step, acquired here (step > 0) and carried
+//    to the copies by a proxy fence.  A column that releases nothing is not overlapped (step = 0);
 //  - lanes fetch the pivot row's entries straight from L, 32 / CPW tiles ahead (gathered by the last CTA
 //    of the step before: up to 8 us);
 //  - the rows' state is loaded before the stream, and the argmax carries the row with its position;
 //  - the leading `keep` columns stay in L2 (64 MB of them: 4 ms of the build; 96 MB: 1 ms).
 template <int NT>
 __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
-    const __grid_constant__ CUtensorMap map, int64_t n, int64_t m, int64_t nch, int64_t keep, int select, float* __restrict__ L,
-    const double* __restrict__ col, double* __restrict__ d,
-    unsigned char* __restrict__ chosen, int64_t* __restrict__ perm, int64_t* __restrict__ posof,
-    int64_t* __restrict__ pivots, double* __restrict__ trace, PivState* __restrict__ ps,
-    ArgMaxPart* __restrict__ part, unsigned* __restrict__ ticket, int* __restrict__ err) {
+    const __grid_constant__ CUtensorMap map, int64_t n, int64_t m, int64_t nch, int64_t keep, int select, unsigned step, float* L,
+    const double* col, double* d, unsigned char* chosen, int64_t* perm, int64_t* posof, int64_t* pivots, double* trace,
+    PivState* ps, ArgMaxPart* part, unsigned* ticket, int* err) {
   constexpr int RC = 128 * NT, COLS = 32 / NT, CPW = 4 / NT;
   constexpr int kW = kWsWarps + 1;
   grid_trigger();  // (the next column's CTAs may start once all of these have)
-  if (__ldcg(&ps->stop)) return;  // (up to grid_wait, state is read past L1, which may hold the last step's)
   extern __shared__ uint8_t ws_smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(ws_smem_raw) + kWsAlign - 1) &
                                              ~uintptr_t(kWsAlign - 1));
@@ -446,23 +456,32 @@ __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
   __shared__ bool last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntiles = (int)((m + COLS - 1) / COLS);
-  const int64_t piv = __ldcg(&ps->piv);
-  const double lmm = __ldcg(&ps->lmm), ilmm = __ldcg(&ps->ilmm);
-  const int64_t other = select && threadIdx.x == 0 ? __ldcg(perm + m + 1) : 0;
   if (threadIdx.x == 0) {
     ws_init(full, empty, cbar, abort_flag);
     issued_s = 0;
+    if (step > 0 && !acquire_step(&ps->step, step)) {
+      atomicExch(err, tc::ERR_TIMEOUT_DONE);
+      *abort_flag = 1;
+    }
   }
   __syncthreads();
+  // (up to grid_wait, state is read past L1, which may hold the last step's)
+  const int stop = __ldcg(&ps->stop);
+  const int64_t piv = __ldcg(&ps->piv);
+  const double lmm = __ldcg(&ps->lmm), ilmm = __ldcg(&ps->ilmm);
+  const int64_t other = select && threadIdx.x == 0 ? __ldcg(perm + m + 1) : 0;
+  if (stop) return;
   ArgMax best{-1.0 / 0.0, INT64_MAX};
   double sum = 0.0;
   if (warp == kWsWarps) {
-    if (lane == 0)
+    if (lane == 0) {
+      asm volatile("fence.proxy.async;" ::: "memory");  // columns of L by ordinary stores, read by TMA
       issued_s = ws_produce<NT, true>(&map, ring, full, empty, abort_flag, nch, ntiles, (int)(keep / COLS), err);
+    }
   } else {
     WsRing rp;
     uint32_t ci = 0;
-    bool go = true;
+    bool go = !*abort_flag;
     for (int64_t ch = blockIdx.x; ch < nch && go; ch += gridDim.x, ++ci) {
       float2 h2[NT][2], l2[NT][2];
 #pragma unroll
@@ -672,17 +691,17 @@ void pivchol_run_df(const PivCholArgs& a, float* L, cudaStream_t st) {
     }
     const int64_t keep = ((int64_t)64 << 20) / (4 * a.n);
     for (int64_t m = 0; m < a.k; ++m) {
-      a.get_col(a.pivots + m, a.col, &a.ps->stop, st);
+      const unsigned step = a.get_col(a.pivots + m, a.col, a.ps, (unsigned)(m + 1), st) ? (unsigned)(m + 1) : 0u;
       const int select = m + 1 < a.k ? 1 : 0;
       if (plan.rc == 256)
-        { launch_after(true, pc_schur_finish_ws_kernel<2>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
+        { launch_after(step > 0, pc_schur_finish_ws_kernel<2>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, step, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
       else
-        { launch_after(true, pc_schur_finish_ws_kernel<1>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
+        { launch_after(step > 0, pc_schur_finish_ws_kernel<1>, plan.grid, kWsThreads, kWsSmemN, st, plan.map, a.n, m, plan.nch, keep, select, step, L, a.col, a.d, a.chosen, a.perm, a.posof, a.pivots, a.trace, a.ps, a.part, a.ticket, a.err); count_launch(); }
     }
     return;
   }
   for (int64_t m = 0; m < a.k; ++m) {
-    a.get_col(a.pivots + m, a.col, &a.ps->stop, st);
+    (void)a.get_col(a.pivots + m, a.col, a.ps, 0, st);
     // column groups: enough CTAs for ~4 per SM, at least 32 columns per group
     int groups = 0;
     if (m > 0) {
@@ -704,7 +723,7 @@ void pivchol_run(const PivCholArgs& a, TL* L, cudaStream_t st) {
   for (int64_t m = 0; m < a.k; ++m) {
     { pc_argmax_kernel<<<arg_blocks(), kArgThreads, 0, st>>>(m, a.n, 1, a.d, a.perm, a.chosen, a.pivots, a.trace,
                                                          a.ps, a.part, a.ticket); count_launch(); }
-    a.get_col(a.pivots + m, a.col, &a.ps->stop, st);
+    (void)a.get_col(a.pivots + m, a.col, a.ps, 0, st);
     { pc_update_kernel<TL><<<(unsigned)cdiv(a.n, 256), 256, 0, st>>>(m, a.n, L, a.col, a.d, a.chosen, a.ps); count_launch(); }
   }
   // trace after the last step

@@ -1,5 +1,5 @@
-"""Launches that start while the one before them drains (OZAKI matvec and apply outside capture) must
-give the bits of the same launches one after another.
+"""Launches that start while the one before them drains (OZAKI matvec and apply outside capture, the
+steps of Algorithm 1 with an FP32 factor) must give the bits of the same launches one after another.
 
 Reference: a process of its own with CUDA_LAUNCH_BLOCKING=1, where no two kernels are ever under way
 together.  Here the same calls run back to back on a stream of their own, each on other vectors than
@@ -22,6 +22,10 @@ NV, ROUNDS = 6, 5
 # (n % 4 != 0; odd and even k), staged passes with the separate k x k products (odd k)
 SYSTEMS = [(9, 200, False, 101), (15, 777, False, 77), (13, 333, False, 64), (21, 1000, False, 0), (9, 151, True, 0)]
 
+# Algorithm 1: N, M, k, precision (steps of one and several chunks of rows; k = n, where the residual
+# diagonal ends and the remaining steps return at once)
+BUILDS = [(9, 200, 400, "ozaki"), (21, 400, 600, "ozaki"), (9, 100, 200, "df64"), (4, 8, 96, "ozaki")]
+
 
 def context(N, M, sym, k, stream=None):
     perms = [[0, 1, 2], [0, 2, 1], [1, 0, 2], [1, 2, 0], [2, 0, 1], [2, 1, 0]]
@@ -38,6 +42,16 @@ def vectors(n):
     return torch.from_numpy(np.random.default_rng(n).standard_normal((NV, n))).cuda()
 
 
+def build(N, M, k, precision, stream=None):
+    R = torch.from_numpy(synth.geometries(synth.template(N, 1), M, 0.05, 2)).cuda()
+    torch.cuda.synchronize()
+    ctx = gdml.kernel_setup(R, 10.0, 1e-3, precision, stream=stream)
+    piv, trace = ctx.precond_build("pivchol", k, pivots=True, trace=True)
+    out = dict(piv=piv.cpu().numpy(), trace=trace.cpu().numpy(), L=ctx.precond_factor().cpu().numpy())
+    ctx.destroy()
+    return out
+
+
 def serial(path):
     """What the reference process computes."""
     out = {}
@@ -48,6 +62,8 @@ def serial(path):
             if k:
                 out[f"ap{s}_{i}"] = ctx.precond_apply(v).cpu().numpy()
         ctx.destroy()
+    for b, args in enumerate(BUILDS):
+        out.update({f"build{b}_{k}": v for k, v in build(*args).items()})
     np.savez(path, **out)
 
 
@@ -99,3 +115,10 @@ def test_calls_in_a_row_equal_serial_launches(reference, s):
         if k:
             assert np.array_equal(b.cpu().numpy(), reference[f"ap{s}_{i}"])
     ctx.destroy()
+
+
+@pytest.mark.parametrize("b", range(len(BUILDS)))
+def test_algorithm_1_equals_serial_launches(reference, b):
+    for r in range(ROUNDS):
+        for name, got in build(*BUILDS[b], torch.cuda.Stream()).items():
+            assert np.array_equal(got, reference[f"build{b}_{name}"]), (r, name)

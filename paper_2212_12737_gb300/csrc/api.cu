@@ -333,10 +333,10 @@ gdml_status chol_jitter(gdml_ctx* c, const double* src, double* work, int64_t k,
     // the jitter scale tr/k must be positive (a nonzero PSD block has tr > 0); otherwise
     // no retry can help, and eps would stay 0 forever
     if (!(scale > 0.0) || !std::isfinite(scale))
-      return ctx_fail(c, GDML_ERR_NOT_SPD, "Cholesky of the inducing block failed and tr/k is not positive");
+      return ctx_fail(c, GDML_ERR_NOT_SPD, "Cholesky of the inducing block failed at column " + std::to_string(h - 1) + " and tr/k is not positive");
     eps = (eps == 0.0) ? 1e-14 * scale : eps * 10.0;
     if (!(eps <= 1e-6 * scale * 1.0000001))
-      return ctx_fail(c, GDML_ERR_NOT_SPD, "Cholesky of the inducing block failed even with jitter 1e-6 tr/k");
+      return ctx_fail(c, GDML_ERR_NOT_SPD, "Cholesky of the inducing block failed at column " + std::to_string(h - 1) + " even with jitter 1e-6 tr/k");
   }
   *eps_out = eps;
   return GDML_OK;

@@ -30,7 +30,7 @@ constexpr int kOwn = NB / kGroup;
 __global__ void __launch_bounds__(32 * kGroup) potrf_diag_kernel(double* __restrict__ A, int64_t lda, int64_t j0,
                                                                  int nb, int* __restrict__ status) {
   __shared__ double colv[2][NB];
-  __shared__ int s_bad;
+  __shared__ int s_bad[2];  // of even and odd steps, as colv: what is tested after a step's barrier is next written after the next one's
   if (*status) return;
   const int r = threadIdx.x & 31, w = threadIdx.x >> 5;
   double* row = A + (j0 + r) * lda + j0;
@@ -40,15 +40,16 @@ __global__ void __launch_bounds__(32 * kGroup) potrf_diag_kernel(double* __restr
     const int c = kGroup * q + w;
     a[q] = (r < nb && c <= r) ? row[c] : (c == r ? 1.0 : 0.0);
   }
-  if (threadIdx.x == 0) s_bad = 0;
+  if (threadIdx.x < 2) s_bad[threadIdx.x] = 0;
   __syncthreads();
+  int bad = 0;
 #pragma unroll
   for (int c = 0; c < NB; ++c) {
     double* v = colv[c & 1];
     if (w == c % kGroup) {
       const double d = __shfl_sync(0xffffffffu, a[c / kGroup], c);
       const bool ok = d > 0.0 && isfinite(d);
-      if (!ok && r == 0) s_bad = c + 1;
+      if (!ok && r == 0) s_bad[c & 1] = c + 1;
       // 1 / l and l = d / l by a correction of each other (one square root, no division)
       const double inv = rsqrt(ok ? d : 1.0), l0 = d * inv;
       const double l = fma(fma(-l0, l0, d), 0.5 * inv, l0);
@@ -56,7 +57,8 @@ __global__ void __launch_bounds__(32 * kGroup) potrf_diag_kernel(double* __restr
       v[r] = a[c / kGroup];
     }
     __syncthreads();
-    if (s_bad) break;
+    bad = s_bad[c & 1];
+    if (bad) break;
     const double x = v[r];
 #pragma unroll
     for (int q = c / kGroup; q < kOwn; ++q) {
@@ -64,8 +66,8 @@ __global__ void __launch_bounds__(32 * kGroup) potrf_diag_kernel(double* __restr
       if (cc > c) a[q] = fma(-x, v[cc], a[q]);
     }
   }
-  if (s_bad) {
-    if (threadIdx.x == 0) *status = (int)(j0 + s_bad);
+  if (bad) {
+    if (threadIdx.x == 0) *status = (int)(j0 + bad);
     return;
   }
   if (r < nb)

@@ -625,6 +625,22 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, uint32_t
   return false;
 }
 
+// one thread's bounded wait for an arrival that is under way, given up where another role has failed
+__device__ __forceinline__ bool wait_landed(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  const uint32_t addr = tc::smem_u32(bar);
+  for (uint32_t it = 0; it < tc::kSpinLimit; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(addr), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if ((it & 255) == 255 && *abort_flag) return false;
+  }
+  return false;
+}
+
 __device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
@@ -644,7 +660,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   uint64_t* tfull = empty + kMaxSlots;                         // [2] a chunk's MMAs have completed
   uint64_t* tempty = tfull + 2;                                // [2] both CTAs' epilogues have read it (leader's)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);  // raised in both CTAs
+  volatile int* peer = abort_flag + 1;  // [2] in the leader: k-blocks the other CTA copied; in the other: the leader's
+                                        // k-blocks and chunks of MMAs
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // provably uniform
   const int bn = g.bn, slots = g.slots;
   uint32_t rank;
@@ -664,6 +682,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       tc::mbar_init(&tempty[b], 2 * kEpiWarps);
     }
     *abort_flag = 0;
+    peer[0] = peer[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -676,10 +695,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync();
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  // (both words are read by the other CTA after a cluster barrier, or earlier as a hint to give up)
+  auto tell_peer = [&](volatile int* word, int x) {
+    asm volatile("st.volatile.shared::cluster.u32 [%0], %1;" ::"r"(mapa(tc::smem_u32((const void*)word), rank ^ 1u)), "r"(x) : "memory");
+  };
   auto fail_with = [&](int code) {
     atomicExch(g.err, code);
     *abort_flag = 1;
+    tell_peer(abort_flag, 1);
   };
+  int copied = 0;  // producer: k-blocks issued
 
   grid_trigger();
   grid_wait();
@@ -692,7 +717,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // ---------------- TMA producer
     const uint32_t leader0 = mapa(full0, 0), a0 = tc::smem_u32(smem), b0 = tc::smem_u32(smem_b);
     const uint32_t tx = rank == 0 ? 2u * (uint32_t)(kATile + b_bytes) : 0u;
-    int slot = 0, issued = 0;
+    int slot = 0;
     uint32_t ph = 1;
     bool ok = true;
     for (int u = u0; u < units && ok; u += du) {
@@ -705,7 +730,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (!ok) break;
         tma_load_pair(a0 + slot * kATile, mA, full0 + 8u * slot, leader0 + 8u * slot, tx, kx, ya);
         tma_load_pair(b0 + slot * b_bytes, mB, full0 + 8u * slot, leader0 + 8u * slot, 0u, kx, yb);
-        ++issued;
+        ++copied;
         if (++slot == slots) {
           slot = 0;
           ph ^= 1u;
@@ -714,12 +739,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
     if (lane == 0) {
       if (!ok) fail_with(tc::ERR_TIMEOUT_EMPTY);
-      // ok: the MMAs' arrivals on this CTA's barriers have landed before it exits; else: no copy may
-      // outlive the pair (nobody waits for the last tiles issued; the leader knows of both CTAs')
-      for (int i = max(0, issued - slots); i < issued; ++i) {
-        if (ok) (void)tc::mbar_wait_bounded(&empty[i % slots], (uint32_t)(i / slots) & 1u);
-        else if (rank == 0) (void)tc::mbar_wait_bounded(&full[i % slots], (uint32_t)(i / slots) & 1u);
-      }
+      if (rank == 1) tell_peer(peer, copied);
+      // the MMAs' arrivals on this CTA's barriers land before it exits (after a failure: see below)
+      for (int i = max(0, copied - slots); i < copied && ok; ++i) ok = wait_landed(&empty[i % slots], (uint32_t)(i / slots) & 1u, abort_flag);
+      if (!ok && !*abort_flag) fail_with(tc::ERR_TIMEOUT_DONE);
     }
     __syncwarp();
   } else if (warp == 1 && rank == 0) {
@@ -757,6 +780,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       if (!ok) fail_with(tc::ERR_TIMEOUT_FULL);
       // every MMA and commit has completed before the tensor memory is released
+      tell_peer(peer, issued);
+      tell_peer(peer + 1, chunks);
       if (issued > 0) (void)tc::mbar_wait_bounded(&empty[(issued - 1) % slots], (uint32_t)((issued - 1) / slots) & 1u);
       if (chunks > 0) (void)tc::mbar_wait_bounded(&tfull[(chunks - 1) & 1], (uint32_t)((chunks - 1) >> 1) & 1u);
     }
@@ -830,6 +855,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   tc::fence_before_sync();
   __syncthreads();
   cluster_sync();  // no CTA of the pair leaves while the other's MMAs or arrivals reach it
+  if (*abort_flag) {  // (of both CTAs, by now)  nothing in flight outlives the pair
+    if (warp == 0 && lane == 0) {
+      if (rank == 0) {  // copies of both CTAs land on the leader's barriers
+        const int theirs = peer[0], n = max(copied, theirs);
+        for (int i = max(0, n - slots); i < n; ++i) {
+          uint64_t* bar = &full[i % slots];
+          if (i >= copied) tc::mbar_expect_tx(bar, (uint32_t)(kATile + b_bytes));  // theirs alone
+          if (i >= theirs)  // theirs was never issued
+            asm volatile("mbarrier.complete_tx.shared::cta.b64 [%0], %1;" ::"r"(tc::smem_u32(bar)), "r"((uint32_t)(kATile + b_bytes)) : "memory");
+          (void)tc::mbar_wait_bounded(bar, (uint32_t)(i / slots) & 1u);
+        }
+      } else {  // the leader's commits arrive here too
+        const int n = peer[0], chunks = peer[1];
+        for (int i = max(0, n - slots); i < n; ++i) (void)tc::mbar_wait_bounded(&empty[i % slots], (uint32_t)(i / slots) & 1u);
+        for (int q = max(0, chunks - 2); q < chunks; ++q) (void)tc::mbar_wait_bounded(&tfull[q & 1], (uint32_t)(q >> 1) & 1u);
+      }
+    }
+    __syncwarp();
+    __syncthreads();
+    cluster_sync();
+  }
   if (warp == 1) {
     tc::fence_after_sync();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));

@@ -5,7 +5,9 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -39,6 +41,23 @@ int num_sms() {
   if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) v = 1;
   cache[dev].store(v, std::memory_order_relaxed);
   return v;
+}
+
+bool allow_smem_of(const void* fn, size_t bytes) {
+  if (bytes <= 32 * 1024) return true;  // (48 KB with a kernel's static share need no leave)
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> allowed;
+  std::lock_guard<std::mutex> lock(mu);
+  size_t& most = allowed[{dev, fn}];
+  if (bytes <= most) return true;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  most = bytes;
+  return true;
 }
 
 }  // namespace gdml

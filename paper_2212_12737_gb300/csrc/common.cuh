@@ -15,6 +15,14 @@ namespace gdml {
 // device; grids are sized in multiples of it.
 int num_sms();
 
+// Lets launches of `fn` on the current device take `bytes` of dynamic shared memory; false if CUDA refuses.
+// Per device, and raised only: a thread whose call needs less leaves what another one's launch relies on.
+bool allow_smem_of(const void* fn, size_t bytes);
+template <typename F>
+bool allow_smem(F* fn, size_t bytes) {
+  return allow_smem_of(reinterpret_cast<const void*>(fn), bytes);
+}
+
 // Host-side error carrier: every internal call returns a gdml_status and
 // writes a message into the context.
 struct Err {

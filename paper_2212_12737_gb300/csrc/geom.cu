@@ -702,13 +702,7 @@ static bool kcol_bulk(const int64_t* cols, int64_t ncols, const float2* X2, cons
                       const double* A, int64_t ldA, int64_t M, int N, int D, double c, double* out, int64_t ldo,
                       float2* scratch, cudaStream_t st) {
   const size_t smem = 2 * NA * (size_t)D * sizeof(float4);
-  static size_t attr = 0;
-  if (smem > 32 * 1024 && smem > attr) {
-    if (cudaFuncSetAttribute(kcol_bulk_df_kernel<NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-      return false;
-    attr = smem;
-  }
+  if (!allow_smem(kcol_bulk_df_kernel<NA>, smem)) return false;
   for (int64_t c0 = 0; c0 < ncols; c0 += kColBatch) {
     const int64_t nc = std::min<int64_t>(kColBatch, ncols - c0), LC = cdiv(nc, kColBlock) * kColBlock;
     float4* XP = reinterpret_cast<float4*>(scratch);
@@ -742,11 +736,7 @@ bool launch_kcol_df(const int64_t* cols, int64_t ncols, const float2* X2, const 
   const int64_t want = std::max<int64_t>(1, M * ncols / (2 * (int64_t)sms));
   if (want < W) W = (int)want;
   const size_t wsmem = fixed + W * per_warp;
-  static size_t attr = 0;
-  if (wsmem > 48 * 1024 && wsmem > attr) {
-    cudaFuncSetAttribute(kcol_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
-    attr = wsmem;
-  }
+  (void)allow_smem(kcol_df_kernel, wsmem);
   dim3 g((unsigned)cdiv(M, W), (unsigned)ncols);
   // stop_flag: Algorithm 1's step, which follows the previous one without waiting for it to drain
   { launch_after(stop_flag != nullptr, kcol_df_kernel, g, 32 * W, wsmem, st, cols, X2, G2, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag, released, step); count_launch(); }
@@ -814,8 +804,7 @@ void launch_backproj(const TU* U, int64_t ldU, int splits, int64_t split_stride,
                      const double* Xc, const double* G, const double* v, int64_t M, int N, int D, double lam,
                      int add_lambda, double* out, cudaStream_t st) {
   const size_t smem = D * sizeof(double);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(backproj_kernel<TU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  (void)allow_smem(backproj_kernel<TU>, smem);
   { backproj_kernel<TU><<<(unsigned)M, 128, smem, st>>>(U, ldU, splits, split_stride, rowsum, Xc, G, v, N, D,
                                                        lam, add_lambda, out); count_launch(); }
 }
@@ -839,11 +828,7 @@ void launch_kcol(const int64_t* cols, int64_t ncols, const double* X, const doub
   }
   if (W >= 1 && ncols <= 65535) {
     const size_t wsmem = fixed + W * per_warp;
-    static size_t attr = 0;
-    if (wsmem > 48 * 1024 && wsmem > attr) {
-      cudaFuncSetAttribute(kcol_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
-      attr = wsmem;
-    }
+    (void)allow_smem(kcol_warp_kernel, wsmem);
     dim3 g((unsigned)cdiv(M, W), (unsigned)ncols);
     { kcol_warp_kernel<<<g, 32 * W, wsmem, st>>>(cols, X, G, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag); count_launch(); }
     return;
@@ -851,7 +836,7 @@ void launch_kcol(const int64_t* cols, int64_t ncols, const double* X, const doub
   const int per = 8;
   dim3 grid((unsigned)M, (unsigned)cdiv(ncols, per));
   size_t smem = (2 * (size_t)D + N) * sizeof(double);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(kcol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  (void)allow_smem(kcol_kernel, smem);
   { kcol_kernel<<<grid, 128, smem, st>>>(cols, ncols, per, X, G, S, A, ldA, M, N, D, c * c, out, ldo, stop_flag); count_launch(); }
 }
 
@@ -970,7 +955,7 @@ __global__ void __launch_bounds__(256) kdiag_sym_kernel(const double* __restrict
 void launch_kdiag_sym(const double* X, const double* G, int64_t M, int N, int D, const int* pis, const int* pinv,
                       int S, double c, double* diag, cudaStream_t st) {
   const size_t smem = (size_t)D * sizeof(double);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(kdiag_sym_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  (void)allow_smem(kdiag_sym_kernel, smem);
   { kdiag_sym_kernel<<<(unsigned)M, 256, smem, st>>>(X, G, N, D, pis, pinv, S, c, diag); count_launch(); }
 }
 
@@ -1061,12 +1046,7 @@ bool launch_kcol_sym(const int64_t* cols, int64_t ncols, const double* X, const 
   const int W = (int)std::min<size_t>(8, (200 * 1024) / per_warp);
   if (W < 1 || ncols < 1 || ncols > 65535) return false;
   const size_t smem = W * per_warp;
-  static size_t attr = 0;
-  if (smem > 48 * 1024 && smem > attr) {
-    if (cudaFuncSetAttribute(kcol_sym_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return false;
-    attr = smem;
-  }
+  if (!allow_smem(kcol_sym_kernel, smem)) return false;
   dim3 g((unsigned)cdiv(M, W), (unsigned)ncols);
   { kcol_sym_kernel<<<g, 32 * W, smem, st>>>(cols, X, G, Stab, Atab, ldA, M, MB, N, D, pis, pinv, S, c * c, out, ldo, stop_flag); count_launch(); }
   return true;

@@ -1158,14 +1158,9 @@ int oz_auto_chunks_per_cta(int64_t tiles, int64_t nchunks) {
 static gdml_status oz_gemm(const OzOperand& A, const OzOperand& B, float2* out, int64_t ldo, int64_t split_stride,
                            int* err, cudaStream_t st, int G, int* groups_out = nullptr, int nlev = oz::S,
                            const OzOperand* A2 = nullptr, const OzOperand* B2 = nullptr) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    for (auto fn : {oz_gemm_kernel<1>, oz_gemm_kernel<2>, oz_gemm_kernel<3>, oz_gemm_kernel<4>, oz_gemm_kernel<5>,
-                    oz_gemm_kernel<6>, oz_gemm_kernel<7>})
-      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotalM) != cudaSuccess)
-        return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(sliced gemm)");
-    attr_set = true;
-  }
+  for (auto fn : {oz_gemm_kernel<1>, oz_gemm_kernel<2>, oz_gemm_kernel<3>, oz_gemm_kernel<4>, oz_gemm_kernel<5>,
+                  oz_gemm_kernel<6>, oz_gemm_kernel<7>})
+    if (!allow_smem(fn, kSmemTotalM)) return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(sliced gemm)");
   if (A.Kp != B.Kp) return fail(GDML_ERR_ARG, "sliced gemm: K mismatch");
   if (A.Kp % oz::KB != 0 || (A2 && A.Kp % oz::KC != 0)) return fail(GDML_ERR_ARG, "sliced gemm: K padding");
   if (nlev < 1 || nlev > oz::S) return fail(GDML_ERR_ARG, "sliced gemm: levels outside 1..7");
@@ -1287,8 +1282,7 @@ gdml_status oz_matvec(OzMatvec& oz, const double* G, const float2* G2, const dou
     nsplit2 = 2 * groups2;
   }
   const size_t smem = 3 * (size_t)D * sizeof(float2);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(oz_backproj_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  (void)allow_smem(oz_backproj_df_kernel, smem);
   { oz_backproj_df_kernel<<<(unsigned)M, 256, smem, st>>>(oz.Up, nsplit2, M, D, oz.rs2, (int)nch, oz.Xc2, G2, v, oz.N, lam, add_lambda, out); count_launch(); }
   if (cudaGetLastError() != cudaSuccess) return fail(GDML_ERR_CUDA, "sliced matvec kernels");
   return GDML_OK;

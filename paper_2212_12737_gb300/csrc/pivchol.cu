@@ -683,12 +683,8 @@ void pivchol_run_df(const PivCholArgs& a, float* L, cudaStream_t st) {
   { pc_argmax_kernel<<<arg_blocks(), kArgThreads, 0, st>>>(0, a.n, 1, a.d, a.perm, a.chosen, a.pivots, nullptr,
                                                        a.ps, a.part, a.ticket, a.posof); count_launch(); }
   if (plan.ok) {  // two launches per step: the kernel column, and Schur sums + finish beside it
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(pc_schur_finish_ws_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWsSmemN);
-      cudaFuncSetAttribute(pc_schur_finish_ws_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWsSmemN);
-      attr = true;
-    }
+    (void)allow_smem(pc_schur_finish_ws_kernel<1>, kWsSmemN);
+    (void)allow_smem(pc_schur_finish_ws_kernel<2>, kWsSmemN);
     const int64_t keep = ((int64_t)64 << 20) / (4 * a.n);
     for (int64_t m = 0; m < a.k; ++m) {
       const unsigned step = a.get_col(a.pivots + m, a.col, a.ps, (unsigned)(m + 1), st) ? (unsigned)(m + 1) : 0u;

@@ -1122,12 +1122,7 @@ static void gemm_shape(int64_t M, int64_t N, int64_t nkb, int64_t planes, int ca
 // residues of A B^T (or of both segments' products) into out
 template <bool BUILD>
 static gdml_status launch_gemm(GemmArgs& g, int segs, int chunks, bool pdl, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(rns_gemm_kernel<BUILD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
-      return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(residue gemm)");
-    attr_set = true;
-  }
+  if (!allow_smem(rns_gemm_kernel<BUILD>, kSmem)) return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(residue gemm)");
   for (int i = 0; i < rns::kMaxMod; ++i) {
     g.p[i] = (float)rns::kMods[i];
     g.inv[i] = 1.0f / (float)rns::kMods[i];
@@ -1214,10 +1209,7 @@ void rns_product_shape(RnsProduct& q, int cap) {
 
 template <typename F>
 static gdml_status big_smem(F* fn, size_t bytes) {
-  if (bytes > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-    return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(residue matvec)");
-  return GDML_OK;
+  return allow_smem(fn, bytes) ? GDML_OK : fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(residue matvec)");
 }
 
 gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, const double* Xc, const double* A, int64_t ldA,

@@ -275,12 +275,7 @@ static gdml_status launch_gemm(const CUtensorMap& mA, const CUtensorMap& mB, int
                                const Epi& epi, int* err, cudaStream_t st) {
   using SM = Smem<BN, STAGES>;
   auto kern = gemm_kernel<BF16, BN, STAGES, Epi>;
-  static bool attr_set = false;  // per instantiation
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SM::TOTAL) != cudaSuccess)
-      return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(tcgen05 gemm)");
-    attr_set = true;
-  }
+  if (!allow_smem(kern, SM::TOTAL)) return fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(tcgen05 gemm)");
   const int kb_per_split = (int)cdiv(num_kb, splits);
   splits = (int)cdiv(num_kb, kb_per_split);
   dim3 grid((unsigned)cdiv(N, BN), (unsigned)cdiv(M, BM), (unsigned)splits);
@@ -400,8 +395,7 @@ static gdml_status matvec_impl(TcMatvec& tc, const double* G, const double* v, d
   const int kb_per_split = (int)cdiv(tc.K2p / span, tc.splits2);
   const int splits = (int)cdiv(tc.K2p / span, kb_per_split);
   const size_t smem = tc.D * sizeof(float);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(tc_backproj_kernel<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  (void)allow_smem(tc_backproj_kernel<BF16>, smem);
   { tc_backproj_kernel<BF16><<<(unsigned)M, 128, smem, st>>>(tc.U, splits, M * tc.Dp, tc.Dp, tc.rs_part, (int)cdiv(M, 32), M, (const T*)tc.Xc_lp, tc.G32, v, tc.N, tc.D, lam, add_lambda, out); count_launch(); }
   if (cudaGetLastError() != cudaSuccess) return fail(GDML_ERR_CUDA, "tensor-core matvec kernels");
   return GDML_OK;

@@ -627,18 +627,9 @@ void ws_plan(WsPlan& plan, const float* L, int64_t n, int64_t k, int rows) {
   plan = WsPlan();
   if (!L || n < 4 || k < 1 || n % 4 != 0 || n > (int64_t(1) << 30) || k > (int64_t(1) << 30)) return;
   const int sms = num_sms();
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(ws_gemv_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWsSmemT) != cudaSuccess ||
-        cudaFuncSetAttribute(ws_gemv_n_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWsSmemN) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(ws_gemv_n_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWsSmemN) !=
-            cudaSuccess) {
-      (void)cudaGetLastError();
-      return;
-    }
-    attr = true;
-  }
+  if (!allow_smem(ws_gemv_t_kernel, kWsSmemT) || !allow_smem(ws_gemv_n_kernel<1>, kWsSmemN) ||
+      !allow_smem(ws_gemv_n_kernel<2>, kWsSmemN))
+    return;
   // resident CTAs per SM (two by design; fewer if the shared-memory carve-out says so)
   int occ = 0, occ_t = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ws_gemv_n_kernel<2>, kWsThreads, kWsSmemN) !=
@@ -1059,11 +1050,7 @@ static void launch_core_fused(const double* part, int64_t nchunks, int64_t k, co
                               double* t, float2* t2, double* u, float2* u2, float2* e2, unsigned* bar, int* err,
                               cudaStream_t st) {
   const size_t smem = (size_t)k * sizeof(float2);
-  static size_t attr = 0;
-  if (smem > 48 * 1024 && smem > attr) {
-    cudaFuncSetAttribute(woodbury_core_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = smem;
-  }
+  (void)allow_smem(woodbury_core_fused_kernel, smem);
   // as many CTAs as can be resident at once (at most 4 per SM): the cooperative launch needs
   // them co-resident, and more warps keep more of each phase's row loads in flight
   int per_sm = 1;

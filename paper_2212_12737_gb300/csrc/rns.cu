@@ -1,6 +1,6 @@
 // Residue-number matvec of GDML_OZAKI contexts (see rns.cuh for the scheme).  One matvec is six
 // kernels: projection (W = J v, its row residues), column residues of W, the products' residues
-// T, beta (T from its residues, beta's residues), U, back-projection.
+// T, beta (T from its residues, beta's residues), U, back-projection; the last four per panel of rows.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -506,7 +506,8 @@ static_assert(kSmem <= 227 * 1024, "shared memory per CTA");
 struct GemmArgs {
   CUtensorMap a[2], b[2];  // per K segment
   float p[rns::kMaxMod], inv[rns::kMaxMod];
-  int nmod, M, N, Ra, Rb;  // Ra, Rb: operand rows per modulus
+  int nmod, M, N, Rb;   // Ra, Rb: operand rows per modulus; row0: first row of A (per K segment)
+  int Ra[2], row0[2];
   int bn, tn, tm;
   int nkb, kb_group, groups, slabs;  // k-blocks per segment and per slab; slabs = segments x groups
   int slots;                         // of the ring
@@ -516,7 +517,6 @@ struct GemmArgs {
   int units;
   // the builds' products (BUILD)
   int shape;    // RNS_FULL, RNS_TRI, RNS_LOWER
-  int row0;     // first row of A
   int n_first;  // RNS_LOWER: column tiles of the first row of tiles
   int tiles;    // RNS_LOWER: tiles
 };
@@ -723,7 +723,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     for (int u = u0; u < units && ok; u += du) {
       const Unit x = unit_of<BUILD>(g, u);
       const CUtensorMap *mA = &g.a[x.seg], *mB = &g.b[x.seg];
-      const int ya = x.mod * g.Ra + (BUILD ? g.row0 : 0) + x.m0 + (int)rank * kBM, yb = x.mod * g.Rb + x.n0 + (int)rank * (bn >> 1);
+      const int ya = x.mod * g.Ra[x.seg] + g.row0[x.seg] + x.m0 + (int)rank * kBM, yb = x.mod * g.Rb + x.n0 + (int)rank * (bn >> 1);
       int kx = x.kb0 * kKB;
       for (int kb = 0; kb < x.nk; ++kb, kx += kKB) {
         ok = wait_bar<false>(empty0 + 8u * slot, ph, limit, abort_flag);
@@ -889,9 +889,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 // is formed twice.  Four CTAs of 256 threads per SM (64 registers, 50 bytes of spills more than at 80)
 // against three; rows that fit the chip as CTAs of 128 threads run in one round (see row_threads).
 constexpr int64_t kBetaStage = 24 * 1024;
+constexpr int64_t kPanelBytes = (int64_t)2 << 30;
 template <int NM, bool STAGE>
 __global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* Tp, int slabs, int chunks,
-                                                          int64_t M, int64_t MB, int64_t ldT,
+                                                          int64_t M, int64_t MB, int64_t ldT, int64_t Rd,
                                                           const int* __restrict__ sA, const int* sW,
                                                           const float2* __restrict__ S2, const float2* t2,
                                                           float rootMB, int64_t Kp, int bits, bf16* __restrict__ d,
@@ -931,7 +932,7 @@ __global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* Tp, in
   const int s = row_scale(m, rootMB, bits);
   if (tid == 0) sc[a] = s;
   bf16* da = d + a * Kp;
-  const int64_t dplane = M * Kp;
+  const int64_t dplane = Rd * Kp;  // (of the operand: rows of a whole panel)
   for (unsigned b = 4 * tid; b < n; b += 4 * blockDim.x) {
     const df2 zero{f2(0.f), f2(0.f)};
     float2 dx[4], dy[4];
@@ -1136,7 +1137,7 @@ static gdml_status launch_gemm(GemmArgs& g, int segs, int chunks, bool pdl, cuda
   g.slots = std::min(kMaxSlots, kRing / (kATile + g.bn * 64));
   int64_t tiles = (int64_t)g.tm * g.tn;
   if (BUILD && g.shape == RNS_LOWER) {
-    g.n_first = g.row0 / (2 * kBM) + 1;
+    g.n_first = g.row0[0] / (2 * kBM) + 1;
     tiles = 0;
     for (int m = 0; m < g.tm; ++m) tiles += g.n_first + m;
     g.tiles = (int)tiles;
@@ -1152,14 +1153,17 @@ static gdml_status launch_gemm(GemmArgs& g, int segs, int chunks, bool pdl, cuda
   return GDML_OK;
 }
 
-static gdml_status rns_gemm(const RnsOperand* A, const RnsOperand* B, int segs, int bn, int chunks,
-                            uint16_t* out, int64_t ldo, int* err, bool pdl, cudaStream_t st, int* slabs_out) {
+// rows row0[s] .. row0[s] + M of segment s's A
+static gdml_status rns_gemm(const RnsOperand* A, const RnsOperand* B, const int64_t* row0, int64_t M, int segs, int bn,
+                            int chunks, uint16_t* out, int64_t ldo, int* err, bool pdl, cudaStream_t st, int* slabs_out) {
   GemmArgs g{};
   for (int s = 0; s < 2; ++s) {
     g.a[s] = A[s < segs ? s : 0].map;
     g.b[s] = B[s < segs ? s : 0].map;
+    g.Ra[s] = (int)A[s < segs ? s : 0].rows;
+    g.row0[s] = (int)row0[s < segs ? s : 0];
   }
-  g.M = g.Ra = (int)A[0].rows;
+  g.M = (int)M;
   g.N = g.Rb = (int)B[0].rows;
   g.bn = bn;
   g.nkb = (int)(A[0].Kp / kKB);
@@ -1181,7 +1185,7 @@ gdml_status rns_product(RnsProduct& q, int* err, cudaStream_t st) {
   g.b[1] = g.b[0];
   g.M = (int)q.M;
   g.N = (int)q.N;
-  g.Ra = (int)q.Ra;
+  g.Ra[0] = (int)q.Ra;
   g.Rb = (int)q.Rb;
   g.bn = q.bn;
   g.nkb = (int)(q.Kp / kKB);
@@ -1189,7 +1193,7 @@ gdml_status rns_product(RnsProduct& q, int* err, cudaStream_t st) {
   g.out = q.out;
   g.err = err;
   g.shape = q.shape;
-  g.row0 = (int)q.row0;
+  g.row0[0] = (int)q.row0;
   return launch_gemm<true>(g, 1, q.chunks, false, st);
 }
 
@@ -1235,15 +1239,23 @@ gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, co
   auto slab_cap = [](int64_t entries, int64_t nch) {
     return (int)std::max<int64_t>(cdiv(nch, kMaxChunks), std::min<int64_t>(std::min<int64_t>(nch, 4), ((int64_t)1 << 29) / (2 * NM * std::max<int64_t>(entries, 1))));
   };
-  r.cap1 = slab_cap(M * r.ldT, r.nch1);
-  r.cap2 = slab_cap(2 * M * r.ldU, r.nch2);
-  gemm_shape(M, MB, cdiv(D, kKB), NM, r.cap1, &r.bn1, &r.g1);
-  gemm_shape(M, D + 1, cdiv(MB, kKB), 2 * NM, r.cap2, &r.bn2, &r.g2);
+  // T, beta and U exist for a panel of rows at a time: 56 bytes per pair of rows and training rows, which
+  // with the 68 that stay (S, [A | beta] and T in FP64, c^2 S, A's residues) would be more than the 76 of
+  // sliced operands; within kPanelBytes (M = 6,100 at D = 210) all rows are one panel
+  {
+    const int64_t row = 2 * NM * (cdiv(r.nch1, kMaxChunks) * r.ldT + cdiv(MB, kKB) * kKB + 2 * cdiv(r.nch2, kMaxChunks) * r.ldU);
+    const int64_t fit = std::max<int64_t>(1, kPanelBytes / row / 256) * 256;
+    r.P = M <= fit ? M : cdiv(cdiv(M, cdiv(M, fit)), 256) * 256;
+  }
+  r.cap1 = slab_cap(r.P * r.ldT, r.nch1);
+  r.cap2 = slab_cap(2 * r.P * r.ldU, r.nch2);
+  gemm_shape(r.P, MB, cdiv(D, kKB), NM, r.cap1, &r.bn1, &r.g1);
+  gemm_shape(r.P, D + 1, cdiv(MB, kKB), 2 * NM, r.cap2, &r.bn2, &r.g2);
   RNS_TRY(make_operand(r, r.Xc1, M, D, kBM, st));
   RNS_TRY(make_operand(r, r.W1, MB, D, r.bn1 / 2, st));
   RNS_TRY(make_operand(r, r.A2, M, MB, kBM, st));
   RNS_TRY(make_operand(r, r.WT2, D + 1, MB, r.bn2 / 2, st));  // row D: zeros
-  RNS_TRY(make_operand(r, r.B2, M, MB, kBM, st));
+  RNS_TRY(make_operand(r, r.B2, r.P, MB, kBM, st));
   RNS_TRY(make_operand(r, r.XT2, D + 1, MB, r.bn2 / 2, st));  // row D: ones
   RNS_TRY(rns_alloc(r, &r.G3, (size_t)(3 * M * r.Dp), st));
   RNS_TRY(rns_alloc(r, &r.Xc2, (size_t)(M * r.Dp), st));
@@ -1251,8 +1263,8 @@ gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, co
   RNS_TRY(rns_alloc(r, &r.colmax, (size_t)(kColCopies * r.Dp), st));
   RNS_TRY(rns_alloc(r, &r.t2, (size_t)r.ldT, st));
   RNS_TRY(rns_alloc(r, &r.S2, (size_t)(M * r.ldT), st));
-  RNS_TRY(rns_alloc(r, &r.Tp, (size_t)(r.cap1 * NM * M * r.ldT), st));
-  RNS_TRY(rns_alloc(r, &r.Up, (size_t)(2 * r.cap2 * NM * M * r.ldU), st));
+  RNS_TRY(rns_alloc(r, &r.Tp, (size_t)(r.cap1 * NM * r.P * r.ldT), st));
+  RNS_TRY(rns_alloc(r, &r.Up, (size_t)(2 * r.cap2 * NM * r.P * r.ldU), st));
   RNS_TRY(rns_alloc(r, &r.JX, (size_t)(3 * M * N), st));
   RNS_TRY(rns_alloc(r, &r.err, 1, st));
   if (Ssym > 1) {
@@ -1326,27 +1338,28 @@ gdml_status rns_matvec(RnsMatvec& r, const double* G, const double* Xc, const do
     { rns_proj_kernel<NM><<<(unsigned)M, nt, sm, st>>>((const float4*)r.G3, (const float4*)r.Xc2, (const uint2*)r.ij, v, M, r.N, r.Dp, rootD, (float4*)r.Wf, r.t2, r.W1.Kp, bits, r.W1.d, r.W1.s, r.colmax); count_launch(); }
     { launch_after(pdl, rns_cols_kernel<NM, float2>, gc, 256, 0, st, r.Wf, MB, D, r.Dp, r.colmax, r.WT2.Kp, D + 1, bits, r.WT2.d, r.WT2.s); count_launch(); }
   }
-  int s1 = 0, s2 = 0;
-  RNS_TRY(rns_gemm(&r.Xc1, &r.W1, 1, r.bn1, rns_chunks(r.nch1, r.g1, r.cap1), r.Tp, r.ldT, r.err, pdl, st, &s1));
-  const int nr = row_threads(M, cdiv(MB, 2), MB <= kBetaStage ? (size_t)r.ldT * sizeof(float2) : 0);
-  if (MB <= kBetaStage) {
-    const size_t sm = (size_t)r.ldT * sizeof(float2);
-    RNS_TRY(big_smem(rns_beta_kernel<NM, true>, sm));
-    { launch_after(pdl, rns_beta_kernel<NM, true>, (unsigned)M, nr, sm, st, r.Tp, s1, (int)r.nch1, M, MB, r.ldT, r.Xc1.s, r.W1.s, r.S2, r.t2, rootMB, r.B2.Kp, bits, r.B2.d, r.B2.s); count_launch(); }
-  } else {
-    { launch_after(pdl, rns_beta_kernel<NM, false>, (unsigned)M, nr, 0, st, r.Tp, s1, (int)r.nch1, M, MB, r.ldT, r.Xc1.s, r.W1.s, r.S2, r.t2, rootMB, r.B2.Kp, bits, r.B2.d, r.B2.s); count_launch(); }
-  }
-  const RnsOperand a[2] = {r.A2, r.B2}, b[2] = {r.WT2, r.XT2};
-  RNS_TRY(rns_gemm(a, b, 2, r.bn2, rns_chunks(r.nch2, r.g2, r.cap2), r.Up, r.ldU, r.err, pdl, st, &s2));
-  const size_t sm = 3 * (size_t)r.Dp * sizeof(float2);
-  const int nb = row_threads(M, cdiv(D + 1, 2), sm);
-  int lanes = 4;  // per atom in the last step: as many as the threads give, up to 16
-  while (lanes < 16 && 2 * lanes * r.N <= nb) lanes *= 2;
+  const size_t beta_sm = MB <= kBetaStage ? (size_t)r.ldT * sizeof(float2) : 0, back_sm = 3 * (size_t)r.Dp * sizeof(float2);
+  auto* beta = MB <= kBetaStage ? rns_beta_kernel<NM, true> : rns_beta_kernel<NM, false>;
   const bool wide = r.nch2 > rns::kSumChunks;
   const int per_sum = rns::kSumChunks / rns_chunks(r.nch2, r.g2, r.cap2);
   auto* backproj = wide ? rns_backproj_kernel<NM, true> : rns_backproj_kernel<NM, false>;
-  RNS_TRY(big_smem(backproj, sm));
-  { launch_after(pdl, backproj, (unsigned)M, nb, sm, st, r.Up, s2, per_sum, (int)r.nch2, M, D, r.Dp, r.ldU, r.A2.s, r.WT2.s, r.B2.s, r.XT2.s, r.JX, (const float4*)r.G3, v, r.N, lam, add_lambda, lanes, r.colmax, out); count_launch(); }
+  RNS_TRY(big_smem(beta, beta_sm));
+  RNS_TRY(big_smem(backproj, back_sm));
+  for (int64_t a0 = 0; a0 < M; a0 += r.P) {  // panels of rows
+    const int64_t rows = std::min(r.P, M - a0);
+    int s1 = 0, s2 = 0;
+    RNS_TRY(rns_gemm(&r.Xc1, &r.W1, &a0, rows, 1, r.bn1, rns_chunks(r.nch1, r.g1, r.cap1), r.Tp, r.ldT, r.err, pdl, st, &s1));
+    const int nr = row_threads(rows, cdiv(MB, 2), beta_sm);
+    { launch_after(pdl, beta, (unsigned)rows, nr, beta_sm, st, r.Tp, s1, (int)r.nch1, rows, MB, r.ldT, r.P, r.Xc1.s + a0, r.W1.s, r.S2 + a0 * r.ldT, r.t2, rootMB, r.B2.Kp, bits, r.B2.d, r.B2.s); count_launch(); }
+    const RnsOperand a[2] = {r.A2, r.B2}, b[2] = {r.WT2, r.XT2};
+    const int64_t row0[2] = {a0, 0};
+    RNS_TRY(rns_gemm(a, b, row0, rows, 2, r.bn2, rns_chunks(r.nch2, r.g2, r.cap2), r.Up, r.ldU, r.err, pdl, st, &s2));
+    const int nb = row_threads(rows, cdiv(D + 1, 2), back_sm);
+    int lanes = 4;  // per atom in the last step: as many as the threads give, up to 16
+    while (lanes < 16 && 2 * lanes * r.N <= nb) lanes *= 2;
+    const int64_t c0 = a0 * 3 * r.N;
+    { launch_after(pdl, backproj, (unsigned)rows, nb, back_sm, st, r.Up, s2, per_sum, (int)r.nch2, rows, D, r.Dp, r.ldU, r.A2.s + a0, r.WT2.s, r.B2.s, r.XT2.s, r.JX + c0, (const float4*)(r.G3 + a0 * 3 * r.Dp), v + c0, r.N, lam, add_lambda, lanes, r.colmax, out + c0); count_launch(); }
+  }
   if (cudaGetLastError() != cudaSuccess) return fail(GDML_ERR_CUDA, "residue matvec kernels");
   return GDML_OK;
 }

@@ -149,7 +149,7 @@ struct RnsMatvec {
   RnsOperand W1;   //             B, per matvec
   RnsOperand A2;   // U = A W + beta Xc: A of the first product, fixed
   RnsOperand WT2;  //                    B of the first product, per matvec
-  RnsOperand B2;   //                    A of the second (beta), per matvec
+  RnsOperand B2;   //                    A of the second (beta), per panel
   RnsOperand XT2;  //                    B of the second, fixed
   double* W = nullptr;      // M x D, MB x D: FP64 projections (S > 1)
   double* WB = nullptr;
@@ -162,8 +162,9 @@ struct RnsMatvec {
   float2* Xc2 = nullptr;    // [M][Dp] the centred descriptors
   float2* t2 = nullptr;     // t_b = xc_b . w_b over the mantissa of P
   float2* S2 = nullptr;     // M x ldT: c^2 S_ab times the mantissa of P
-  uint16_t* Tp = nullptr;   // [slab][modulus][M][ldT] residues of T: sums over the chunks of residue + 256
-  uint16_t* Up = nullptr;   // [slab of A W | slab of beta Xc][modulus][M][ldU]
+  int64_t P = 0;            // rows per panel: T, beta and U exist for these only (M, or a multiple of 256)
+  uint16_t* Tp = nullptr;   // [slab][modulus][P][ldT] residues of T: sums over the chunks of residue + 256
+  uint16_t* Up = nullptr;   // [slab of A W | slab of beta Xc][modulus][P][ldU]
   float2* JX = nullptr;     // 3 N M: J_a^T xc_a
   int64_t ldT = 0, ldU = 0;
   int bn1 = 256, bn2 = 256;     // columns per tile of the two products

@@ -72,3 +72,36 @@ def test_more_chunks_than_a_16_bit_sum_holds(M, equal):
     MB = M * len(perms)
     print(f"M={M} S={len(perms)} chunks={-(-MB // 512)}: {err:.2e}")
     assert err <= 8 * 2.0 ** -48 + (16 + np.sqrt(2 * MB)) * EPS
+
+
+@pytest.mark.parametrize("N,M", [(5, 9501), (3, 6400)])
+def test_panels_of_rows(N, M):
+    """T, beta and U of more rows than one panel holds (the last panel ragged), against FP64."""
+    R = dev(synth.geometries(synth.template(N, 5), M, 0.1, 6))
+    v = dev(np.random.default_rng(M).standard_normal(3 * N * M))
+    ctx = gdml.kernel_setup(R, 3.0, 1e-6, precision="ozaki")
+    got, again = ctx.matvec(v), ctx.matvec(v)
+    ctx.tc_check()
+    ctx.destroy()
+    f64 = gdml.kernel_setup(R, 3.0, 1e-6, precision="fp64")
+    ref = f64.matvec(v)
+    f64.destroy()
+    err = rel(got, ref)
+    print(f"N={N} M={M}: {err:.2e}")
+    assert torch.equal(got, again)
+    assert err <= 8 * 2.0 ** -48 + (16 + np.sqrt(2 * M)) * EPS
+
+
+def test_memory_per_pair_of_geometries():
+    """A plain context of short descriptors holds 76 bytes per pair of geometries at most (the sliced
+    form's), so that one of 60,000 geometries fits the card."""
+    N, M = 4, 30000
+    R = dev(synth.geometries(synth.template(N, 5), M, 0.1, 6))
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    ctx = gdml.kernel_setup(R, 3.0, 1e-6, precision="ozaki")
+    held = before - torch.cuda.mem_get_info()[0]
+    ctx.destroy()
+    print(f"{held / M ** 2:.1f} bytes per pair")
+    assert held <= 76 * M * M + 2 ** 28

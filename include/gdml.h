@@ -269,10 +269,13 @@ gdml_status gdml_set_inner_rtol(gdml_ctx* ctx, double inner_rtol);
  * levels < 7 cuts every 256-entry chunk of an operand row into BF16 slices of 7 bits and keeps only
  * the slice pairs i + j < levels (slices counted from 0) in both contractions (21, 15, 10 products
  * for 6, 5, 4 levels): a matvec error of roughly 2^-(7 levels - 2) relative to |K||v| instead of
- * ~1e-14.  The first call with levels < 7 sets up that form's operands.  The recurrence then
+ * ~1e-14.  The first call with levels < 7 sets up that form's operands, beside the full product's or,
+ * where the device does not hold both, in their place: the full product (gdml_matvec) is then the sliced
+ * one with all 7 levels (28 products, ~1e-14), and a caller's graph that captured calls on this context
+ * has to be captured anew.  The recurrence then
  * solves a slightly perturbed system; gdml_pcg_solve recomputes the true residual with the FP64
  * matvec whenever the recurrence passes and restarts PCG from alpha (at most 10 times), so the
- * reported residual is the FP64 one.  gdml_matvec and the build are not affected.
+ * reported residual is the FP64 one.  gdml_matvec (but for that) and the build are not affected.
  * Errors: GDML_ERR_ARG (not an OZAKI context, levels outside 1..7), GDML_ERR_OOM, GDML_ERR_CUDA. */
 gdml_status gdml_set_inner_levels(gdml_ctx* ctx, int32_t levels);
 

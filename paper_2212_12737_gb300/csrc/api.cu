@@ -249,14 +249,16 @@ gdml_status matvec_df(gdml_ctx* c, const double* v, double* out, int add_lambda)
   return check_launch(c, "matvec_df");
 }
 
-// lev: slice levels of an OZAKI context's matvec (7: the full, FP64-class product)
+// lev: slice levels of an OZAKI context's matvec (7: the full, FP64-class product, by residues unless
+// their operands have given way to the sliced ones: see set_up_slices)
 gdml_status matvec_any(gdml_ctx* c, const double* v, double* out, int add_lambda, bool force_fp64, int lev = 7) {
   if (force_fp64 || c->precision == GDML_FP64) return matvec_fp64(c, v, out, add_lambda);
   if (c->precision == GDML_DF64) return matvec_df(c, v, out, add_lambda);
   if (c->precision == GDML_OZAKI) {
-    gdml_status s = lev == 7 ? rns_matvec(c->rn, c->G, c->Xc(), v, out, add_lambda, c->lam, c->st)
+    const bool residues = lev == 7 && c->rn.ready;
+    gdml_status s = residues ? rns_matvec(c->rn, c->G, c->Xc(), v, out, add_lambda, c->lam, c->st)
                              : oz_matvec(c->oz, c->G, c->G2, c->Xc(), v, out, add_lambda, c->lam, c->st, lev);
-    if (s != GDML_OK) return ctx_fail(c, s, "sliced tensor-core matvec: " + last_msg());
+    if (s != GDML_OK) return ctx_fail(c, s, (residues ? "residue matvec: " : "sliced tensor-core matvec: ") + last_msg());
     return check_launch(c, "matvec_oz");
   }
   gdml_status s = tc_matvec(c->tc, c->G, v, out, add_lambda, c->lam, c->st);
@@ -839,11 +841,41 @@ gdml_status setup_impl(gdml_ctx** out, const double* R_dev, int64_t M, int32_t N
   if (precision == GDML_OZAKI) {
     gdml_status s = rns_setup(c->rn, M, N, (int)D, c->G, c->XcA, c->P64, 2 * MB, c->S, c->c, c->st, c->Ssym, c->pis,
                               c->XcB());
-    if (s != GDML_OK) return ctx_fail(C, s, "sliced tensor-core setup: " + last_msg());
+    if (s != GDML_OK) return ctx_fail(C, s, "residue matvec setup: " + last_msg());
   }
   CTRY(C, cudaStreamSynchronize(c->st));
   *out = c.release();
   return GDML_OK;
+}
+
+// The sliced operands that a reduced number of levels reads, beside the residues; where the device does not
+// hold both, in their place (the full product is then the sliced one with all 7 levels).
+gdml_status set_up_slices(gdml_ctx* c) {
+  auto slices = [c]() {
+    gdml_status s = oz_setup(c->oz, c->M, c->N, c->D, c->XcA, c->P64, 2 * c->MB, c->S, c->c, c->st, c->Ssym, c->pis,
+                             c->XcB());
+    if (s != GDML_OK) {
+      cudaStreamSynchronize(c->st);
+      oz_destroy(c->oz);
+      c->oz = OzMatvec();
+    }
+    return s;
+  };
+  gdml_status s = slices();
+  if (s != GDML_ERR_OOM || !c->rn.ready) return s;
+  drop_graphs(c);
+  CTRY(c, cudaStreamSynchronize(c->st));
+  rns_destroy(c->rn);
+  c->rn = RnsMatvec();
+  s = slices();
+  if (s != GDML_OK) {  // as it was
+    const std::string why = last_msg();
+    const gdml_status back = rns_setup(c->rn, c->M, c->N, c->D, c->G, c->XcA, c->P64, 2 * c->MB, c->S, c->c, c->st,
+                                       c->Ssym, c->pis, c->XcB());
+    if (back != GDML_OK) return back;
+    fail(s, why);
+  }
+  return s;
 }
 
 }  // namespace
@@ -1203,13 +1235,8 @@ gdml_status gdml_set_inner_levels(gdml_ctx* c, int32_t levels) {
   if (c->precision != GDML_OZAKI) return ctx_fail(c, GDML_ERR_ARG, "inner levels apply to OZAKI contexts only");
   if (levels < 1 || levels > 7) return ctx_fail(c, GDML_ERR_ARG, "inner levels must be in 1..7");
   if (levels < 7 && !c->oz.ready) {  // the sliced operands, which only this operator reads
-    gdml_status s = oz_setup(c->oz, c->M, c->N, c->D, c->XcA, c->P64, 2 * c->MB, c->S, c->c, c->st, c->Ssym, c->pis,
-                             c->XcB());
-    if (s != GDML_OK) {
-      oz_destroy(c->oz);
-      c->oz = OzMatvec();
-      return ctx_fail(c, s, "sliced tensor-core setup: " + last_msg());
-    }
+    gdml_status s = set_up_slices(c);
+    if (s != GDML_OK) return ctx_fail(c, s, "sliced tensor-core setup: " + last_msg());
   }
   if (levels != c->inner_lev) drop_graphs(c);  // the captured loop bakes the GEMMs' level count in
   c->inner_lev = levels;
@@ -1610,7 +1637,10 @@ gdml_status gdml_autotune(gdml_ctx* c, int32_t* choice_out) {
   CTRY(c, cudaEventCreate(&e0));
   CTRY(c, cudaEventCreate(&e1));
   if (c->precision == GDML_OZAKI) {
-    // the residue products' 512-entry K chunks per unit (T = Xc W^T, U = A W + beta Xc)
+    // the residue products' 512-entry K chunks per unit (T = Xc W^T, U = A W + beta Xc), or the sliced
+    // ones' 256-entry chunks per CTA
+    int& c1 = c->rn.ready ? c->rn.g1 : c->oz.g1;
+    int& c2 = c->rn.ready ? c->rn.g2 : c->oz.g2;
     auto time_mv = [&](float* ms) -> gdml_status {
       for (int w = 0; w < 2; ++w) TRY(matvec_any(c, v, out, 1, false));
       CTRY(c, cudaEventRecord(e0, c->st));
@@ -1620,16 +1650,16 @@ gdml_status gdml_autotune(gdml_ctx* c, int32_t* choice_out) {
       cudaEventElapsedTime(ms, e0, e1);
       return GDML_OK;
     };
-    const int n1 = (int)c->rn.nch1, n2 = (int)c->rn.nch2;
+    const int n1 = (int)(c->rn.ready ? c->rn.nch1 : c->oz.W1.nchunks), n2 = (int)(c->rn.ready ? c->rn.nch2 : c->oz.nch2);
     std::vector<int> cand2;
     for (int g = 1; g <= n2; g = g < 4 ? g + 1 : g * 2) cand2.push_back(g);
     if (cand2.back() != n2) cand2.push_back(n2);
-    int best1 = c->rn.g1, best2 = c->rn.g2;
+    int best1 = c1, best2 = c2;
     float best_ms = 1e30f;
     for (int g1 : {1, n1}) {
       for (int g2 : cand2) {
-        c->rn.g1 = g1;
-        c->rn.g2 = g2;
+        c1 = g1;
+        c2 = g2;
         float ms = 0.f;
         gdml_status ts = time_mv(&ms);
         if (ts != GDML_OK) {
@@ -1647,8 +1677,8 @@ gdml_status gdml_autotune(gdml_ctx* c, int32_t* choice_out) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    c->rn.g1 = best1;
-    c->rn.g2 = best2;
+    c1 = best1;
+    c2 = best2;
     drop_graphs(c);
     if (choice_out) *choice_out = best1 * 65536 + best2;
     return GDML_OK;
@@ -1690,8 +1720,13 @@ gdml_status gdml_set_tuning(gdml_ctx* c, int32_t splits) {
     const int64_t n1 = cdiv(c->D, 256), n2 = cdiv(c->MB, 256), max2 = cdiv(c->MB, 128) % 2 == 0 ? 2 * n2 : n2;
     if (g1 < 1 || g1 > n1 || g2 < 1 || g2 > max2)
       return ctx_fail(c, GDML_ERR_ARG, "chunks per unit out of range");
-    c->rn.g1 = g1;
-    c->rn.g2 = g2;
+    if (c->rn.ready) {
+      c->rn.g1 = g1;
+      c->rn.g2 = g2;
+    } else {
+      c->oz.g1 = g1;
+      c->oz.g2 = g2;
+    }
     drop_graphs(c);
     return GDML_OK;
   }

@@ -105,3 +105,34 @@ def test_memory_per_pair_of_geometries():
     ctx.destroy()
     print(f"{held / M ** 2:.1f} bytes per pair")
     assert held <= 76 * M * M + 2 ** 28
+
+
+def test_reduced_levels_where_both_forms_do_not_fit():
+    """The sliced operands of reduced levels take the residues' place when the device has no room for both:
+    matvec, solve and autotuner go on, and back at 7 levels the matvec is FP64-class."""
+    N, M = 6, 8000  # residues: 2.3 GB and panels of 2 GB; slices: 2.8 GB
+    tmpl = synth.template(N, 5)
+    Rh = synth.geometries(tmpl, M, 0.1, 6)
+    R, y = dev(Rh), dev(synth.morse_forces(Rh, tmpl).reshape(-1))
+    v = dev(np.random.default_rng(7).standard_normal(Rh.size))
+    ctx = gdml.kernel_setup(R, 3.0, 1.0, precision="ozaki")
+    ref = ctx.matvec_fp64(v)
+    before = ctx.matvec(v)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (3 << 29), dtype=torch.uint8, device="cuda")
+    ctx.set_inner_levels(5)
+    bound = 8 * 2.0 ** -48 + (16 + np.sqrt(2 * M)) * EPS
+    after = ctx.matvec(v)
+    assert rel(before, ref) <= bound and rel(after, ref) <= bound
+    alpha, _, res, _ = ctx.pcg_solve(y, rtol=1e-8)
+    assert res <= 1e-8
+    ctx.set_inner_levels(7)
+    ctx.autotune()
+    assert rel(ctx.matvec(v), ref) <= bound
+    r = y - ctx.matvec_fp64(alpha)
+    assert torch.linalg.norm(r) <= 2e-8 * torch.linalg.norm(y)
+    ctx.tc_check()
+    ctx.destroy()
+    del fill
+    torch.cuda.empty_cache()

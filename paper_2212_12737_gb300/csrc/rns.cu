@@ -889,7 +889,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 // is formed twice.  Four CTAs of 256 threads per SM (64 registers, 50 bytes of spills more than at 80)
 // against three; rows that fit the chip as CTAs of 128 threads run in one round (see row_threads).
 constexpr int64_t kBetaStage = 24 * 1024;
-constexpr int64_t kPanelBytes = (int64_t)2 << 30;
+// Bytes of T, beta and U at a time.  With 2 GB the rounds of units that end each panel cost 4 to 9 % at M = 8,000 to
+// 20,000 (12,000 rows, D = 210: 4.41 -> 4.83 ms)
+constexpr int64_t kPanelBytes = (int64_t)8 << 30;
 template <int NM, bool STAGE>
 __global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* Tp, int slabs, int chunks,
                                                           int64_t M, int64_t MB, int64_t ldT, int64_t Rd,
@@ -1241,7 +1243,7 @@ gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, co
   };
   // T, beta and U exist for a panel of rows at a time: 56 bytes per pair of rows and training rows, which
   // with the 68 that stay (S, [A | beta] and T in FP64, c^2 S, A's residues) would be more than the 76 of
-  // sliced operands; within kPanelBytes (M = 6,100 at D = 210) all rows are one panel
+  // sliced operands; within kPanelBytes (M = 12,300 at D = 210) all rows are one panel
   {
     const int64_t row = 2 * NM * (cdiv(r.nch1, kMaxChunks) * r.ldT + cdiv(MB, kKB) * kKB + 2 * cdiv(r.nch2, kMaxChunks) * r.ldU);
     const int64_t fit = std::max<int64_t>(1, kPanelBytes / row / 256) * 256;

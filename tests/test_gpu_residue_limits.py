@@ -74,7 +74,7 @@ def test_more_chunks_than_a_16_bit_sum_holds(M, equal):
     assert err <= 8 * 2.0 ** -48 + (16 + np.sqrt(2 * MB)) * EPS
 
 
-@pytest.mark.parametrize("N,M", [(5, 9501), (3, 6400)])
+@pytest.mark.parametrize("N,M", [(5, 16001), (3, 12800)])
 def test_panels_of_rows(N, M):
     """T, beta and U of more rows than one panel holds (the last panel ragged), against FP64."""
     R = dev(synth.geometries(synth.template(N, 5), M, 0.1, 6))
@@ -95,7 +95,7 @@ def test_panels_of_rows(N, M):
 def test_memory_per_pair_of_geometries():
     """A plain context of short descriptors holds 76 bytes per pair of geometries at most (the sliced
     form's), so that one of 60,000 geometries fits the card."""
-    N, M = 4, 30000
+    N, M = 4, 36000
     R = dev(synth.geometries(synth.template(N, 5), M, 0.1, 6))
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
@@ -110,7 +110,7 @@ def test_memory_per_pair_of_geometries():
 def test_reduced_levels_where_both_forms_do_not_fit():
     """The sliced operands of reduced levels take the residues' place when the device has no room for both:
     matvec, solve and autotuner go on, and back at 7 levels the matvec is FP64-class."""
-    N, M = 6, 8000  # residues: 2.3 GB and panels of 2 GB; slices: 2.8 GB
+    N, M = 6, 8000  # residues: 2.3 GB, T, beta and U 3.6 GB; slices: 2.8 GB
     tmpl = synth.template(N, 5)
     Rh = synth.geometries(tmpl, M, 0.1, 6)
     R, y = dev(Rh), dev(synth.morse_forces(Rh, tmpl).reshape(-1))

@@ -79,12 +79,16 @@ __global__ void __launch_bounds__(32 * kGroup) potrf_diag_kernel(double* __restr
 }
 
 // x <- x L^-T for the row x spread over four neighbouring lanes (lane g: entries g, g + 4, ...); inv: the
-// reciprocals of L's diagonal
+// reciprocals of L's diagonal, whose product with x is corrected to the rounded quotient (a division takes
+// ten times the operations)
 __device__ __forceinline__ void solve_row(double (&x)[kOwn], const double (&L)[NB][NB + 1], const double* inv) {
   const int g = threadIdx.x & (kGroup - 1), first = (threadIdx.x & 31) & ~(kGroup - 1);
 #pragma unroll
   for (int c = 0; c < NB; ++c) {  // column by column: the updates of the later ones are independent
-    if (g == c % kGroup) x[c / kGroup] *= inv[c];
+    if (g == c % kGroup) {
+      const double q = x[c / kGroup] * inv[c];
+      x[c / kGroup] = fma(fma(-q, L[c][c], x[c / kGroup]), inv[c], q);
+    }
     const double xc = __shfl_sync(0xffffffffu, x[c / kGroup], first + c % kGroup);
 #pragma unroll
     for (int q = c / kGroup; q < kOwn; ++q) {

@@ -1282,10 +1282,14 @@ gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, co
   };
   fixed(Xc, D, r.Xc1);
   fixed(A, ldA, r.A2);
-  double* XT = nullptr;
-  if (cudaMalloc(&XT, (size_t)(MB * (D + 1)) * sizeof(double)) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return fail(GDML_ERR_OOM, "residue set-up scratch");
+  // the transposed descriptors go where T's residues will be, if these take more room
+  double *XT = reinterpret_cast<double*>(r.Tp), *own = nullptr;
+  if ((size_t)(r.cap1 * NM * r.P * r.ldT) * sizeof(uint16_t) < (size_t)(MB * (D + 1)) * sizeof(double)) {
+    if (cudaMalloc(&own, (size_t)(MB * (D + 1)) * sizeof(double)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return fail(GDML_ERR_OOM, "residue set-up scratch");
+    }
+    XT = own;
   }
   { rns_transpose_kernel<<<dim3((unsigned)cdiv(D + 1, 32), (unsigned)cdiv(MB, 32)), dim3(32, 8), 0, st>>>(r.XcB, MB, D, XT); count_launch(); }
   fixed(XT, MB, r.XT2);  // D + 1 rows
@@ -1294,7 +1298,7 @@ gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, co
   constexpr rns::Crt<NM> C{};
   { rns_s2_kernel<<<(unsigned)cdiv(M * MB, 256), 256, 0, st>>>(S, M, MB, r.ldT, c * c * ((double)C.pih + (double)C.pil), r.S2); count_launch(); }
   const bool bad = cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess;
-  cudaFree(XT);
+  if (own) cudaFree(own);
   if (bad) return fail(GDML_ERR_CUDA, "residue setup kernels");
   r.ready = true;
   return GDML_OK;

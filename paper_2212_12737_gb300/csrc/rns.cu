@@ -889,9 +889,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 // is formed twice.  Four CTAs of 256 threads per SM (64 registers, 50 bytes of spills more than at 80)
 // against three; rows that fit the chip as CTAs of 128 threads run in one round (see row_threads).
 constexpr int64_t kBetaStage = 24 * 1024;
-// Bytes of T, beta and U at a time.  With 2 GB the rounds of units that end each panel cost 4 to 9 % at M = 8,000 to
-// 20,000 (12,000 rows, D = 210: 4.41 -> 4.83 ms)
-constexpr int64_t kPanelBytes = (int64_t)8 << 30;
 template <int NM, bool STAGE>
 __global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* Tp, int slabs, int chunks,
                                                           int64_t M, int64_t MB, int64_t ldT, int64_t Rd,
@@ -1218,6 +1215,10 @@ static gdml_status big_smem(F* fn, size_t bytes) {
   return allow_smem(fn, bytes) ? GDML_OK : fail(GDML_ERR_CUDA, "cudaFuncSetAttribute(residue matvec)");
 }
 
+// Bytes of T, beta and U at a time.  With 2 GB the rounds of units that end each panel cost 4 to 9 % at M = 8,000 to
+// 20,000 (12,000 rows, D = 210: 4.41 -> 4.83 ms)
+constexpr int64_t kPanelBytes = (int64_t)8 << 30;
+
 gdml_status rns_setup(RnsMatvec& r, int64_t M, int N, int D, const double* G, const double* Xc, const double* A, int64_t ldA,
                       const double* S, double c, cudaStream_t st, int Ssym, const int* pis, const double* XcB) {
   constexpr int NM = rns::kMvMods;
@@ -1332,25 +1333,25 @@ gdml_status rns_matvec(RnsMatvec& r, const double* G, const double* Xc, const do
   const bool pdl = chained(M, st);
   const float rootD = std::sqrt((float)D) * 1.0001f, rootMB = std::sqrt((float)MB) * 1.0001f;
   const dim3 gc((unsigned)cdiv(MB, 32), (unsigned)cdiv(D, 32));
+  const size_t proj_sm = (size_t)(3 * r.N + r.Dp) * sizeof(float2);
+  const size_t beta_sm = MB <= kBetaStage ? (size_t)r.ldT * sizeof(float2) : 0, back_sm = 3 * (size_t)r.Dp * sizeof(float2);
+  auto* beta = MB <= kBetaStage ? rns_beta_kernel<NM, true> : rns_beta_kernel<NM, false>;
+  const bool wide = r.nch2 > rns::kSumChunks;
+  const int per_sum = rns::kSumChunks / rns_chunks(r.nch2, r.g2, r.cap2);
+  auto* backproj = wide ? rns_backproj_kernel<NM, true> : rns_backproj_kernel<NM, false>;
+  RNS_TRY(big_smem(rns_proj_kernel<NM>, proj_sm));
+  RNS_TRY(big_smem(beta, beta_sm));
+  RNS_TRY(big_smem(backproj, back_sm));
   if (r.S > 1) {  // w_b = J_b v_b, then row b S + q = P_q w_b with t = xc_(bS+q) . w_(bS+q)
     launch_proj(G, Xc, v, M, r.N, D, r.W, D, r.t, st);
     launch_sym_gather(r.W, M, D, r.pis, r.S, r.XcB, r.WB, r.t, st);
     { rns_rows_kernel<NM><<<(unsigned)MB, 256, 0, st>>>(r.WB, MB, D, r.W1.Kp, bits, r.W1.d, r.W1.s, r.colmax, r.t, r.t2); count_launch(); }
     { launch_after(pdl, rns_cols_kernel<NM, double>, gc, 256, 0, st, r.WB, MB, D, D, r.colmax, r.WT2.Kp, D + 1, bits, r.WT2.d, r.WT2.s); count_launch(); }
   } else {
-    const size_t sm = (size_t)(3 * r.N + r.Dp) * sizeof(float2);
-    RNS_TRY(big_smem(rns_proj_kernel<NM>, sm));
     const int nt = (int)std::min<int64_t>(512, std::max<int64_t>(64, cdiv(cdiv(D, 2), 32) * 32));
-    { rns_proj_kernel<NM><<<(unsigned)M, nt, sm, st>>>((const float4*)r.G3, (const float4*)r.Xc2, (const uint2*)r.ij, v, M, r.N, r.Dp, rootD, (float4*)r.Wf, r.t2, r.W1.Kp, bits, r.W1.d, r.W1.s, r.colmax); count_launch(); }
+    { rns_proj_kernel<NM><<<(unsigned)M, nt, proj_sm, st>>>((const float4*)r.G3, (const float4*)r.Xc2, (const uint2*)r.ij, v, M, r.N, r.Dp, rootD, (float4*)r.Wf, r.t2, r.W1.Kp, bits, r.W1.d, r.W1.s, r.colmax); count_launch(); }
     { launch_after(pdl, rns_cols_kernel<NM, float2>, gc, 256, 0, st, r.Wf, MB, D, r.Dp, r.colmax, r.WT2.Kp, D + 1, bits, r.WT2.d, r.WT2.s); count_launch(); }
   }
-  const size_t beta_sm = MB <= kBetaStage ? (size_t)r.ldT * sizeof(float2) : 0, back_sm = 3 * (size_t)r.Dp * sizeof(float2);
-  auto* beta = MB <= kBetaStage ? rns_beta_kernel<NM, true> : rns_beta_kernel<NM, false>;
-  const bool wide = r.nch2 > rns::kSumChunks;
-  const int per_sum = rns::kSumChunks / rns_chunks(r.nch2, r.g2, r.cap2);
-  auto* backproj = wide ? rns_backproj_kernel<NM, true> : rns_backproj_kernel<NM, false>;
-  RNS_TRY(big_smem(beta, beta_sm));
-  RNS_TRY(big_smem(backproj, back_sm));
   for (int64_t a0 = 0; a0 < M; a0 += r.P) {  // panels of rows
     const int64_t rows = std::min(r.P, M - a0);
     int s1 = 0, s2 = 0;

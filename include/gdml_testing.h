@@ -48,6 +48,12 @@ gdml_status gdml_test_oz_gemm_tall(const double* A_dev, int64_t n, int64_t K, co
                                    int64_t ldb, int32_t tri_b, int32_t rowsq, double* out_dev, float* out32_dev,
                                    void* cuda_stream);
 
+/* The Gram matrix of the OZAKI preconditioner build (Eq. 4's L^T L, by residue products): the lower
+ * triangle of C = X X^T for X: k x K row-major, FP32 (f32 != 0: the stored factor's columns) or FP64; C: k x k
+ * FP64 row-major, its strict upper triangle untouched.  1 <= k <= 16384, 1 <= K <= 2^31.  Synchronises the
+ * stream.  Errors: GDML_ERR_ARG, GDML_ERR_OOM, GDML_ERR_CUDA, GDML_ERR_TIMEOUT. */
+gdml_status gdml_test_oz_syrk(const void* X_dev, int32_t f32, int64_t k, int64_t K, double* C_dev, void* cuda_stream);
+
 /* The two passes over the FP32-stored factor L_k of the Woodbury apply (Eq. 4) in
  * DF64/OZAKI contexts: t = L^T r and z = (r - L u) / lambda, with exact FP32
  * products of L and the float-pair split of r (u) and double-float sums.  L: n x k

@@ -1435,6 +1435,15 @@ gdml_status gdml_test_set_wait_limit(uint32_t polls) {
   return GDML_OK;
 }
 
+gdml_status gdml_test_oz_syrk(const void* X_dev, int32_t f32, int64_t k, int64_t K, double* C_dev, void* stream) {
+  clear_msg();
+  if (!X_dev || !C_dev || k < 1 || k > 16384 || K < 1 || K > ((int64_t)1 << 31))
+    return fail(GDML_ERR_ARG, "bad syrk test arguments");
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  return f32 ? rns_syrk_lower(static_cast<const float*>(X_dev), k, K, K, C_dev, k, st)
+             : rns_syrk_lower(static_cast<const double*>(X_dev), k, K, K, C_dev, k, st);
+}
+
 gdml_status gdml_test_cholesky_jitter(const double* A_dev, int64_t k, double* L_dev, double* eps_out, void* stream) {
   clear_msg();
   if (!A_dev || !L_dev || !eps_out || k < 1 || k > 16384) return fail(GDML_ERR_ARG, "bad cholesky test arguments");

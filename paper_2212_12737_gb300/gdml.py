@@ -25,7 +25,7 @@ SELECT = {"uniform": 0, "rls": 1, "pivchol": 2, "weighted": 3, "svd": 4}
 
 EXPORTS = ["gdml_kernel_setup", "gdml_kernel_setup_sym", "gdml_matvec", "gdml_matvec_fp64", "gdml_precond_build", "gdml_precond_info",
            "gdml_precond_apply", "gdml_pcg_solve", "gdml_set_inner_rtol", "gdml_last_outer_steps",
-           "gdml_last_error", "gdml_destroy", "gdml_test_tc_gemm", "gdml_test_oz_gemm", "gdml_test_df_passes", "gdml_test_oz_gemm_tall", "gdml_test_precond_factor", "gdml_test_set_wait_limit",
+           "gdml_last_error", "gdml_destroy", "gdml_test_tc_gemm", "gdml_test_oz_gemm", "gdml_test_df_passes", "gdml_test_oz_gemm_tall", "gdml_test_oz_syrk", "gdml_test_precond_factor", "gdml_test_set_wait_limit",
            "gdml_test_cholesky_jitter", "gdml_test_set_lambda", "gdml_tc_check",
            "gdml_launch_count", "gdml_matvec_noalloc", "gdml_pcg_solve_batched", "gdml_autotune",
            "gdml_set_tuning", "gdml_precond_build_scored", "gdml_rls_scores", "gdml_descriptors",
@@ -79,6 +79,7 @@ def load() -> ctypes.CDLL:
         "gdml_test_oz_gemm": [P, P, I64, I64, I64, I32, I32, P, P],
         "gdml_test_df_passes": [P, I64, I64, P, P, D, I32, P, P, P],
         "gdml_test_oz_gemm_tall": [P, I64, I64, P, I64, I64, I32, I32, P, P, P],
+        "gdml_test_oz_syrk": [P, I32, I64, I64, P, P],
         "gdml_test_precond_factor": [P, P],
         "gdml_test_set_wait_limit": [ctypes.c_uint32],
         "gdml_test_cholesky_jitter": [P, I64, P, ctypes.POINTER(D), P],
@@ -412,6 +413,19 @@ def test_oz_gemm_tall(A: torch.Tensor, B: torch.Tensor, tri_b: bool = False, row
     if st != 0:
         raise GdmlError(st, lib.gdml_last_error(None).decode())
     return out if rowsq else (out.t(), out32.t())
+
+
+def test_oz_syrk(X: torch.Tensor) -> torch.Tensor:
+    """The OZAKI build's Gram matrix: the lower triangle of X X^T (zero above) for X (k x K), FP32 or FP64."""
+    lib = load()
+    X = X.contiguous()
+    k, K = X.shape
+    C = torch.zeros(k, k, dtype=torch.float64, device=X.device)
+    st = lib.gdml_test_oz_syrk(_ptr(X), int(X.dtype == torch.float32), k, K, _ptr(C),
+                               ctypes.c_void_p(torch.cuda.current_stream(X.device).cuda_stream))
+    if st != 0:
+        raise GdmlError(st, lib.gdml_last_error(None).decode())
+    return C
 
 
 def test_df_passes(L: torch.Tensor, r: torch.Tensor, u: torch.Tensor, lam: float, staged=True):

@@ -1,8 +1,9 @@
 """The build's Gram matrices by residue products, entry by entry.
 
-Each panel of K' <= 16,384 entries is exact for operands rounded to 2^-57 of max sqrt(K') of their row:
-an entry of X moves by at most 2^-58 max sqrt(K'), so a product sum by
-2^-58 sqrt(K') (max_i sum |x_j| + max_j sum |x_i|); one FP64 rounding per panel and of each addition."""
+Each panel of K' <= 16,384 entries is exact for operands rounded to integers of 56 bits or more below
+max sqrt(K') of their row: an entry of X moves by at most 2^-57 max sqrt(K'), so a product sum by
+2^-57 sqrt(K') (max_i sum |x_j| + max_j sum |x_i|).  Its reconstruction in fixed point adds at most 1.5 units of
+2^55, that is 1.5 2^-57 K' max_i max_j, and there is one FP64 rounding per panel and of each addition."""
 import os
 
 import numpy as np
@@ -58,9 +59,10 @@ def test_entries(k, K, dtype):
     X = X.astype(np.float64)
     ref = np.tril(exact_products(X))
     panels = -(-K // 16384)
-    root = np.sqrt(min(K, 16384))
+    Kp = min(K, 16384)
     m, s = np.abs(X).max(axis=1), np.abs(X).sum(axis=1)
-    bound = 2.0 ** -58 * root * (np.outer(m, s) + np.outer(s, m)) + panels * EPS * (np.abs(X) @ np.abs(X).T) + 2 * EPS * np.abs(ref)
+    bound = 2.0 ** -57 * np.sqrt(Kp) * (np.outer(m, s) + np.outer(s, m)) + panels * 1.5 * 2.0 ** -57 * Kp * np.outer(m, m)
+    bound += panels * EPS * (np.abs(X) @ np.abs(X).T) + 2 * EPS * np.abs(ref)
     worst = (np.abs(got - ref) / bound).max()
     print(f"k={k} K={K} {np.dtype(dtype).name}: max error / bound = {worst:.3f}")
     assert worst <= 1.0

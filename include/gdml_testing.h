@@ -81,7 +81,7 @@ gdml_status gdml_test_precond_factor(gdml_ctx* ctx, double* L_out_dev);
 gdml_status gdml_tc_check(gdml_ctx* ctx);
 
 /* Fault injection from the host for the bounded device waits: every mbarrier wait of the
- * library's tcgen05 / TMA pipelines (the TF32/BF16 and sliced GEMMs, the staged Woodbury
+ * library's tcgen05 / TMA pipelines (the TF32/BF16, residue and sliced GEMMs, the staged Woodbury
  * passes and Schur sums) gives up after `polls` polls instead of its default (about 2^26,
  * seconds).  polls = 0 makes each wait give up at once: the waiting role then issues no copy
  * and no MMA, records GDML_ERR_TIMEOUT in the kernel's error word (read by gdml_tc_check) and

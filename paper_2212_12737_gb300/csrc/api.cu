@@ -366,7 +366,8 @@ gdml_status chol_jitter(gdml_ctx* c, const double* src, double* work, int64_t k,
 // L (k x n row-major = n x k col-major) <- Nystrom factor from columns S (Eq. 5).
 // FP64 / DF64 contexts: forward substitution on the FP64 pipe.  OZAKI contexts: the same
 // L_k = K_nk L_kk^-T as K_nk times the transposed triangular inverse of L_kk, as residue
-// products on the tensor cores (rns_build.cu); only the k x k inverse runs on the FP64 pipe.  On return `work` holds L_kk (lower, row-major).
+// products on the tensor cores (rns_build.cu); only the k x k inverse runs on the FP64 pipe.  On return
+// `work` holds L_kk (lower, row-major).
 gdml_status nystrom(gdml_ctx* c, const int64_t* S, int64_t k, double* L, double* Kkk, double* work,
                     double* eps_out) {
   TRY(get_cols(c, S, k, L));

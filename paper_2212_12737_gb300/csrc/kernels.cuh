@@ -206,7 +206,8 @@ struct PivCholArgs {
   double* col;
   // the kernel column of *col, unless ps->stop; with step > 0 it may release ps->step = step (true: it does)
   std::function<bool(const int64_t* col, double* out, PivState* ps, unsigned step, cudaStream_t)> get_col;
-  // DF64 form only: pivot-row gather (k floats) and Schur partials (pivchol_schur_groups() * n pairs)
+  // DF64 form only, steps without TMA (n % 4 != 0): pivot-row gather (k floats) and Schur partials
+  // (pivchol_schur_groups() * n pairs)
   float* prow = nullptr;
   float2* schur = nullptr;
   int64_t* posof = nullptr;  // inverse of perm (position of each index)

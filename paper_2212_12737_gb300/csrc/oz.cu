@@ -26,14 +26,9 @@ using bf16 = __nv_bfloat16;
 // (kEpiWarps: 4 per TMEM lane quarter, 16 of the tile's 64 columns each)
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = 32 * (3 + kEpiWarps);
-constexpr int kAStages = 6;
 constexpr int kATile = oz::BM * 128;     // 16 KB: 128 rows x one 128-byte K span
 constexpr int kBTile = oz::BN * 128;     // 8 KB
-constexpr int kBGroup = oz::S * kBTile;  // all slices of one B k-block
-constexpr int kSmemData = 2 * kBGroup + kAStages * kATile;
-constexpr int kSmemTotal = kSmemData + 1024 + 256;
 constexpr uint32_t kTmemCols = 512;
-constexpr int kKbPerChunk = oz::KC / oz::KB;
 constexpr int kStageLd = oz::BN + 1;  // padded row of the staged output tile (float2)
 // matvec GEMM: k-blocks of 64 K entries (one 128-byte swizzle span per tile).  The B group of
 // a k-block (7 slices, 56 KB) is double-buffered; the A slices stream through a 6-deep ring
@@ -51,9 +46,7 @@ constexpr int kLevelsPerMma = 4;     // slice pairs (adjacent levels) per MMA: N
 static_assert(oz::BM * kStageLd * 8 <= kSmemDataM, "output staging fits the operand buffers");
 static_assert(kSmemTotalM <= 227 * 1024, "shared memory per CTA");
 static_assert(kEpiCols % 8 == 0, "epilogue columns in groups of 8");
-static_assert(oz::BM * kStageLd * 8 <= kSmemData, "output staging fits the operand buffers");
 static_assert(oz::S * oz::BN <= (int)kTmemCols, "one TMEM accumulator per level");
-static_assert(kSmemTotal <= 227 * 1024, "shared memory per CTA");
 
 // ------------------------------------------------------------ double-float helpers
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -64,13 +57,6 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {  // needs |a| >= |b| or a == 0
   s = __fadd_rn(a, b);
   e = __fsub_rn(b, __fsub_rn(s, a));
-}
-// (h, l) += x
-__device__ __forceinline__ void df_add_f(float& h, float& l, float x) {
-  float s, e;
-  two_sum(h, x, s, e);
-  e = __fadd_rn(e, l);
-  fast_two_sum(s, e, h, l);
 }
 // (h, l) += (bh, bl)
 __device__ __forceinline__ void df_add(float& h, float& l, float bh, float bl) {
@@ -127,16 +113,6 @@ __device__ __forceinline__ void slice_write(float2 xs, int ex, bf16* __restrict_
     yh = __fmul_rn(h, up);
     yl = __fmul_rn(l, up);
   }
-}
-
-// 16 columns of one TMEM lane quarter (32x32b.x16), without waiting for completion
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
 }
 
 // 8 columns of one TMEM lane quarter (32x32b.x8), without waiting for completion

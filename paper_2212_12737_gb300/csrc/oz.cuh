@@ -1,6 +1,6 @@
 // Sliced-BF16 products on the tensor cores (GDML_OZAKI contexts): the matvec with a reduced number of
-// slice levels (gdml_set_inner_levels; the full matvec is the residue form, rns.cuh) and the
-// preconditioner build's tall products.
+// slice levels (gdml_set_inner_levels).  The full matvec is the residue form (rns.cuh), or this one with all
+// 7 levels where the device does not hold the operands of both.
 //
 // The matvec's two descriptor contractions of K v (the same algebra as the FP64 path),
 //   GEMM 1:  T = Xc W^T                              (M x M, K = D)

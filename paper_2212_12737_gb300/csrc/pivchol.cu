@@ -432,7 +432,7 @@ __device__ __forceinline__ bool acquire_step(const unsigned* p, unsigned step) {
 //  - lanes fetch the pivot row's entries straight from L, 32 / CPW tiles ahead (gathered by the last CTA
 //    of the step before: up to 8 us);
 //  - the rows' state is loaded before the stream, and the argmax carries the row with its position;
-//  - the leading `keep` columns stay in L2 (64 MB of them: 4 ms of the build; 96 MB: 1 ms).
+//  - the leading `keep` columns stay in L2 (64 MB of them: 4 ms of the build; 96 MB: nothing).
 template <int NT>
 __global__ void __launch_bounds__(kWsThreads, 2) pc_schur_finish_ws_kernel(
     const __grid_constant__ CUtensorMap map, int64_t n, int64_t m, int64_t nch, int64_t keep, int select, unsigned step, float* L,

@@ -68,10 +68,6 @@ __device__ __noinline__ float scale2_slow(float x, int e) {
   }
   return x * pow2f(e);
 }
-__device__ __forceinline__ float scale2(float x, int e) {
-  if ((unsigned)(e + 126) <= 253u) return x * pow2f(e);
-  return scale2_slow(x, e);
-}
 
 // Scale of a row whose largest magnitude has the bits m and whose K entries the other operand's
 // row meets: 2^s |row|_2 <= 2^s m sqrt(K) < 2^bits.  NaN and infinity have the largest bits.
@@ -886,8 +882,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 // beta_ab = c^2 S_ab (T_ab - t_b) in double-float (T from its residues) and its row residues.  One
 // CTA per row a, two columns per thread and step in packed arithmetic.  STAGE: beta is kept in shared
 // memory between the row's maximum and its residues; else (rows of more than kBetaStage columns) it
-// is formed twice.  Four CTAs of 256 threads per SM (64 registers, 50 bytes of spills more than at 80)
-// against three; rows that fit the chip as CTAs of 128 threads run in one round (see row_threads).
+// is formed twice.  Four CTAs of 256 threads per SM (64 registers) against three at 80; rows that fit the
+// chip as CTAs of 128 threads run in one round (see row_threads).
 constexpr int64_t kBetaStage = 24 * 1024;
 template <int NM, bool STAGE>
 __global__ void __launch_bounds__(256, 4) rns_beta_kernel(const uint16_t* Tp, int slabs, int chunks,

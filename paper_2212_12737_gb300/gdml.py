@@ -301,7 +301,7 @@ class Context:
     def autotune(self, cache: str | None = None) -> int:
         """Time the matvec's tunable tile parameters for this context's shapes and keep the
         fastest (FP64 / TF32 / BF16: the K-split of the second contraction; OZAKI: the K chunks
-        each CTA of the sliced GEMMs accumulates); with a cache file, reuse / record the choice."""
+        each unit of the two residue products accumulates); with a cache file, reuse / record the choice."""
         import json
         key = f"M{self.M}_N{self.N}_{self.precision}"
         table = {}

@@ -15,13 +15,14 @@ namespace gdml {
 // rest is one product.  An SM's FP64 pipe does under two multiply-adds per cycle, so the work of the
 // serial kernels (the diagonal block on one SM, ~NB^3 / 3; a panel's rows at NB^2 / 2 each) decides:
 // with steps of 64 the diagonal block took 105 us and a panel 150-190 us.  32 rows per CTA
-// spread a panel over all SMs.  Two factorisations and two triangular inverses at k = 1500: 62 ms
-// with one level of 64, 21 ms so.
+// spread a panel over all SMs.  The four factorisations and four triangular inverses of a leverage-score build
+// at k = 1500: 62 ms with one level of 64, 22 ms so.
 constexpr int NB = 32;
 constexpr int NO = 128;
 
 // A warp's FP64 operation takes 64 cycles on its quarter of an SM, so all three kernels below use four
-// warps per 32 rows: one warp each took 53, 31 and 24 us (23, 16 and 19 us so).
+// warps per 32 rows: one warp each took 53, 31 and 24 us (22, 18 and 20 us so; 2 us of the two solves are the
+// quotients' corrections, see solve_row).
 constexpr int kGroup = 4;  // lanes (potrf: warps) that share a row: every fourth column each
 constexpr int kOwn = NB / kGroup;
 

@@ -31,7 +31,8 @@ constexpr int kOwn = NB / kGroup;
 __global__ void __launch_bounds__(32 * kGroup) potrf_diag_kernel(double* __restrict__ A, int64_t lda, int64_t j0,
                                                                  int nb, int* __restrict__ status) {
   __shared__ double colv[2][NB];
-  __shared__ int s_bad[2];  // of even and odd steps, as colv: what is tested after a step's barrier is next written after the next one's
+  // of even and odd steps, as colv: what is tested after a step's barrier is next written after the next one's
+  __shared__ int s_bad[2];
   if (*status) return;
   const int r = threadIdx.x & 31, w = threadIdx.x >> 5;
   double* row = A + (j0 + r) * lda + j0;

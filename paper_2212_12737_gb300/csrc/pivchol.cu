@@ -421,8 +421,9 @@ __device__ __forceinline__ bool acquire_step(const unsigned* p, unsigned step) {
 }
 
 // Algorithm 1 step m in one TMA-staged pass: the Schur sums s_i = sum_{j<m} L[i + j n] L[piv + j n],
-// followed row by row (as each chunk's sums are combined) by pc_finish_select_df_kernel's work: l_{i,m}, column m of L, the residual diagonal, the
-// argmax and the trace.  The last CTA to finish selects the pivot of step m + 1 and performs the swap.
+// followed row by row (as each chunk's sums are combined) by pc_finish_select_df_kernel's work: l_{i,m},
+// column m of L, the residual diagonal, the argmax and the trace.  The last CTA to finish selects the pivot
+// of step m + 1 and performs the swap.
 // Bounded by HBM while it streams; what comes before and after is a chain of latencies, at n = 63,000,
 // k = 2,000 at the end 36 us of a step's 111 (160 ms for the build; 140 ms so), therefore
 //  - it starts beside the step's kernel column (see launch_after) and waits for it only at the end.  What

@@ -1312,9 +1312,10 @@ static int row_threads(int64_t M, int64_t pairs, size_t smem) {
 }
 
 // Whether the matvec's kernels may start while the one before them drains (each waits for it before it
-// reads, and reads what a kernel of the same matvec wrote past L1, never as read-only data): about 1.5 us of launch and start-up per kernel.  Outside capture only, and where a kernel's rows
-// are resident at once: M = 200, D = 36 28.3 us, 38.6 without; M = 1,000, D = 210 92.9 and 98.9; but M = 5,000,
-// D = 861 1,660 and 1,588, and a captured solve at M = 1,000 8.96 and 8.85 ms.
+// reads, and reads what a kernel of the same matvec wrote past L1, never as read-only data): about 1.5 us of
+// launch and start-up per kernel.  Outside capture only, and where a kernel's rows are resident at once:
+// M = 200, D = 36 28.3 us, 38.6 without; M = 1,000, D = 210 92.9 and 98.9; but M = 5,000, D = 861 1,660 and
+// 1,588, and a captured solve at M = 1,000 8.96 and 8.85 ms.
 static bool chained(int64_t M, cudaStream_t st) {
   return M <= 8 * (int64_t)num_sms() && not_capturing(st);
 }

@@ -1090,8 +1090,8 @@ void woodbury_apply_df(const float* L, int64_t n, int64_t k, const double* C, co
   }
   // Outside capture the launches of this path may start while the one before them drains: each waits for it
   // before it reads anything but L and the k x k matrices, and lets the next one start only then, so that at
-  // most two are under way; what a launch of the chain writes is read past L1, never as read-only data.  Eight launches of
-  // 3 to 11 us: n = 34,965, k = 77 45.1 -> 32.4 us.
+  // most two are under way; what a launch of the chain writes is read past L1, never as read-only data.  Eight
+  // launches of 3 to 11 us: n = 34,965, k = 77 45.1 -> 32.4 us.
   df_pass_t(L, n, k, rs, part, t, t2, plan, err, st);
   // u = C^-1 t, refined once with the residual t - C u (see woodbury_apply)
   symv_df(Ci2, k, t2, 0, t, u, u2, st);
